@@ -8,8 +8,9 @@
 // inputs and outputs from the caller and keeps its only scratch -- one loss
 // partial per block -- in the file-scope device array below.  That array is
 // part of the library image: every GPU that loads the library holds it
-// (GCP_NOALLOC_MAX_SAMPLES / 2048 blocks x 16 bytes = 128 KB) until the
+// (8192 slots x 16 bytes = 128 KB) until the
 // process exits.
+#include <algorithm>
 #include <mutex>
 
 #include "../../include/gcp.h"
@@ -21,8 +22,8 @@ using namespace gcpdev;
 namespace {
 
 constexpr int kNaThreads = 256;
-constexpr int kNaSamplesPerBlock = 2048;
-constexpr int kNaMaxBlocks = (int)(GCP_NOALLOC_MAX_SAMPLES / kNaSamplesPerBlock);
+constexpr int kNaWarps = kNaThreads / 32;
+constexpr int kNaMaxBlocks = 8192;
 constexpr int kNaMaxDevices = 64;
 
 // Per-block (loss partial, skipped-sample count), shared by every call on a
@@ -32,60 +33,160 @@ constexpr int kNaMaxDevices = 64;
 __device__ __align__(256) double2 g_na_partials[kNaMaxBlocks];
 
 struct NaShape {
-    int d, R;
+    int R;
+    int log2L;                       // lanes per sample
     int64_t dims[GCP_MAX_NDIM];
     int64_t rowoff[GCP_MAX_NDIM];
 };
 
-// One warp per sample; lane l owns columns l, l+32, ... of the rows.
-__global__ void __launch_bounds__(kNaThreads) k_na_grad(const NaShape sh, int loss, int64_t n,
-                                                        const int32_t *__restrict__ idx, const float *__restrict__ x,
-                                                        const float *__restrict__ w, const float *__restrict__ A,
-                                                        float *__restrict__ G, double2 *partials) {
+// V consecutive columns of a row of A, or added to a row of G: one 16-byte
+// vector (V = 4) or a scalar (V = 1).
+template <int V>
+__device__ __forceinline__ void na_load(const float *p, float *o) {
+    if (V == 4)
+        Quad<float>::load(p, o);
+    else
+        o[0] = __ldg(p);
+}
+template <int V>
+__device__ __forceinline__ void na_add(float *p, const float *c) {
+    if (V == 4)
+        red_add_v4(p, c[0], c[1], c[2], c[3]);
+    else
+        atomicAdd(p, c[0]);
+}
+
+// Sampled gradient of a sample list.  A warp takes tiles of 32 consecutive
+// samples: lane l reads sample l's coordinates, value and weight (the next
+// tile's are in flight while this one is evaluated), then groups of L lanes
+// take the tile's samples in turn, their row offsets, values and weights
+// handed over by shuffles.  Lane g of a group owns columns V (g + L q) ..
+// V (g + L q) + V - 1 for q < NQ; those past the rank are skipped, so rows
+// need no padding.  Each lane keeps its own sample's loss and adds it in
+// FP64 once per tile (three FP64 instructions per 32 samples).
+// Bound by the row traffic through L2 (d rows gathered, d rows reduced per
+// sample) and, on skewed data, by the reductions that meet in one row: the
+// entry point has no scratch for replicas.  2^18 samples of the 2000 x 1500
+// x 1000 x 200 Zipf tensor at rank 32, drawn with gcp_sample and passed
+// here: 156 us a pass, against 745 us with one warp per sample walking 256
+// samples one after another on 128 blocks.
+template <int D, int V, int NQ>
+__global__ void __launch_bounds__(kNaThreads, (D <= 4 ? 3 : 1))
+    k_na_grad(const NaShape sh, int loss, int64_t n, const int32_t *__restrict__ idx, const float *__restrict__ x,
+              const float *__restrict__ w, const float *__restrict__ A, float *__restrict__ G, double2 *partials) {
+    constexpr int C = V * NQ;  // columns per lane
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-    const int64_t first = (int64_t)blockIdx.x * kNaSamplesPerBlock;
-    const int64_t last = first + kNaSamplesPerBlock < n ? first + kNaSamplesPerBlock : n;
-    double acc = 0.0, skipped = 0.0;
-    for (int64_t s = first + warp; s < last; s += kNaThreads / 32) {
-        int32_t ii[GCP_MAX_NDIM];
-        bool ok = true;
-        for (int k = 0; k < sh.d; ++k) {
-            ii[k] = idx[s * sh.d + k];
-            ok = ok && ii[k] >= 0 && ii[k] < sh.dims[k];
-        }
-        if (!ok) {  // out-of-range coordinates: the sample is skipped and counted
-            skipped += 1.0;
-            continue;
-        }
-        float m = 0.0f;
-        for (int r = lane; r < sh.R; r += 32) {
-            float prod = 1.0f;
-            for (int k = 0; k < sh.d; ++k) prod *= __ldg(A + (sh.rowoff[k] + ii[k]) * sh.R + r);
-            m += prod;
-        }
+    const int L = 1 << sh.log2L;
+    const int glane = lane & (L - 1), grp = lane >> sh.log2L, ngrp = 32 >> sh.log2L;
+    int col[NQ];
+    bool on[NQ];
 #pragma unroll
-        for (int o = 16; o > 0; o >>= 1) m += __shfl_xor_sync(0xFFFFFFFFu, m, o);
-        float f, df;
-        loss_eval(loss, __ldg(x + s), m, f, df);
-        const float ws = __ldg(w + s);
-        acc += (double)ws * (double)f;
-        const float y = ws * df;
-        for (int r = lane; r < sh.R; r += 32) {
-            for (int nmode = 0; nmode < sh.d; ++nmode) {
-                float prod = y;
-                for (int k = 0; k < sh.d; ++k)
-                    if (k != nmode) prod *= __ldg(A + (sh.rowoff[k] + ii[k]) * sh.R + r);
-                atomicAdd(G + (sh.rowoff[nmode] + ii[nmode]) * sh.R + r, prod);
+    for (int q = 0; q < NQ; ++q) {
+        col[q] = V * (glane + L * q);
+        on[q] = col[q] < sh.R;
+    }
+    const int64_t ntiles = (n + 31) >> 5;
+    const int64_t nwarps = (int64_t)gridDim.x * kNaWarps;
+    int32_t ni[D];  // the next tile's sample of this lane
+    float nx = 0.0f, nw = 0.0f;
+    auto fetch = [&](int64_t tile) {
+        const int64_t s = (tile << 5) + lane;
+        if (s < n) {
+#pragma unroll
+            for (int k = 0; k < D; ++k) ni[k] = __ldg(idx + s * D + k);
+            nx = __ldg(x + s);
+            nw = __ldg(w + s);
+        } else {
+#pragma unroll
+            for (int k = 0; k < D; ++k) ni[k] = 0;
+        }
+    };
+    double acc = 0.0;
+    int skipped = 0;
+    int64_t tile = (int64_t)blockIdx.x * kNaWarps + warp;
+    fetch(tile);
+    for (; tile < ntiles; tile += nwarps) {
+        bool ok = true;
+        int64_t row[D];
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            ok = ok && ni[k] >= 0 && ni[k] < sh.dims[k];
+            row[k] = (sh.rowoff[k] + ni[k]) * sh.R;
+        }
+        const float myx = nx, myw = nw;
+        const bool in = (tile << 5) + lane < n;
+        skipped += in && !ok;  // out-of-range coordinates: the sample is skipped and counted
+        const unsigned okmask = __ballot_sync(0xFFFFFFFFu, in && ok);
+        fetch(tile + nwarps);
+        float myf = 0.0f;
+        for (int it = 0; it < L; ++it) {
+            const int src = it * ngrp + grp;
+            const bool live = (okmask >> src) & 1u;  // uniform within the group
+            const float xs = __shfl_sync(0xFFFFFFFFu, myx, src), ws = __shfl_sync(0xFFFFFFFFu, myw, src);
+            int64_t off[D];
+            float a[D][C];
+#pragma unroll
+            for (int k = 0; k < D; ++k) {
+                off[k] = __shfl_sync(0xFFFFFFFFu, row[k], src);
+#pragma unroll
+                for (int v = 0; v < C; ++v) a[k][v] = 0.0f;
+            }
+            if (live)
+#pragma unroll
+                for (int k = 0; k < D; ++k)
+#pragma unroll
+                    for (int q = 0; q < NQ; ++q)
+                        if (on[q]) na_load<V>(A + off[k] + col[q], a[k] + V * q);
+            float suf[D][C];  // suf[k] = prod_{j>k} a_j
+#pragma unroll
+            for (int v = 0; v < C; ++v) suf[D - 1][v] = 1.0f;
+#pragma unroll
+            for (int k = D - 2; k >= 0; --k)
+#pragma unroll
+                for (int v = 0; v < C; ++v) suf[k][v] = suf[k + 1][v] * a[k + 1][v];
+            float m = 0.0f;
+#pragma unroll
+            for (int v = 0; v < C; ++v) m = fmaf(a[0][v], suf[0][v], m);
+            for (int o = L >> 1; o > 0; o >>= 1) m += __shfl_xor_sync(0xFFFFFFFFu, m, o);
+            float f, df;
+            loss_eval(loss, xs, m, f, df);
+            // sample `lane` was evaluated by group lane % ngrp in round lane / ngrp
+            const float fl = __shfl_sync(0xFFFFFFFFu, f, (lane & (ngrp - 1)) << sh.log2L);
+            if ((lane >> (5 - sh.log2L)) == it) myf = fl;
+            if (!live) continue;
+            float pre[C];
+#pragma unroll
+            for (int v = 0; v < C; ++v) pre[v] = ws * df;
+#pragma unroll
+            for (int k = 0; k < D; ++k) {
+#pragma unroll
+                for (int q = 0; q < NQ; ++q) {
+                    if (!on[q]) continue;
+                    float c[V];
+#pragma unroll
+                    for (int v = 0; v < V; ++v) c[v] = pre[V * q + v] * suf[k][V * q + v];
+                    na_add<V>(G + off[k] + col[q], c);
+                }
+#pragma unroll
+                for (int v = 0; v < C; ++v) pre[v] *= a[k][v];
             }
         }
+        __syncwarp();
+        if ((okmask >> lane) & 1u) acc += (double)myw * (double)myf;
     }
-    // block partial: lane 0 of each warp holds the warp's sums
-    __shared__ double2 red[kNaThreads / 32];
-    if (lane == 0) red[warp] = make_double2(acc, skipped);
+    // block partial: a fixed butterfly over the lanes, then the warps in order
+    double sk = (double)skipped;
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) {
+        acc += __shfl_xor_sync(0xFFFFFFFFu, acc, o);
+        sk += __shfl_xor_sync(0xFFFFFFFFu, sk, o);
+    }
+    __shared__ double2 red[kNaWarps];
+    if (lane == 0) red[warp] = make_double2(acc, sk);
     __syncthreads();
     if (threadIdx.x == 0) {
         double2 t = make_double2(0.0, 0.0);
-        for (int i = 0; i < kNaThreads / 32; ++i) {
+        for (int i = 0; i < kNaWarps; ++i) {
             t.x += red[i].x;
             t.y += red[i].y;
         }
@@ -114,6 +215,44 @@ __global__ void __launch_bounds__(kNaThreads) k_na_sum(const double2 *partials, 
     if (threadIdx.x == 0) {
         loss_out[0] = sh[0].x;
         loss_out[1] = sh[0].y;
+    }
+}
+
+// Columns per lane and lanes per sample.  Vectors need a rank that is a
+// multiple of 4 and 16-byte aligned A and G (every row then starts on a
+// 16-byte boundary); other calls add one column at a time, a lane's columns
+// L apart so that a group's reduction covers consecutive floats.
+struct NaPlan {
+    int v, nq, log2L;
+};
+
+NaPlan na_plan(int R, bool aligned) {
+    NaPlan p{};
+    p.v = (R % 4 == 0 && aligned) ? 4 : 1;
+    const int units = R / p.v;  // vectors or columns of a row, at most 32 or 128
+    p.nq = p.v == 4 ? (units > 8 ? 2 : 1) : (units > 64 ? 4 : (units > 16 ? 2 : 1));
+    while ((p.nq << p.log2L) < units) ++p.log2L;
+    return p;
+}
+
+using NaKernel = void (*)(NaShape, int, int64_t, const int32_t *, const float *, const float *, const float *, float *,
+                          double2 *);
+
+template <int D>
+NaKernel na_kernel_d(const NaPlan &p) {
+    if (p.v == 4) return p.nq == 2 ? k_na_grad<D, 4, 2> : k_na_grad<D, 4, 1>;
+    return p.nq == 4 ? k_na_grad<D, 1, 4> : (p.nq == 2 ? k_na_grad<D, 1, 2> : k_na_grad<D, 1, 1>);
+}
+
+NaKernel na_kernel(int d, const NaPlan &p) {
+    switch (d) {
+    case 2: return na_kernel_d<2>(p);
+    case 3: return na_kernel_d<3>(p);
+    case 4: return na_kernel_d<4>(p);
+    case 5: return na_kernel_d<5>(p);
+    case 6: return na_kernel_d<6>(p);
+    case 7: return na_kernel_d<7>(p);
+    default: return na_kernel_d<8>(p);
     }
 }
 
@@ -159,9 +298,11 @@ extern "C" gcp_status gcp_grad_samples_noalloc(int32_t ndim, const int64_t *dims
                                     "entry point's fixed scratch; split the samples over several calls");
     if (!A || !G || !loss_out || (nsamples > 0 && (!idx || !x || !w)))
         return na_fail(GCP_ERR_ARG, "NULL device pointer");
+    const bool aligned = ((reinterpret_cast<uintptr_t>(A) | reinterpret_cast<uintptr_t>(G)) & 15) == 0;
+    const NaPlan plan = na_plan(rank, aligned);
     NaShape sh{};
-    sh.d = ndim;
     sh.R = rank;
+    sh.log2L = plan.log2L;
     int64_t rows = 0;
     for (int k = 0; k < ndim; ++k) {
         if (dims[k] < 1 || dims[k] > INT32_MAX) return na_fail(GCP_ERR_ARG, "mode size out of range");
@@ -175,8 +316,20 @@ extern "C" gcp_status gcp_grad_samples_noalloc(int32_t ndim, const int64_t *dims
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     if ((e = cudaMemsetAsync(G, 0, (size_t)rows * rank * sizeof(float), st)) != cudaSuccess)
         return na_fail(GCP_ERR_CUDA, cudaGetErrorString(e));
-    const int nblocks = (int)((nsamples + kNaSamplesPerBlock - 1) / kNaSamplesPerBlock);
-    if (nblocks > 0) k_na_grad<<<nblocks, kNaThreads, 0, st>>>(sh, loss, nsamples, idx, x, w, A, G, scratch);
+    int nblocks = 0;
+    if (nsamples > 0) {
+        // a grid of at most the blocks that fit on the GPU at once; fewer
+        // when there are fewer tiles than warps
+        const NaKernel k = na_kernel(ndim, plan);
+        int dev = 0, sms = 0, per_sm = 0;
+        if ((e = cudaGetDevice(&dev)) != cudaSuccess ||
+            (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
+            (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kNaThreads, 0)) != cudaSuccess)
+            return na_fail(GCP_ERR_CUDA, cudaGetErrorString(e));
+        const int64_t want = ((nsamples + 31) / 32 + kNaWarps - 1) / kNaWarps;
+        nblocks = (int)std::min<int64_t>(want, std::min<int64_t>((int64_t)std::max(1, per_sm) * sms, kNaMaxBlocks));
+        k<<<nblocks, kNaThreads, 0, st>>>(sh, loss, nsamples, idx, x, w, A, G, scratch);
+    }
     k_na_sum<<<1, kNaThreads, 0, st>>>(scratch, nblocks, loss_out);
     if ((e = cudaGetLastError()) != cudaSuccess) return na_fail(GCP_ERR_CUDA, cudaGetErrorString(e));
     return GCP_OK;

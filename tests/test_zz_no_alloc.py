@@ -117,3 +117,39 @@ def test_noalloc_skips_out_of_range_samples(env, loss):
     assert abs(L - Lo) <= TOL * abs(Lo), (L, Lo)
     assert rel_err(G.cpu().numpy(), np.concatenate([g.ravel() for g in Go])) <= TOL
     ctx.close()
+
+
+@pytest.mark.parametrize("shift", [0, 1])
+@pytest.mark.parametrize("ndim,R", [(2, 1), (3, 4), (3, 7), (4, 16), (3, 17), (5, 31), (3, 33), (3, 36), (4, 64), (8, 64),
+                                    (3, 65), (3, 100), (2, 128), (3, 127)])
+def test_noalloc_ranks_alignments_and_ragged_counts(env, ndim, R, shift):
+    """Every split of a row over lanes: ranks at the edges of one, two and
+    four columns or vectors per lane, factor and gradient arrays that start
+    on a 16-byte boundary or 4 bytes past one (no vector access possible),
+    sample counts of one sample, a partial tile and many tiles; against the
+    FP64 oracle, with the entries outside G left alone."""
+    import oracle
+
+    gcp, torch = env
+    dims = [23, 19, 40, 11, 5, 4, 3, 6][:ndim]
+    rng = np.random.default_rng(1000 * ndim + R)
+    factors = synth.factors_uniform(dims, R, 931, lo=0.1, hi=1.0)
+    flat = np.concatenate([a.ravel() for a in factors])
+    A = torch.zeros(flat.size + 4, device="cuda")[shift:shift + flat.size]
+    A.copy_(torch.from_numpy(flat))
+    for n in (1, 33, 5003):
+        idx = np.stack([rng.integers(0, I, n) for I in dims], 1).astype(np.int32)
+        x = rng.poisson(2.0, n).astype(np.float32)
+        w = rng.uniform(0.5, 2.0, n).astype(np.float32)
+        buf = torch.full((flat.size + 8,), 7.0, device="cuda")
+        G = buf[shift:shift + flat.size]
+        out = torch.full((2,), float("nan"), dtype=torch.float64, device="cuda")
+        gcp.gcp_grad_samples_noalloc(dims, R, "poisson", torch.from_numpy(idx).cuda(), torch.from_numpy(x).cuda(),
+                                     torch.from_numpy(w).cuda(), A, G, out)
+        L, skipped = out.cpu().numpy()
+        Lo, Go = oracle.sampled_loss_grad(dims, factors, "poisson", idx, x.astype(np.float64), w.astype(np.float64))
+        assert skipped == 0
+        assert abs(L - Lo) <= TOL * abs(Lo), (n, L, Lo)
+        assert rel_err(G.cpu().numpy(), np.concatenate([g.ravel() for g in Go])) <= TOL, n
+        rest = torch.cat([buf[:shift], buf[shift + flat.size:]])
+        assert bool((rest == 7.0).all())

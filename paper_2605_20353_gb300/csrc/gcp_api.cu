@@ -256,6 +256,33 @@ gcp_status check_counts(gcp_ctx *c, int64_t p, int64_t q) {
     return GCP_OK;
 }
 
+// Replicas of the hot rows for a sample set.  The reductions that meet in one
+// 128-byte line are applied one after another, about 4.7 ns each (with no
+// replicas the benchmark's step takes 0.90 ms and the dense 5-way gradient
+// 1.92 ms, which is their hottest line's expected count x 4.6-5.5 ns), so the
+// hottest line bounds the pass from below by that count x 4.7 ns / nrep.  A
+// line holds 32 / Rp rows of a padded rank below 32.  Every replica costs the
+// fold 8 B per entry of every hot row: on 16 clients of 500 hot rows and
+// 16,384 samples each, 64 replicas cost 23 us of a 58-us local step.  So
+// replicas are taken until the chain is under 6% of the pass's row traffic
+// (2 x 4 B x D Rp per sample at about 9 TB/s) or under 4 us, less than the
+// latency of the shortest pass, rounded up to a count the folds are built
+// for.  Measured per call with 0 / 4 / 16 / 64 replicas: benchmark step 900 /
+// 487 / 278 / 247 us (rule: 64); dense 5-way gradient, 2^22 samples 1916 /
+// 852 / 421 / 367 us (64); 172 x 25,000 x 300, rank 50, 2^16 samples 48.5 /
+// 52.3 / 52.3 / 54.3 us (0); 211 x 187 x 95 x 24, rank 10, 10^4 samples 18.7 /
+// 18.6 / 18.6 / 18.6 us per fit iteration (4).
+int replicas_for(const gcp_ctx *c, int64_t p, int64_t q) {
+    if (!c->Grep) return 0;
+    const double line = c->Rp >= 32 ? 1.0 : 32.0 / c->Rp;  // rows of a 128-byte line
+    const double cell = std::min(1.0, c->share_cell * line);
+    const bool uniform = c->opt.sampling == GCP_SAMPLING_UNIFORM;
+    const double hits = uniform ? (double)p * cell : (double)p * c->share_nz + (double)q * cell;
+    const double pass = (double)(p + q) * 8.0 * c->d * c->Rp / 9000.0;  // ns
+    const double want = hits * 4.7 / std::max(0.06 * pass, 4000.0);
+    return want <= 1.0 ? 0 : (want <= 4.0 ? 4 : (want <= 16.0 ? 16 : gcpk::kReplicas));
+}
+
 // One fused pass: loss always, gradient into c->G when `grad`.
 }  // namespace
 
@@ -277,9 +304,10 @@ gcpk::FusedSpec gcpk_make_spec(const gcp_ctx *c, uint64_t iter, int64_t p, int64
     f.w_z = (float)w_z;
     f.dscale = dscale;
     f.partials = c->partials;
-    for (int k = 0; k < c->d; ++k) f.small_base[k] = c->small_base[k];
-    f.Grep = c->Grep;
-    f.Htot = c->Htot;
+    f.nrep = grad ? replicas_for(c, p, q) : 0;
+    for (int k = 0; k < c->d; ++k) f.small_base[k] = f.nrep ? c->small_base[k] : -1;
+    f.Grep = f.nrep ? c->Grep : nullptr;
+    f.Htot = f.nrep ? c->Htot : 0;
     if (w_nz_out) *w_nz_out = w_nz;
     if (w_z_out) *w_z_out = w_z;
     return f;
@@ -324,13 +352,13 @@ gcp_status run_fused(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, bool grad,
         m.vstride = 1;
         GCP_CUDA(c, gcpk::launch_fused(m, c->Abf != nullptr, c->cols, c->max_blocks, c->st, &blocks));
         m.G = c->G;  // pass 2: MTTKRP of the stored gradient tensor
-        GCP_CUDA(c, gcpk::launch_mttkrp_nonfused(m, c->hot_slot, c->Abf != nullptr, c->cols, c->max_blocks, c->st));
+        GCP_CUDA(c, gcpk::launch_mttkrp_nonfused(m, f.nrep ? c->hot_slot : nullptr, c->Abf != nullptr, c->cols, c->max_blocks, c->st));
     } else {
         GCP_CUDA(c, gcpk::launch_fused(f, c->Abf != nullptr, c->cols, c->max_blocks, c->st, &blocks));
     }
     if (stop) GCP_CUDA(c, cudaEventRecord(stop, c->st));
     if (grad && c->opt.mttkrp != GCP_MTTKRP_DETERMINISTIC)
-        GCP_CUDA(c, gcpk::launch_fold_replicas(c->G, c->Grep, c->hot_row, c->Htot, c->Rp, c->st));
+        GCP_CUDA(c, gcpk::launch_fold_replicas(c->G, f.Grep, c->hot_row, f.Htot, c->Rp, f.nrep, c->st));
     GCP_CUDA(c, gcpk::launch_finish_loss(c->partials, blocks, w_nz, w_z, c->dloss, c->status, c->st));
     return GCP_OK;
 }
@@ -371,14 +399,15 @@ gcp_status do_step(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, const gcp_ad
     ps.n = (int64_t)c->total_rows * c->Rp;
     ps.Rp = c->Rp;
     ps.R = c->R;
-    ps.Htot = c->Htot;
+    ps.Htot = f.Htot;
+    ps.nrep = f.nrep;
     ps.G = c->G;
-    ps.Grep = c->Grep;
+    ps.Grep = f.Grep;
     ps.A = c->A;
     ps.B = c->B;
     ps.C = c->C;
     ps.Abf = c->Abf;
-    ps.hot_slot = c->hot_slot;
+    ps.hot_slot = f.nrep ? c->hot_slot : nullptr;
     ps.hot_row = c->hot_row;
     ps.lr = (float)prm->lr;
     ps.beta1 = (float)prm->beta1;
@@ -510,6 +539,8 @@ gcp_status refresh_bf16(gcp_ctx *c) {
 // first.  A nonzero record stores the slots of its rows.
 gcp_status setup_hot_rows(gcp_ctx *c, const std::vector<int64_t> &counts) {
     std::vector<int> slot((size_t)c->total_rows, -1), row;
+    for (int64_t n : counts) c->share_nz = std::max(c->share_nz, (double)n / (double)c->nnz);
+    for (int k = 0; k < c->d; ++k) c->share_cell = std::max(c->share_cell, 1.0 / (double)c->dims[k]);
     for (int k = 0; k < c->d; ++k) {
         c->small_base[k] = -1;
         if (c->dims[k] > 512) continue;

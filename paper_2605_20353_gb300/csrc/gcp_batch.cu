@@ -52,8 +52,8 @@ struct ClientAux {
     float *A, *B, *C, *G, *Grep;
     void *Abf;
     const int *hot_row;   // replica slot -> row
-    const int *hot_slot;  // row -> replica slot, or -1
-    int Htot;
+    const int *hot_slot;  // row -> replica slot, or -1; null without replicas
+    int Htot, nrep;       // replicated rows and replicas of the client's sample count (both 0: none)
     int64_t nparam;  // total_rows * Rp
     int R, Rp;
     double w_nz, w_z;
@@ -165,9 +165,9 @@ __device__ __forceinline__ void adam_quad(const ClientAux &a, int64_t qi, int co
 //    one per thread, all loads (gradient, moments, factor, replica slot)
 //    issued before any is used, then Algorithm 1; quads of hot rows are
 //    left to the hot chunks;
-//  - code <= -2: the client's hot quads h .. h + kThreads / kHotLanes - 1
+//  - code <= -2: the client's hot quads h .. h + 4 kThreads / nrep - 1
 //    (h = -2 - code; hot quad h is column quad h % (Rp/4) of replica slot
-//    h / (Rp/4)), one per group of kHotLanes lanes: the group loads all
+//    h / (Rp/4)), one per group of nrep / 4 lanes: the group loads all
 //    replica quads at once (gcpe::hot_quad_sum, which clears them), its
 //    first lane adds them to the gradient quad and applies Algorithm 1.
 // G itself is cleared at the start of the next step, just before the fused
@@ -180,8 +180,34 @@ __device__ __forceinline__ void adam_quad(const ClientAux &a, int64_t qi, int co
 constexpr int kPostUnroll = 3;
 constexpr int kPostMinBlocks = 3;
 constexpr int kPostQuads = kThreads * kPostUnroll;              // quads of a streaming chunk
-constexpr int kHotQuadsPerChunk = kThreads / gcpe::kHotLanes;   // hot quads of a hot chunk
-static_assert(gcpk::kReplicas % gcpe::kHotLanes == 0, "hot-quad replicas split evenly over the folding lanes");
+
+// A hot chunk of client a, whose sample count uses NREP replicas.
+template <int NREP>
+__device__ __forceinline__ void post_hot_chunk(const ClientAux &a, int64_t h0, const AdamConsts &k) {
+    constexpr int H = gcpe::hot_lanes<NREP>();
+    const int log2Q = __ffs(a.Rp) - 3;  // log2 of the quads of a row
+    const int64_t hq = h0 + threadIdx.x / H;
+    if (hq >= ((int64_t)a.Htot << log2Q)) return;  // the whole group leaves together
+    const int slot = (int)(hq >> log2Q), cq = (int)(hq & ((1 << log2Q) - 1));
+    const int64_t q = ((int64_t)__ldg(a.hot_row + slot) << log2Q) + cq;
+    const bool lead = (threadIdx.x & (H - 1)) == 0;
+    float4 g4, b4, c4, x4;
+    if (lead) {
+        g4 = reinterpret_cast<const float4 *>(a.G)[q];
+        b4 = reinterpret_cast<const float4 *>(a.B)[q];
+        c4 = reinterpret_cast<const float4 *>(a.C)[q];
+        x4 = reinterpret_cast<const float4 *>(a.A)[q];
+    }
+    const float4 t = gcpe::hot_quad_sum<NREP>(reinterpret_cast<float4 *>(a.Grep), ((int64_t)a.Htot * a.Rp) >> 2, hq,
+                                              gcpe::hot_group_mask<NREP>());
+    const int col = cq << 2;
+    if (!lead || col >= a.R) return;
+    g4.x += t.x;
+    g4.y += t.y;
+    g4.z += t.z;
+    g4.w += t.w;
+    adam_quad(a, q, col, g4, b4, c4, x4, k);
+}
 
 __global__ void __launch_bounds__(kThreads, kPostMinBlocks) k_batch_post(const ClientAux *__restrict__ aux,
                                                          const int2 *__restrict__ chunks,
@@ -200,30 +226,14 @@ __global__ void __launch_bounds__(kThreads, kPostMinBlocks) k_batch_post(const C
     const float4 *__restrict__ A4 = reinterpret_cast<const float4 *>(a.A);
     const float4 *__restrict__ B4 = reinterpret_cast<const float4 *>(a.B);
     const float4 *__restrict__ C4 = reinterpret_cast<const float4 *>(a.C);
-    if (ch.y <= -2) {  // hot quads, one per group of kHotLanes lanes
-        const int log2Q = log2Rp - 2;
-        const int64_t hq = (int64_t)(-2 - ch.y) + threadIdx.x / gcpe::kHotLanes;
-        if (hq >= ((int64_t)a.Htot << log2Q)) return;  // the whole group leaves together
-        const int slot = (int)(hq >> log2Q), cq = (int)(hq & ((1 << log2Q) - 1));
-        const int64_t q = ((int64_t)__ldg(a.hot_row + slot) << log2Q) + cq;
-        const bool lead = (threadIdx.x & (gcpe::kHotLanes - 1)) == 0;
-        float4 g4, b4, c4, x4;
-        if (lead) {
-            g4 = G4[q];
-            b4 = B4[q];
-            c4 = C4[q];
-            x4 = A4[q];
-        }
-        const float4 t = gcpe::hot_quad_sum<gcpk::kReplicas>(reinterpret_cast<float4 *>(a.Grep),
-                                                             ((int64_t)a.Htot * a.Rp) >> 2, hq,
-                                                             gcpe::hot_group_mask());
-        const int col = cq << 2;
-        if (!lead || col >= a.R) return;
-        g4.x += t.x;
-        g4.y += t.y;
-        g4.z += t.z;
-        g4.w += t.w;
-        adam_quad(a, q, col, g4, b4, c4, x4, k);
+    if (ch.y <= -2) {  // hot quads, one per group of nrep / 4 lanes
+        const int64_t h0 = (int64_t)(-2 - ch.y);
+        if (a.nrep == 64)
+            post_hot_chunk<64>(a, h0, k);
+        else if (a.nrep == 16)
+            post_hot_chunk<16>(a, h0, k);
+        else
+            post_hot_chunk<4>(a, h0, k);
         return;
     }
     const int64_t nq = a.nparam >> 2;
@@ -484,11 +494,12 @@ gcp_status gcp_batch_create(int32_t nclients, gcp_ctx *const *clients, const int
         a.B = c->B;
         a.C = c->C;
         a.G = c->G;
-        a.Grep = c->Grep;
+        a.Grep = f.Grep;
         a.Abf = c->Abf;
         a.hot_row = c->hot_row;
-        a.hot_slot = c->hot_slot;
-        a.Htot = c->Htot;
+        a.hot_slot = f.nrep ? c->hot_slot : nullptr;
+        a.Htot = f.Htot;
+        a.nrep = f.nrep;
         a.nparam = c->total_rows * c->Rp;
         a.R = c->R;
         a.Rp = c->Rp;
@@ -507,7 +518,7 @@ gcp_status gcp_batch_create(int32_t nclients, gcp_ctx *const *clients, const int
     for (int i = 0; i < nclients; ++i)
         for (int64_t q0 = 0; q0 < aux[i].nparam / 4; q0 += gcpb::kPostQuads) chunks.push_back(make_int2(i, (int)q0));
     for (int i = 0; i < nclients; ++i)  // hot chunks: code -2 - (first hot quad)
-        for (int64_t h = 0; h < (int64_t)aux[i].Htot * (aux[i].Rp / 4); h += gcpb::kHotQuadsPerChunk)
+        for (int64_t h = 0; h < (int64_t)aux[i].Htot * (aux[i].Rp / 4); h += 4 * gcpb::kThreads / aux[i].nrep)
             chunks.push_back(make_int2(i, (int)(-2 - h)));
     b->nchunks = (int)chunks.size();
     cudaError_t e;

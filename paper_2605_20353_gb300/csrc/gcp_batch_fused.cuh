@@ -198,7 +198,7 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
         const int p = (int)P.s.p;
         const int tbase = (tile - __ldg(tile_start + cur_client[st])) * TS;
         const bool semi = P.s.sampling == GCP_SAMPLING_SEMI_STRATIFIED;
-        float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (gcpk::kReplicas - 1)) * P.Htot * Rp : nullptr;
+        float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (P.nrep - 1)) * P.Htot * Rp : nullptr;
         float tf_nz = 0.0f, tf_z = 0.0f;
         for (int it = 0; it * ngrp < TS; ++it) {
             const int src = it * ngrp + grp;
@@ -247,7 +247,7 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
 #pragma unroll
             for (int n = 0; n < D; ++n) {
                 unsigned hs;
-                if (is_nz)
+                if (is_nz && grep)
                     hs = ((unsigned)slot[D + 1 + n / 2] >> (16 * (n & 1))) & 0xFFFFu;
                 else
                     hs = P.small_base[n] >= 0 ? (unsigned)(P.small_base[n] + ii[n]) : gcpk::kNoSlot;

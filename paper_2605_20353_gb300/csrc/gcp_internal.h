@@ -45,22 +45,26 @@ struct FusedSpec {
     double *partials;               // per block: sum f over nonzero / zero samples, attempts, -
     int small_base[GCP_MAX_NDIM];   // replica slot of row 0 of a mode whose rows all have
                                     // slots (contiguous), else -1; used for drawn cells
-    float *Grep;                    // kReplicas x Htot x Rp replica rows (zero between calls)
+    float *Grep;                    // nrep x Htot x Rp replica rows (zero between calls), or null:
+                                    // every row is added to G itself
     int Htot;                       // replicated rows
+    int nrep;                       // replicas this call uses: 0 (Grep null), 4, 16 or 64
     int32_t *Ycoord;                // materialize mode (G null): per-sample coordinates
     float *Yval;                    //   and gradient-tensor values w f' scale (0 if no sample):
     int ystride, vstride;           //   sample s at Ycoord[s * ystride + k], Yval[s * vstride]
 };
 
 // Rows that many samples hit (Zipf heads, rows of small modes) are
-// accumulated in this many global replicas, then folded into G.
+// accumulated in up to this many global replicas, then folded into G.  A
+// call uses as many as its sample count and the hottest row's share call for
+// (replicas_for): none, 4, 16 or all 64.
 constexpr int kReplicas = 64;
 
 // The epilogue of one training step (gcp_step): loss finish, replica fold,
 // Adam and gradient clearing in one launch.
 struct PostSpec {
     int64_t n;                      // total_rows * Rp
-    int Rp, R, Htot;
+    int Rp, R, Htot, nrep;          // nrep 0: no replicas (Htot 0, hot_slot null)
     float *G, *Grep, *A, *B, *C;
     void *Abf;
     const int *hot_slot;            // row -> replica slot, or -1
@@ -88,7 +92,8 @@ cudaError_t launch_sample(const SampleSpec &s, int32_t *idx_out, float *x_out, f
                           float w_z, cudaStream_t st);
 cudaError_t launch_fused(const FusedSpec &f, bool bf16, int cols, int max_blocks, cudaStream_t st,
                          int *blocks_used);
-cudaError_t launch_fold_replicas(float *G, float *Grep, const int *hot_row, int Htot, int Rp, cudaStream_t st);
+cudaError_t launch_fold_replicas(float *G, float *Grep, const int *hot_row, int Htot, int Rp, int nrep,
+                                 cudaStream_t st);
 cudaError_t launch_mttkrp_nonfused(const FusedSpec &f, const int *hot_slot, bool bf16, int cols, int max_blocks,
                                    cudaStream_t st);
 cudaError_t launch_finish_loss(const double *partials, int nblocks, double w_nz, double w_z, double *dloss,
@@ -142,6 +147,8 @@ struct gcp_ctx {
     int small_base[GCP_MAX_NDIM] = {0};
     float *Grep = nullptr;        // [kReplicas x Htot x Rp]
     int Htot = 0;
+    double share_nz = 0.0;        // largest share of the nonzeros in one row
+    double share_cell = 0.0;      // the same of all cells: 1 / the smallest mode size
 
     // deterministic MTTKRP scratch
     void *det_scratch = nullptr;

@@ -121,9 +121,10 @@ __device__ __forceinline__ bool draw_sample(const SampleSpec &S, int64_t s, int3
 //      COLS columns as COLS/4 quads (4g..4g+3, and Rp/2+4g.. when COLS = 8),
 //      so a group's loads and vector reductions cover whole 32-byte sectors
 //      and, for rows up to 128 bytes, one whole row per instruction.
-// Gradient rows that many samples hit go to one of kReplicas replicas
+// Gradient rows that many samples hit go to one of the call's nrep replicas
 // (chosen by warp), folded into G afterwards, so that the reductions of hot
-// rows do not serialise on one address.
+// rows do not serialise on one address; with nrep = 0 (few samples) every
+// row is added to G itself.
 constexpr int kWarps = kThreads / 32;
 
 template <int D, typename TF, int COLS>
@@ -153,7 +154,7 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
     const float scale = P.dscale ? __ldg(P.dscale) : 1.0f;
     const bool semi = P.s.sampling == GCP_SAMPLING_SEMI_STRATIFIED;
     const bool uniform = P.s.sampling == GCP_SAMPLING_UNIFORM;
-    float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (kReplicas - 1)) * P.Htot * P.Rp : nullptr;
+    float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (P.nrep - 1)) * P.Htot * P.Rp : nullptr;
 
     double acc_nz = 0.0, acc_z = 0.0;
     int attempts = 0;
@@ -313,7 +314,7 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
                     // replica slot: stored in a nonzero's record; for drawn
                     // cells, rows of fully replicated modes only
                     unsigned hs;
-                    if (is_nz)
+                    if (is_nz && grep)
                         hs = ((unsigned)slot[D + 1 + n / 2] >> (16 * (n & 1))) & 0xFFFFu;
                     else
                         hs = P.small_base[n] >= 0 ? (unsigned)(P.small_base[n] + ii[n]) : kNoSlot;
@@ -359,33 +360,27 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
 
 // G(hot row) += sum over replicas, then the replicas are cleared for the
 // next call (fixed replica order).  G may already hold contributions of
-// drawn cells to a replicated row of a large mode.  All kReplicas loads of
+// drawn cells to a replicated row of a large mode.  All NREP loads of
 // an element are issued before any add: there are few hot elements, so one
 // round trip per element beats the occupancy that fewer registers would
-// give (16 loads at a time measured 8 µs against 5 µs per launch).
-__device__ __forceinline__ void fold_range(float *__restrict__ G, float *__restrict__ Grep,
-                                           const int *__restrict__ hot_row, int Htot, int Rp, int64_t first,
-                                           int64_t stride) {
-    const int64_t n = (int64_t)Htot * Rp, plane = (int64_t)Htot * Rp;
-    for (int64_t e = first; e < n; e += stride) {
-        float v[kReplicas];
+// give (16 of 64 loads at a time measured 8 us against 5 us per launch).
+template <int NREP>
+__global__ void k_fold_replicas(float *__restrict__ G, float *__restrict__ Grep, const int *__restrict__ hot_row,
+                                int Htot, int Rp) {
+    const int64_t n = (int64_t)Htot * Rp, plane = n;
+    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
+        float v[NREP];
 #pragma unroll
-        for (int r = 0; r < kReplicas; ++r) v[r] = Grep[r * plane + e];
+        for (int r = 0; r < NREP; ++r) v[r] = Grep[r * plane + e];
         float t = 0.0f;
 #pragma unroll
-        for (int r = 0; r < kReplicas; ++r) t += v[r];
+        for (int r = 0; r < NREP; ++r) t += v[r];
 #pragma unroll
-        for (int r = 0; r < kReplicas; ++r) Grep[r * plane + e] = 0.0f;
+        for (int r = 0; r < NREP; ++r) Grep[r * plane + e] = 0.0f;
         const int log2Rp = __ffs(Rp) - 1;  // Rp is a power of two
         const int slot = (int)(e >> log2Rp), col = (int)(e & (Rp - 1));
         G[(int64_t)hot_row[slot] * Rp + col] += t;
     }
-}
-
-__global__ void k_fold_replicas(float *__restrict__ G, float *__restrict__ Grep, const int *__restrict__ hot_row,
-                                int Htot, int Rp) {
-    fold_range(G, Grep, hot_row, Htot, Rp, (int64_t)blockIdx.x * blockDim.x + threadIdx.x,
-               (int64_t)gridDim.x * blockDim.x);
 }
 
 // Fixed-order reduction of the block partials (one block).
@@ -507,9 +502,10 @@ __global__ void k_adam(int64_t n, int Rp, int R, float *__restrict__ A, float *_
 //    their loads (gradient, moments, factor, replica slot) before using any,
 //    then applies Algorithm 1 and clears G for the next step;
 //  - the blocks between take the quads of hot rows, one per group of
-//    kHotLanes lanes: the group loads the quad's kReplicas replica quads at
+//    NREP / 4 lanes: the group loads the quad's NREP replica quads at
 //    once (gcpe::hot_quad_sum, which also clears them), and its first lane
-//    adds them to the gradient quad and applies Algorithm 1.
+//    adds them to the gradient quad and applies Algorithm 1.  With NREP = 0
+//    there are no hot rows and no such blocks.
 // The streaming blocks run at the copy rate on models larger than L2; the
 // hot quads cost one memory round trip each instead of one per group of
 // replica loads.
@@ -518,8 +514,8 @@ __global__ void k_adam(int64_t n, int Rp, int R, float *__restrict__ A, float *_
 // 6.0 TB/s; two or four per thread, with fewer resident warps, at 3.6 and
 // 4.1 TB/s.
 constexpr int kPostUnroll = 1;
-static_assert(kReplicas % gcpe::kHotLanes == 0, "hot-quad replicas split evenly over the folding lanes");
 
+template <int NREP>
 __global__ void __launch_bounds__(kThreads) k_post_step(PostSpec P, int ncold) {
     if (blockIdx.x == gridDim.x - 1) {  // the last block only finishes the loss
         __shared__ double sh[3][kThreads];
@@ -547,37 +543,39 @@ __global__ void __launch_bounds__(kThreads) k_post_step(PostSpec P, int ncold) {
     float4 *__restrict__ C4 = reinterpret_cast<float4 *>(P.C);
     uint2 *__restrict__ Abf = static_cast<uint2 *>(P.Abf);
     const int log2Rp = __ffs(P.Rp) - 1;
-    if ((int)blockIdx.x >= ncold) {  // hot quads, one per group of kHotLanes lanes
-        const int log2Q = log2Rp - 2;  // quads per row = Rp / 4
-        const int64_t hq = (int64_t)(blockIdx.x - ncold) * (kThreads / gcpe::kHotLanes) +
-                           (threadIdx.x / gcpe::kHotLanes);
-        if (hq >= ((int64_t)P.Htot << log2Q)) return;  // the whole group leaves together
-        const int slot = (int)(hq >> log2Q), cq = (int)(hq & ((1 << log2Q) - 1));
-        const int64_t q = ((int64_t)__ldg(P.hot_row + slot) << log2Q) + cq;
-        const bool lead = (threadIdx.x & (gcpe::kHotLanes - 1)) == 0;
-        float4 g, a, b, c;
-        if (lead) {
-            g = G4[q];
-            a = A4[q];
-            b = B4[q];
-            c = C4[q];
+    if constexpr (NREP > 0) {
+        if ((int)blockIdx.x >= ncold) {  // hot quads, one per group of NREP / 4 lanes
+            constexpr int H = gcpe::hot_lanes<NREP>();
+            const int log2Q = log2Rp - 2;  // quads per row = Rp / 4
+            const int64_t hq = (int64_t)(blockIdx.x - ncold) * (kThreads / H) + (threadIdx.x / H);
+            if (hq >= ((int64_t)P.Htot << log2Q)) return;  // the whole group leaves together
+            const int slot = (int)(hq >> log2Q), cq = (int)(hq & ((1 << log2Q) - 1));
+            const int64_t q = ((int64_t)__ldg(P.hot_row + slot) << log2Q) + cq;
+            const bool lead = (threadIdx.x & (H - 1)) == 0;
+            float4 g, a, b, c;
+            if (lead) {
+                g = G4[q];
+                a = A4[q];
+                b = B4[q];
+                c = C4[q];
+            }
+            const float4 t = gcpe::hot_quad_sum<NREP>(reinterpret_cast<float4 *>(P.Grep),
+                                                      ((int64_t)P.Htot * P.Rp) >> 2, hq, gcpe::hot_group_mask<NREP>());
+            if (!lead) return;
+            g.x += t.x;
+            g.y += t.y;
+            g.z += t.z;
+            g.w += t.w;
+            G4[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            const int col = cq << 2;
+            if (col >= P.R) return;  // a quad of padding columns
+            adam_quad(a, b, c, g, col, P.R, P.lr, P.beta1, P.beta2, P.c1inv, P.c2inv, P.eps, P.lower,
+                      Abf ? Abf + q : nullptr);
+            A4[q] = a;
+            B4[q] = b;
+            C4[q] = c;
+            return;
         }
-        const float4 t = gcpe::hot_quad_sum<kReplicas>(reinterpret_cast<float4 *>(P.Grep),
-                                                       ((int64_t)P.Htot * P.Rp) >> 2, hq, gcpe::hot_group_mask());
-        if (!lead) return;
-        g.x += t.x;
-        g.y += t.y;
-        g.z += t.z;
-        g.w += t.w;
-        G4[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
-        const int col = cq << 2;
-        if (col >= P.R) return;  // a quad of padding columns
-        adam_quad(a, b, c, g, col, P.R, P.lr, P.beta1, P.beta2, P.c1inv, P.c2inv, P.eps, P.lower,
-                  Abf ? Abf + q : nullptr);
-        A4[q] = a;
-        B4[q] = b;
-        C4[q] = c;
-        return;
     }
     // block tiles of kThreads * kPostUnroll consecutive quads; thread t takes
     // quads t, t + kThreads, ... of its block's tile
@@ -614,19 +612,33 @@ __global__ void __launch_bounds__(kThreads) k_post_step(PostSpec P, int ncold) {
     }
 }
 
-cudaError_t launch_post_step(const PostSpec &p, cudaStream_t st) {
+template <int NREP>
+static cudaError_t launch_post_step_r(const PostSpec &p, cudaStream_t st) {
     static int resident = 0;  // streaming blocks that fit on the GPU at once
     if (!resident) {
         int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_post_step, kThreads, 0);
+        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_post_step<NREP>, kThreads, 0);
         resident = (per_sm < 1 ? 1 : per_sm) * num_sms();
     }
     const int64_t want = ((p.n >> 2) + (int64_t)kThreads * kPostUnroll - 1) / ((int64_t)kThreads * kPostUnroll);
     const int ncold = (int)(want < 1 ? 1 : (want > resident ? resident : want));
-    const int64_t hot_quads = (int64_t)p.Htot * (p.Rp >> 2);
-    const int nhot = (int)((hot_quads + kThreads / gcpe::kHotLanes - 1) / (kThreads / gcpe::kHotLanes));
-    k_post_step<<<ncold + nhot + 1, kThreads, 0, st>>>(p, ncold);  // + the loss block
+    int nhot = 0;
+    if constexpr (NREP > 0) {
+        constexpr int per = kThreads / gcpe::hot_lanes<NREP>();  // hot quads of a block
+        nhot = (int)(((int64_t)p.Htot * (p.Rp >> 2) + per - 1) / per);
+    }
+    k_post_step<NREP><<<ncold + nhot + 1, kThreads, 0, st>>>(p, ncold);  // + the loss block
     return cudaGetLastError();
+}
+
+cudaError_t launch_post_step(const PostSpec &p, cudaStream_t st) {
+    switch (p.nrep) {
+    case 0: return launch_post_step_r<0>(p, st);
+    case 4: return launch_post_step_r<4>(p, st);
+    case 16: return launch_post_step_r<16>(p, st);
+    case 64: return launch_post_step_r<64>(p, st);
+    default: return cudaErrorInvalidValue;
+    }
 }
 
 __global__ void k_to_bf16(int64_t n, const float *__restrict__ A, __nv_bfloat16 *Abf) {
@@ -771,7 +783,7 @@ __global__ void __launch_bounds__(kThreads) k_mttkrp_nonfused(const FusedSpec P,
     const int ngroups = (gridDim.x * blockDim.x) >> P.log2L;
     const int warp0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const TF *__restrict__ F = static_cast<const TF *>(P.F);
-    float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (kReplicas - 1)) * P.Htot * P.Rp : nullptr;
+    float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (P.nrep - 1)) * P.Htot * P.Rp : nullptr;
     int col[NQ];
 #pragma unroll
     for (int q = 0; q < NQ; ++q) col[q] = q * (P.Rp >> 1) + 4 * glane;
@@ -846,9 +858,16 @@ cudaError_t launch_mttkrp_nonfused(const FusedSpec &f, const int *hot_slot, bool
     return cudaGetLastError();
 }
 
-cudaError_t launch_fold_replicas(float *G, float *Grep, const int *hot_row, int Htot, int Rp, cudaStream_t st) {
-    if (Htot == 0) return cudaSuccess;
-    k_fold_replicas<<<elementwise_blocks((int64_t)Htot * Rp), kThreads, 0, st>>>(G, Grep, hot_row, Htot, Rp);
+cudaError_t launch_fold_replicas(float *G, float *Grep, const int *hot_row, int Htot, int Rp, int nrep,
+                                 cudaStream_t st) {
+    if (Htot == 0 || nrep == 0) return cudaSuccess;
+    const int blocks = elementwise_blocks((int64_t)Htot * Rp);
+    switch (nrep) {
+    case 4: k_fold_replicas<4><<<blocks, kThreads, 0, st>>>(G, Grep, hot_row, Htot, Rp); break;
+    case 16: k_fold_replicas<16><<<blocks, kThreads, 0, st>>>(G, Grep, hot_row, Htot, Rp); break;
+    case 64: k_fold_replicas<64><<<blocks, kThreads, 0, st>>>(G, Grep, hot_row, Htot, Rp); break;
+    default: return cudaErrorInvalidValue;
+    }
     return cudaGetLastError();
 }
 

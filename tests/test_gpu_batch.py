@@ -127,6 +127,42 @@ def test_batch_folded_gradient_matches_oracle_client_by_client(env, shards, dtyp
     b.close()
 
 
+def test_batch_clients_with_different_replica_counts(env):
+    """Clients whose sample counts call for no replicas, 4, 16 and 64 of
+    them in one batch (the hottest row of the 8-row mode takes about an
+    eighth of a client's samples): the gradient each folds, twice over,
+    against the oracle."""
+    gcp, torch = env
+    dims, R = [8, 41, 700], 6
+    counts = [(150, 130), (60000, 50000), (900, 700), (7000, 6001)]
+    shards = []
+    for i, (p, q) in enumerate(counts):
+        coords, vals = synth.uniform_sparse(dims, 5000, 640 + i, lam=2.0)
+        shards.append((coords, vals, synth.factors_uniform(dims, R, 650 + i, lo=0.1, hi=1.0), 660 + i))
+    cl = []
+    for coords, vals, fac, seed in shards:
+        c = gcp.gcp_create(dims, coords, vals, R, "poisson", seed=seed)
+        c.set_factors(fac)
+        cl.append(c)
+    b = gcp.GcpBatch(cl, [p for p, _ in counts], [q for _, q in counts])
+    ref = []
+    for (coords, vals, fac, seed), (p, q) in zip(shards, counts):
+        idx, x, w, _ = oracle.stratified_samples(seed, 5, p, q, dims, coords, vals)
+        ref.append(oracle.sampled_loss_grad(dims, fac, "poisson", idx, x, w))
+    prm = readout_params(gcp, max(np.abs(g).max() for _, Go in ref for g in Go))
+    for _ in range(2):  # the second round finds every plane cleared
+        for c, (_, _, fac, _) in zip(cl, shards):
+            c.set_factors(fac)
+            c.reset_adam()
+        b.local_steps(1, prm, 5, 0)
+        losses = b.losses()
+        for c, (_, _, fac, _), (Lo, Go), L in zip(cl, shards, ref, losses):
+            G = recover_gradient(flat(fac), flat(c.get_factors()), prm)
+            assert L == pytest.approx(Lo, rel=1e-5)
+            assert rel_err(G, np.concatenate([g.ravel() for g in Go])) <= 1e-5
+    b.close()
+
+
 def test_graph_replays_continue_the_step_counters(env, shards):
     gcp, torch = env
     adam = gcp.AdamParams(**ADAM)

@@ -697,6 +697,34 @@ def test_step_folded_gradient_matches_oracle(env, dtype, mttkrp):
     ctx.close()
 
 
+@pytest.mark.parametrize("mttkrp", ["atomic", "nonfused"])
+def test_replica_counts_in_turn_on_one_context(env, mttkrp):
+    """Sample counts on both sides of every step of the replica rule (no
+    replicas, 4, 16 and 64: the hottest row of the 8-row mode takes about an
+    eighth of the samples), in an order that mixes them on one context, so
+    that a call must find the planes that larger calls used cleared.  The
+    gradient of gcp_grad and, for the atomic variant, the one folded inside
+    gcp_step against the oracle."""
+    gcp, torch = env
+    dims, R = [8, 41, 700], 6  # one replicated small mode, one of 41 rows, one too large
+    coords, vals, factors = problem(dims, 5000, R, "poisson", 611)
+    ctx = gcp.gcp_create(dims, coords, vals, R, "poisson", seed=612, mttkrp=mttkrp)
+    for t, (p, q) in enumerate([(60000, 50000), (150, 130), (900, 700), (7000, 6001), (900, 700), (60000, 1),
+                                (0, 9000), (300, 0)]):
+        idx, x, w, _ = oracle.stratified_samples(612, t, p, q, dims, coords, vals)
+        Lo, Go = oracle.sampled_loss_grad(dims, factors, "poisson", idx, x, w)
+        ctx.set_factors(factors)
+        Lg, Gg = gpu_grad(gcp, torch, ctx, t, p, q)
+        assert abs(Lg - Lo) <= TOL_FP32 * abs(Lo), (t, Lg, Lo)
+        for n, (a, b) in enumerate(zip(split(Gg, dims, R), Go)):
+            assert rel_err(a, b) <= TOL_FP32, (t, n, rel_err(a, b))
+        if mttkrp == "atomic":
+            G = step_gradient(gcp, ctx, factors, t, p, q, max(np.abs(g).max() for g in Go))
+            for n, (a, b) in enumerate(zip(split(G, dims, R), Go)):
+                assert rel_err(a, b) <= TOL_FP32, (t, n, rel_err(a, b))
+    ctx.close()
+
+
 def test_fit_with_tuned_preset_on_count_data(env):
     """gcp_fit with the paper's tuned GCP-SGD hyperparameters on a Poisson
     count tensor: the objective estimate falls, at most max_fails epochs

@@ -317,12 +317,73 @@ gcp_status gcpk_check_counts(gcp_ctx *c, int64_t p, int64_t q) { return check_co
 
 namespace {
 
-gcp_status run_fused(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, bool grad, const float *dscale) {
+// Whether kernels of the context can write n bytes at p directly: device
+// memory of its device or managed memory, aligned for `align`-byte accesses.
+// Other pointers (host memory, another device) go through the copy calls,
+// which say what is wrong with the ones they do not take.
+bool kernel_writable(const gcp_ctx *c, const void *p, size_t align) {
+    if (reinterpret_cast<uintptr_t>(p) % align) return false;
+    cudaPointerAttributes at{};
+    if (cudaPointerGetAttributes(&at, p) != cudaSuccess) {
+        cudaGetLastError();  // not a sticky error
+        return false;
+    }
+    return at.type == cudaMemoryTypeManaged || (at.type == cudaMemoryTypeDevice && at.device == c->device);
+}
+
+// Where the results of a fused pass go besides the context's own buffers.
+struct Outputs {
+    float *G = nullptr;       // unpadded gradient (host or device), or null
+    double *dloss = nullptr;  // device loss, or null
+    bool host = false;        // the pinned mirrors are read after a synchronisation
+};
+
+// The loss finish of a pass of `blocks` partials.  `copy_loss` tells whether
+// the caller's device double still has to be copied (a pointer that the
+// kernels cannot write).
+gcpk::LossSpec loss_spec(gcp_ctx *c, int blocks, double w_nz, double w_z, const Outputs &o, bool *copy_loss) {
+    gcpk::LossSpec l{};
+    l.partials = c->partials;
+    l.nblocks = blocks;
+    l.w_nz = w_nz;
+    l.w_z = w_z;
+    l.dloss = c->dloss;
+    l.status = c->status;
+    const bool direct = o.dloss && kernel_writable(c, o.dloss, sizeof(double));
+    l.out = direct ? o.dloss : nullptr;
+    *copy_loss = o.dloss && !direct;
+    if (o.host) {
+        l.h_loss = c->h_loss;
+        l.h_status = c->h_status;
+    }
+    return l;
+}
+
+gcp_status copy_loss_out(gcp_ctx *c, double *dloss_out) {
+    GCP_CUDA(c, cudaMemcpyAsync(dloss_out, c->dloss, sizeof(double), cudaMemcpyDeviceToDevice, c->st));
+    return GCP_OK;
+}
+
+// After a pass with Outputs::host: wait, then report the device errors that
+// the loss finish mirrored (clearing them).
+gcp_status host_result(gcp_ctx *c) {
+    GCP_CUDA(c, cudaStreamSynchronize(c->st));
+    const int bits = *c->h_status;
+    if (!bits) return GCP_OK;
+    GCP_CUDA(c, cudaMemsetAsync(c->status, 0, sizeof(int), c->st));
+    const gcp_status s = status_code(bits);
+    return fail(c, s, status_text(s));
+}
+
+gcp_status copy_grad_out(gcp_ctx *c, float *G_out);
+
+gcp_status run_fused(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, bool grad, const float *dscale,
+                     const Outputs &out) {
     gcp_status s = check_counts(c, p, q);
     if (s) return s;
     double w_nz, w_z;
     gcpk::FusedSpec f = gcpk_make_spec(c, iter, p, q, grad, dscale, &w_nz, &w_z);
-    if (grad) {
+    if (grad) {  // also when G is clear: a captured call is replayed on a G that is not
         GCP_CUDA(c, cudaMemsetAsync(c->G, 0, (size_t)c->total_rows * c->Rp * 4, c->st));
         c->g_clear = false;
     }
@@ -352,14 +413,38 @@ gcp_status run_fused(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, bool grad,
         m.vstride = 1;
         GCP_CUDA(c, gcpk::launch_fused(m, c->Abf != nullptr, c->cols, c->max_blocks, c->st, &blocks));
         m.G = c->G;  // pass 2: MTTKRP of the stored gradient tensor
-        GCP_CUDA(c, gcpk::launch_mttkrp_nonfused(m, f.nrep ? c->hot_slot : nullptr, c->Abf != nullptr, c->cols, c->max_blocks, c->st));
+        GCP_CUDA(c, gcpk::launch_mttkrp_nonfused(m, f.nrep ? c->hot_slot : nullptr, c->Abf != nullptr, c->cols,
+                                                 c->max_blocks, c->st));
     } else {
         GCP_CUDA(c, gcpk::launch_fused(f, c->Abf != nullptr, c->cols, c->max_blocks, c->st, &blocks));
     }
     if (stop) GCP_CUDA(c, cudaEventRecord(stop, c->st));
-    if (grad && c->opt.mttkrp != GCP_MTTKRP_DETERMINISTIC)
-        GCP_CUDA(c, gcpk::launch_fold_replicas(c->G, f.Grep, c->hot_row, f.Htot, c->Rp, f.nrep, c->st));
-    GCP_CUDA(c, gcpk::launch_finish_loss(c->partials, blocks, w_nz, w_z, c->dloss, c->status, c->st));
+    bool copy_loss = false;
+    const gcpk::LossSpec loss = loss_spec(c, blocks, w_nz, w_z, out, &copy_loss);
+    bool copy_grad = false;
+    if (grad) {
+        gcpk::GradOutSpec go{};
+        go.loss = loss;
+        go.rows = c->total_rows;
+        go.Rp = c->Rp;
+        go.R = c->R;
+        go.G = c->G;
+        if (c->opt.mttkrp != GCP_MTTKRP_DETERMINISTIC && f.nrep) {
+            go.Htot = f.Htot;
+            go.nrep = f.nrep;
+            go.Grep = f.Grep;
+            go.hot_slot = c->hot_slot;
+            go.hot_row = c->hot_row;
+        }
+        const bool direct = out.G && kernel_writable(c, out.G, sizeof(float));
+        go.out = direct ? out.G : nullptr;
+        copy_grad = out.G && !direct;
+        GCP_CUDA(c, gcpk::launch_grad_finish(go, c->st));
+    } else {
+        GCP_CUDA(c, gcpk::launch_finish_loss(loss, c->st));
+    }
+    if (copy_grad && (s = copy_grad_out(c, out.G))) return s;
+    if (copy_loss && (s = copy_loss_out(c, out.dloss))) return s;
     return GCP_OK;
 }
 
@@ -379,10 +464,14 @@ gcp_status adam_step_impl(gcp_ctx *c, const gcp_adam_params *prm, int64_t t) {
 // One training step: sampled gradient of iteration `iter` and Adam step t.
 // With the atomic MTTKRP the epilogue (replica fold, loss finish, Adam, G
 // cleared for the next step) is one launch after the fused pass.
-gcp_status do_step(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, const gcp_adam_params *prm, int64_t t) {
+// dloss_out (device, nullable) receives the loss.
+gcp_status do_step(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, const gcp_adam_params *prm, int64_t t,
+                   double *dloss_out) {
     gcp_status s;
+    Outputs out;
+    out.dloss = dloss_out;
     if (c->opt.mttkrp != GCP_MTTKRP_ATOMIC) {
-        if ((s = run_fused(c, iter, p, q, true, nullptr))) return s;
+        if ((s = run_fused(c, iter, p, q, true, nullptr, out))) return s;
         return adam_step_impl(c, prm, t);
     }
     if ((s = check_counts(c, p, q))) return s;
@@ -416,15 +505,11 @@ gcp_status do_step(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, const gcp_ad
     ps.c2inv = (float)(1.0 / c2);
     ps.eps = (float)prm->eps;
     ps.lower = (float)prm->lower;
-    ps.partials = c->partials;
-    ps.nblocks = blocks;
-    ps.w_nz = w_nz;
-    ps.w_z = w_z;
-    ps.dloss = c->dloss;
-    ps.status = c->status;
+    bool copy_loss = false;
+    ps.loss = loss_spec(c, blocks, w_nz, w_z, out, &copy_loss);
     GCP_CUDA(c, gcpk::launch_post_step(ps, c->st));
     c->g_clear = true;
-    return GCP_OK;
+    return copy_loss ? copy_loss_out(c, dloss_out) : GCP_OK;
 }
 
 // Values of a dense tensor: bit GCP_ERR_ARG for a non-finite value, bit
@@ -512,17 +597,9 @@ static cudaError_t copy_rows(void *dst, size_t dpitch, const void *src, size_t s
 }
 
 gcp_status copy_grad_out(gcp_ctx *c, float *G_out) {
-    if (!G_out) return GCP_OK;
     GCP_CUDA(c, copy_rows(G_out, (size_t)c->R * 4, c->G, (size_t)c->Rp * 4, (size_t)c->R * 4,
                                   (size_t)c->total_rows, c->st));
     return GCP_OK;
-}
-
-gcp_status read_loss(gcp_ctx *c, double *loss_out) {
-    GCP_CUDA(c, cudaMemcpyAsync(c->h_loss, c->dloss, 2 * sizeof(double), cudaMemcpyDeviceToHost, c->st));
-    gcp_status s = collect(c);
-    if (loss_out) *loss_out = c->h_loss[0];
-    return s;
 }
 
 gcp_status refresh_bf16(gcp_ctx *c) {
@@ -807,41 +884,44 @@ gcp_status gcp_sample(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, int32_t *
 gcp_status gcp_loss(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, double *loss_out) {
     if (!c || !loss_out) return fail(c, GCP_ERR_ARG, "NULL argument");
     DeviceGuard g(c->device);
-    gcp_status s = run_fused(c, iter, p, q, false, nullptr);
+    Outputs out;
+    out.host = true;
+    gcp_status s = run_fused(c, iter, p, q, false, nullptr, out);
     if (s) return s;
-    return read_loss(c, loss_out);
+    s = host_result(c);
+    *loss_out = c->h_loss[0];
+    return s;
 }
 
 gcp_status gcp_loss_async(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, double *dloss_out) {
     if (!c || !dloss_out) return fail(c, GCP_ERR_ARG, "NULL argument");
     DeviceGuard g(c->device);
-    gcp_status s = run_fused(c, iter, p, q, false, nullptr);
-    if (s) return s;
-    GCP_CUDA(c, cudaMemcpyAsync(dloss_out, c->dloss, sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    return GCP_OK;
+    Outputs out;
+    out.dloss = dloss_out;
+    return run_fused(c, iter, p, q, false, nullptr, out);
 }
 
 gcp_status gcp_grad(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, float *G_out, double *loss_out) {
     if (!c) return fail(c, GCP_ERR_ARG, "NULL context");
     DeviceGuard g(c->device);
-    gcp_status s = run_fused(c, iter, p, q, true, nullptr);
-    if (s) return s;
-    s = copy_grad_out(c, G_out);
-    if (s) return s;
-    return loss_out ? read_loss(c, loss_out) : GCP_OK;
+    Outputs out;
+    out.G = G_out;
+    out.host = loss_out != nullptr;
+    gcp_status s = run_fused(c, iter, p, q, true, nullptr, out);
+    if (s || !loss_out) return s;
+    s = host_result(c);
+    *loss_out = c->h_loss[0];
+    return s;
 }
 
 gcp_status gcp_grad_async(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, const float *dscale, float *G_out,
                           double *dloss_out) {
     if (!c) return fail(c, GCP_ERR_ARG, "NULL context");
     DeviceGuard g(c->device);
-    gcp_status s = run_fused(c, iter, p, q, true, dscale);
-    if (s) return s;
-    s = copy_grad_out(c, G_out);
-    if (s) return s;
-    if (dloss_out)
-        GCP_CUDA(c, cudaMemcpyAsync(dloss_out, c->dloss, sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    return GCP_OK;
+    Outputs out;
+    out.G = G_out;
+    out.dloss = dloss_out;
+    return run_fused(c, iter, p, q, true, dscale, out);
 }
 
 gcp_status gcp_grad_factors_async(gcp_ctx *c, const float *const *A_modes, uint64_t iter, int64_t p, int64_t q,
@@ -871,11 +951,10 @@ gcp_status gcp_grad_factors_async(gcp_ctx *c, const float *const *A_modes, uint6
     k_stage_factors<<<(unsigned)(want < 8192 ? want : 8192), 256, 0, c->st>>>(
         src, c->d, c->R, log2Rp, n, c->A, static_cast<__nv_bfloat16 *>(c->Abf));
     GCP_CUDA(c, cudaGetLastError());
-    if ((s = run_fused(c, iter, p, q, G_out != nullptr, nullptr))) return s;
-    if ((s = copy_grad_out(c, G_out))) return s;
-    if (dloss_out)
-        GCP_CUDA(c, cudaMemcpyAsync(dloss_out, c->dloss, sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    return GCP_OK;
+    Outputs out;
+    out.G = G_out;
+    out.dloss = dloss_out;
+    return run_fused(c, iter, p, q, G_out != nullptr, nullptr, out);
 }
 
 gcp_status gcp_scale_async(gcp_ctx *c, const double *dscale, const float *x, float *y, int64_t n) {
@@ -902,11 +981,7 @@ gcp_status gcp_step(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, const gcp_a
     if (!(prm->beta1 >= 0.0 && prm->beta1 < 1.0 && prm->beta2 >= 0.0 && prm->beta2 < 1.0 && prm->eps >= 0.0))
         return fail(c, GCP_ERR_ARG, "Adam parameters out of range");
     DeviceGuard g(c->device);
-    gcp_status s = do_step(c, iter, p, q, prm, t);
-    if (s) return s;
-    if (dloss_out)
-        GCP_CUDA(c, cudaMemcpyAsync(dloss_out, c->dloss, sizeof(double), cudaMemcpyDeviceToDevice, c->st));
-    return GCP_OK;
+    return do_step(c, iter, p, q, prm, t, dloss_out);
 }
 
 gcp_status gcp_grad_norm(gcp_ctx *c, double *norm_out) {
@@ -947,9 +1022,12 @@ gcp_status gcp_fit(gcp_ctx *c, const gcp_fit_params *prm, gcp_fit_report *rep) {
     std::memset(&r, 0, sizeof(r));
     const auto t0 = std::chrono::steady_clock::now();
     auto objective = [&](double &F) -> gcp_status {
-        gcp_status s = run_fused(c, GCP_ITER_OBJECTIVE, prm->p_obj, prm->q_obj, false, nullptr);
+        Outputs out;
+        out.host = true;
+        gcp_status s = run_fused(c, GCP_ITER_OBJECTIVE, prm->p_obj, prm->q_obj, false, nullptr, out);
         if (s) return s;
-        s = read_loss(c, &F);
+        s = host_result(c);
+        F = c->h_loss[0];
         r.attempts_per_zero = prm->q_obj > 0 ? c->h_loss[1] / (double)prm->q_obj : 0.0;
         return s;
     };
@@ -971,7 +1049,7 @@ gcp_status gcp_fit(gcp_ctx *c, const gcp_fit_params *prm, gcp_fit_report *rep) {
     if ((s = backup(true))) return s;
     for (int epoch = 0; epoch < prm->max_epochs; ++epoch) {
         for (int it = 0; it < prm->iters; ++it) {
-            if ((s = do_step(c, iter++, prm->p, prm->q, &adam, t + 1))) return s;
+            if ((s = do_step(c, iter++, prm->p, prm->q, &adam, t + 1, nullptr))) return s;
             ++t;
             ++steps_run;
         }

@@ -60,9 +60,35 @@ struct FusedSpec {
 // (replicas_for): none, 4, 16 or all 64.
 constexpr int kReplicas = 64;
 
+// Where a call's sampled loss goes once the block partials are summed: the
+// context's own words, and, where given, a caller's device double and the
+// pinned mirrors that a host-value call reads after it has synchronised.
+struct LossSpec {
+    const double *partials;
+    int nblocks;
+    double w_nz, w_z;
+    double *dloss;                  // [0] loss, [1] zero attempts
+    double *out;                    // device, or null
+    int *status;
+    double *h_loss;                 // pinned mirrors of dloss[0..1] and *status, or null
+    int *h_status;
+};
+
+// The epilogue of a gradient call: loss, replica fold and the copy of the
+// gradient into the caller's unpadded array in one launch.
+struct GradOutSpec {
+    LossSpec loss;
+    int64_t rows;
+    int Rp, R, Htot, nrep;          // nrep 0: no replicas (Htot 0, hot_slot null)
+    float *G, *Grep;
+    const int *hot_slot, *hot_row;
+    float *out;                     // rows x R, or null
+};
+
 // The epilogue of one training step (gcp_step): loss finish, replica fold,
 // Adam and gradient clearing in one launch.
 struct PostSpec {
+    LossSpec loss;
     int64_t n;                      // total_rows * Rp
     int Rp, R, Htot, nrep;          // nrep 0: no replicas (Htot 0, hot_slot null)
     float *G, *Grep, *A, *B, *C;
@@ -70,11 +96,6 @@ struct PostSpec {
     const int *hot_slot;            // row -> replica slot, or -1
     const int *hot_row;             // replica slot -> row
     float lr, beta1, beta2, c1inv, c2inv, eps, lower;
-    const double *partials;
-    int nblocks;
-    double w_nz, w_z;
-    double *dloss;
-    int *status;
 };
 
 struct LaunchCfg {
@@ -92,12 +113,10 @@ cudaError_t launch_sample(const SampleSpec &s, int32_t *idx_out, float *x_out, f
                           float w_z, cudaStream_t st);
 cudaError_t launch_fused(const FusedSpec &f, bool bf16, int cols, int max_blocks, cudaStream_t st,
                          int *blocks_used);
-cudaError_t launch_fold_replicas(float *G, float *Grep, const int *hot_row, int Htot, int Rp, int nrep,
-                                 cudaStream_t st);
+cudaError_t launch_grad_finish(const GradOutSpec &p, cudaStream_t st);
 cudaError_t launch_mttkrp_nonfused(const FusedSpec &f, const int *hot_slot, bool bf16, int cols, int max_blocks,
                                    cudaStream_t st);
-cudaError_t launch_finish_loss(const double *partials, int nblocks, double w_nz, double w_z, double *dloss,
-                               int *status, cudaStream_t st);
+cudaError_t launch_finish_loss(const LossSpec &l, cudaStream_t st);
 cudaError_t launch_adam(int64_t n, int Rp, int R, float *A, float *B, float *C, const float *G, float lr,
                         float beta1, float beta2, float c1inv, float c2inv, float eps, float lower,
                         void *Abf, cudaStream_t st);

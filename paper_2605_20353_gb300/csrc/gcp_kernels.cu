@@ -358,38 +358,13 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
     }
 }
 
-// G(hot row) += sum over replicas, then the replicas are cleared for the
-// next call (fixed replica order).  G may already hold contributions of
-// drawn cells to a replicated row of a large mode.  All NREP loads of
-// an element are issued before any add: there are few hot elements, so one
-// round trip per element beats the occupancy that fewer registers would
-// give (16 of 64 loads at a time measured 8 us against 5 us per launch).
-template <int NREP>
-__global__ void k_fold_replicas(float *__restrict__ G, float *__restrict__ Grep, const int *__restrict__ hot_row,
-                                int Htot, int Rp) {
-    const int64_t n = (int64_t)Htot * Rp, plane = n;
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        float v[NREP];
-#pragma unroll
-        for (int r = 0; r < NREP; ++r) v[r] = Grep[r * plane + e];
-        float t = 0.0f;
-#pragma unroll
-        for (int r = 0; r < NREP; ++r) t += v[r];
-#pragma unroll
-        for (int r = 0; r < NREP; ++r) Grep[r * plane + e] = 0.0f;
-        const int log2Rp = __ffs(Rp) - 1;  // Rp is a power of two
-        const int slot = (int)(e >> log2Rp), col = (int)(e & (Rp - 1));
-        G[(int64_t)hot_row[slot] * Rp + col] += t;
-    }
-}
-
-// Fixed-order reduction of the block partials (one block).
-__global__ void __launch_bounds__(kThreads) k_finish_loss(const double *__restrict__ partials, int nblocks,
-                                                         double w_nz, double w_z, double *dloss, int *status) {
+// ------------------------------------------------- loss, fold, gradient out
+// Fixed-order reduction of the block partials by one block of kThreads.
+__device__ __forceinline__ void finish_loss_block(const LossSpec &l) {
     __shared__ double sh[3][kThreads];
     double t[3] = {0.0, 0.0, 0.0};
-    for (int b = threadIdx.x; b < nblocks; b += kThreads)
-        for (int c = 0; c < 3; ++c) t[c] += partials[4 * b + c];
+    for (int b = threadIdx.x; b < l.nblocks; b += kThreads)
+        for (int c = 0; c < 3; ++c) t[c] += l.partials[4 * b + c];
     for (int c = 0; c < 3; ++c) sh[c][threadIdx.x] = t[c];
     __syncthreads();
     for (int w = kThreads / 2; w > 0; w >>= 1) {
@@ -398,10 +373,93 @@ __global__ void __launch_bounds__(kThreads) k_finish_loss(const double *__restri
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        const double loss = w_nz * sh[0][0] + w_z * sh[1][0];
-        dloss[0] = loss;
-        dloss[1] = sh[2][0];
-        if (!isfinite(loss)) atomicOr(status, kErrNonfinite);
+        const double loss = l.w_nz * sh[0][0] + l.w_z * sh[1][0];
+        l.dloss[0] = loss;
+        l.dloss[1] = sh[2][0];
+        if (l.out) *l.out = loss;
+        const int bits = isfinite(loss) ? 0 : kErrNonfinite;
+        if (l.h_loss) {
+            l.h_loss[0] = loss;
+            l.h_loss[1] = sh[2][0];
+            // every earlier kernel of the stream has set its bits; this one's
+            // are the non-finite loss alone
+            *l.h_status = atomicOr(l.status, bits) | bits;
+        } else if (bits) {
+            atomicOr(l.status, bits);
+        }
+    }
+}
+
+__global__ void __launch_bounds__(kThreads) k_finish_loss(const LossSpec l) { finish_loss_block(l); }
+
+// The epilogue of a gradient call after the fused pass, in one launch:
+//  - the last block finishes the FP64 loss (and hands it to the caller's
+//    device word or the pinned mirrors);
+//  - with a caller's array, the first `ncold` blocks copy the rows of G that
+//    have no replicas into its rows of R columns, V columns per thread (V = 4
+//    where R and the array's address allow 16-byte stores);
+//  - the blocks between take the quads of hot rows, one per group of NREP / 4
+//    lanes: all replica quads of a hot quad are in flight at once
+//    (gcpe::hot_quad_sum, which clears them for the next call), and the
+//    group's first lane adds them to G (which may already hold contributions
+//    of drawn cells to a replicated row of a large mode) and to the copy.
+// Latency bound on small models, bandwidth bound on large ones.  It takes the
+// place of a fold launch, a loss launch, a (strided) copy of the gradient,
+// one of the loss and, for host results, two copies into pinned words: the
+// smallest gradient call 32.2 -> 23.5 us, rank 50 on 172 x 25,000 x 300 at
+// 2^16 samples 47.4 -> 30.2 us, rank 20 on 4999 x 3001 x 777 at 250,000
+// samples 52.2 -> 41.0 us.
+template <int NREP, int V>
+__global__ void __launch_bounds__(kThreads) k_grad_finish(const GradOutSpec P, int ncold) {
+    if (blockIdx.x == gridDim.x - 1) {
+        finish_loss_block(P.loss);
+        return;
+    }
+    float4 *__restrict__ G4 = reinterpret_cast<float4 *>(P.G);
+    if constexpr (NREP > 0) {
+        if ((int)blockIdx.x >= ncold) {
+            constexpr int H = gcpe::hot_lanes<NREP>();
+            const int log2Q = __ffs(P.Rp) - 3;  // log2 of the quads of a row (Rp is a power of two)
+            const int64_t hq = (int64_t)(blockIdx.x - ncold) * (kThreads / H) + (threadIdx.x / H);
+            if (hq >= ((int64_t)P.Htot << log2Q)) return;  // the whole group leaves together
+            const int slot = (int)(hq >> log2Q), cq = (int)(hq & ((1 << log2Q) - 1));
+            const int row = __ldg(P.hot_row + slot);
+            const int64_t q = ((int64_t)row << log2Q) + cq;
+            const bool lead = (threadIdx.x & (H - 1)) == 0;
+            float4 g;
+            if (lead) g = G4[q];
+            const float4 t = gcpe::hot_quad_sum<NREP>(reinterpret_cast<float4 *>(P.Grep),
+                                                      ((int64_t)P.Htot * P.Rp) >> 2, hq, gcpe::hot_group_mask<NREP>());
+            if (!lead) return;
+            g.x += t.x;
+            g.y += t.y;
+            g.z += t.z;
+            g.w += t.w;
+            G4[q] = g;
+            if (!P.out) return;
+            const int col = cq << 2;
+            float *o = P.out + (int64_t)row * P.R + col;
+            if (V == 4) {
+                if (col < P.R) *reinterpret_cast<float4 *>(o) = g;
+            } else {
+                const float gv[4] = {g.x, g.y, g.z, g.w};
+#pragma unroll
+                for (int j = 0; j < 4; ++j)
+                    if (col + j < P.R) o[j] = gv[j];
+            }
+            return;
+        }
+    }
+    const unsigned units = (unsigned)(P.R / V);  // vectors or columns of a row
+    const int64_t n = P.rows * units;            // below 2^31
+    for (int64_t e = (int64_t)blockIdx.x * kThreads + threadIdx.x; e < n; e += (int64_t)ncold * kThreads) {
+        const unsigned row = (unsigned)e / units, u = (unsigned)e - row * units;
+        if (NREP > 0 && __ldg(P.hot_slot + row) >= 0) continue;  // the hot blocks' rows
+        const float *g = P.G + (int64_t)row * P.Rp + V * u;
+        if (V == 4)
+            reinterpret_cast<float4 *>(P.out)[e] = *reinterpret_cast<const float4 *>(g);
+        else
+            P.out[e] = *g;
     }
 }
 
@@ -518,23 +576,7 @@ constexpr int kPostUnroll = 1;
 template <int NREP>
 __global__ void __launch_bounds__(kThreads) k_post_step(PostSpec P, int ncold) {
     if (blockIdx.x == gridDim.x - 1) {  // the last block only finishes the loss
-        __shared__ double sh[3][kThreads];
-        double t[3] = {0.0, 0.0, 0.0};
-        for (int b = threadIdx.x; b < P.nblocks; b += kThreads)
-            for (int c = 0; c < 3; ++c) t[c] += P.partials[4 * b + c];
-        for (int c = 0; c < 3; ++c) sh[c][threadIdx.x] = t[c];
-        __syncthreads();
-        for (int w = kThreads / 2; w > 0; w >>= 1) {
-            if (threadIdx.x < w)
-                for (int c = 0; c < 3; ++c) sh[c][threadIdx.x] += sh[c][threadIdx.x + w];
-            __syncthreads();
-        }
-        if (threadIdx.x == 0) {
-            const double loss = P.w_nz * sh[0][0] + P.w_z * sh[1][0];
-            P.dloss[0] = loss;
-            P.dloss[1] = sh[2][0];
-            if (!isfinite(loss)) atomicOr(P.status, kErrNonfinite);
-        }
+        finish_loss_block(P.loss);
         return;
     }
     float4 *__restrict__ G4 = reinterpret_cast<float4 *>(P.G);
@@ -858,22 +900,36 @@ cudaError_t launch_mttkrp_nonfused(const FusedSpec &f, const int *hot_slot, bool
     return cudaGetLastError();
 }
 
-cudaError_t launch_fold_replicas(float *G, float *Grep, const int *hot_row, int Htot, int Rp, int nrep,
-                                 cudaStream_t st) {
-    if (Htot == 0 || nrep == 0) return cudaSuccess;
-    const int blocks = elementwise_blocks((int64_t)Htot * Rp);
-    switch (nrep) {
-    case 4: k_fold_replicas<4><<<blocks, kThreads, 0, st>>>(G, Grep, hot_row, Htot, Rp); break;
-    case 16: k_fold_replicas<16><<<blocks, kThreads, 0, st>>>(G, Grep, hot_row, Htot, Rp); break;
-    case 64: k_fold_replicas<64><<<blocks, kThreads, 0, st>>>(G, Grep, hot_row, Htot, Rp); break;
-    default: return cudaErrorInvalidValue;
+template <int NREP, int V>
+static cudaError_t launch_grad_finish_rv(const GradOutSpec &p, cudaStream_t st) {
+    const int ncold = p.out ? elementwise_blocks(p.rows * (p.R / V)) : 0;
+    int nhot = 0;
+    if constexpr (NREP > 0) {
+        constexpr int per = kThreads / gcpe::hot_lanes<NREP>();  // hot quads of a block
+        nhot = (int)(((int64_t)p.Htot * (p.Rp >> 2) + per - 1) / per);
     }
+    k_grad_finish<NREP, V><<<ncold + nhot + 1, kThreads, 0, st>>>(p, ncold);  // + the loss block
     return cudaGetLastError();
 }
 
-cudaError_t launch_finish_loss(const double *partials, int nblocks, double w_nz, double w_z, double *dloss,
-                               int *status, cudaStream_t st) {
-    k_finish_loss<<<1, kThreads, 0, st>>>(partials, nblocks, w_nz, w_z, dloss, status);
+template <int NREP>
+static cudaError_t launch_grad_finish_r(const GradOutSpec &p, cudaStream_t st) {
+    const bool vec = p.R % 4 == 0 && (reinterpret_cast<uintptr_t>(p.out) & 15) == 0;
+    return vec ? launch_grad_finish_rv<NREP, 4>(p, st) : launch_grad_finish_rv<NREP, 1>(p, st);
+}
+
+cudaError_t launch_grad_finish(const GradOutSpec &p, cudaStream_t st) {
+    switch (p.nrep) {
+    case 0: return launch_grad_finish_r<0>(p, st);
+    case 4: return launch_grad_finish_r<4>(p, st);
+    case 16: return launch_grad_finish_r<16>(p, st);
+    case 64: return launch_grad_finish_r<64>(p, st);
+    default: return cudaErrorInvalidValue;
+    }
+}
+
+cudaError_t launch_finish_loss(const LossSpec &l, cudaStream_t st) {
+    k_finish_loss<<<1, kThreads, 0, st>>>(l);
     return cudaGetLastError();
 }
 

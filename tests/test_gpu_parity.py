@@ -271,6 +271,47 @@ def test_grad_scale_and_async_loss(env):
 
 
 # ---------------------------------------------------------------- Adam
+@pytest.mark.parametrize("where", ["vector", "offset", "host", "pinned"])
+@pytest.mark.parametrize("mttkrp,p,q", [("atomic", 60000, 50000), ("atomic", 7000, 6001), ("atomic", 900, 700),
+                                        ("atomic", 150, 130), ("deterministic", 900, 700)])
+@pytest.mark.parametrize("R", [1, 6, 20, 33])
+def test_gradient_copied_out_to_any_array(env, R, mttkrp, p, q, where):
+    """The gradient's unpadded copy, written by the epilogue (64, 16, 4 or no
+    replicas) to a device array on a 16-byte boundary or 4 bytes past one,
+    or copied to host memory: entry for entry the gradient of the same call
+    (held in the context, read through its norm) and nothing outside the
+    array; the loss in the caller's device double, aligned or 4 bytes off,
+    equals the host's."""
+    gcp, torch = env
+    dims = [8, 41, 700]
+    coords, vals, factors = problem(dims, 5000, R, "poisson", 611)
+    ctx = gcp.gcp_create(dims, coords, vals, R, "poisson", seed=612, mttkrp=mttkrp)
+    ctx.set_factors(factors)
+    n, lib = ctx.num_params, gcp.load()
+    shift = 0 if where == "vector" else 1
+    if where in ("vector", "offset"):
+        buf = torch.full((n + 9,), 7.0, device="cuda")
+    else:
+        buf = torch.full((n + 9,), 7.0, pin_memory=where == "pinned")
+    dl = torch.zeros(4, dtype=torch.float64, device="cuda")
+    loss_at = dl.data_ptr() + (8 if where == "vector" else 4)
+    assert lib.gcp_grad_async(ctx.handle, 3, p, q, None, buf.data_ptr() + 4 * shift, loss_at) == 0
+    norm = ctx.grad_norm()
+    torch.cuda.synchronize()
+    got = buf.cpu()
+    assert bool((got[:shift] == 7.0).all()) and bool((got[shift + n:] == 7.0).all())
+    idx, x, w, _ = oracle.stratified_samples(612, 3, p, q, dims, coords, vals)
+    Lo, Go = oracle.sampled_loss_grad(dims, factors, "poisson", idx, x, w)
+    G = got[shift:shift + n].numpy()
+    assert rel_err(G, np.concatenate([g.ravel() for g in Go])) <= TOL_FP32
+    assert norm == pytest.approx(np.linalg.norm(G.astype(np.float64)), rel=1e-12)
+    raw = dl.cpu().numpy().tobytes()
+    L = np.frombuffer(raw[8:16] if where == "vector" else raw[4:12], dtype=np.float64)[0]
+    assert L == ctx.loss_value(3, p, q)
+    assert abs(L - Lo) <= TOL_FP32 * abs(Lo)
+    ctx.close()
+
+
 def test_adam_step_parity(env):
     gcp, torch = env
     dims = [30, 20, 10]

@@ -297,6 +297,7 @@ gcpk::FusedSpec gcpk_make_spec(const gcp_ctx *c, uint64_t iter, int64_t p, int64
     f.F = c->Abf ? c->Abf : (const void *)c->A;
     f.G = grad ? c->G : nullptr;
     f.Rp = c->Rp;
+    f.R = c->R;
     f.log2L = c->log2L;
     for (int k = 0; k < c->d; ++k) f.rowoff[k] = (int)c->rowoff[k];
     f.loss = c->loss;

@@ -61,7 +61,7 @@ __device__ __forceinline__ int client_of(const int *__restrict__ tile_start, int
 // take the tile's samples in turn.  Per tile, the FP32 loss sums (nonzero,
 // zero) go to tile_loss[tile].
 template <int D, typename TF, int COLS, int TS>
-__global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) k_batch_fused(const int4 *__restrict__ specs,
+__global__ void __launch_bounds__(kThreads, gcpk::fused_min_blocks(D, COLS)) k_batch_fused(const int4 *__restrict__ specs,
                                                          const int *__restrict__ tile_start, int nclients,
                                                          int total_tiles, int log2L, int Rp,
                                                          const uint64_t *__restrict__ step, float2 *tile_loss) {

@@ -37,6 +37,8 @@ struct FusedSpec {
     const void *F;                  // factors the kernels read (FP32 or BF16), row stride Rp
     float *G;                       // gradient, row stride Rp; null = loss only
     int Rp;                         // padded row length: cols x lanes per sample (power of 2)
+    int R;                          // rank: columns R .. Rp - 1 hold zeros
+    int tile;                       // samples per warp tile, at most 32 (launch_fused)
     int log2L;                      // log2(lanes per sample); each lane owns cols = 4 or 8 columns
     int rowoff[GCP_MAX_NDIM];       // first row of each mode in F and G
     int loss;
@@ -98,10 +100,15 @@ struct PostSpec {
     float lr, beta1, beta2, c1inv, c2inv, eps, lower;
 };
 
-struct LaunchCfg {
-    int blocks;
-    int threads;
-};
+// Blocks of 256 threads per SM that the fused kernels are held to, as many as
+// leave at most a few bytes of spills: 64 registers (4 blocks) for orders up
+// to 4 with 4 columns per lane, 80 (3 blocks) for orders 5 to 7 and for 8
+// columns up to order 4, else 128 (2 blocks).  Left alone the compiler takes
+// 116 registers at order 5 (2 blocks): 2^22 samples of the dense 5-way
+// tensor at rank 16 then take 365 us forward and backward, against 334 us.
+__host__ __device__ constexpr int fused_min_blocks(int d, int cols) {
+    return d <= 4 ? (cols == 4 ? 4 : 3) : (cols == 4 && d <= 7 ? 3 : 2);
+}
 
 // ---------------------------------------------------------------- kernels
 // All launches are asynchronous on `st`; device errors go to the status word.

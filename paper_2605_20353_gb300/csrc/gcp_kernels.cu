@@ -111,7 +111,7 @@ __device__ __forceinline__ bool draw_sample(const SampleSpec &S, int64_t s, int3
 }
 
 // ------------------------------------------------------------ fused pass
-// Per warp and per tile of 32 consecutive samples:
+// Per warp and per tile of P.tile <= 32 consecutive samples (fused_tile):
 //   A1 (tile t+1, one sample per lane): Philox draw; the nonzero record, the
 //      dense value or the first hash bucket of the zero candidate is copied
 //      into shared memory with cp.async while tile t is processed;
@@ -120,7 +120,10 @@ __device__ __forceinline__ bool draw_sample(const SampleSpec &S, int64_t s, int3
 //   B  (tile t, one sample per group of L = Rp/COLS lanes): lane g owns
 //      COLS columns as COLS/4 quads (4g..4g+3, and Rp/2+4g.. when COLS = 8),
 //      so a group's loads and vector reductions cover whole 32-byte sectors
-//      and, for rows up to 128 bytes, one whole row per instruction.
+//      and, for rows up to 128 bytes, one whole row per instruction.  Quads
+//      beyond the rank hold zeros and are not reduced; they are loaded, as
+//      a test around the loads costs more than the sectors (orders 2 to 8,
+//      ranks 20 to 65, 2^20 samples: 0 to 15% slower with it).
 // Gradient rows that many samples hit go to one of the call's nrep replicas
 // (chosen by warp), folded into G afterwards, so that the reductions of hot
 // rows do not serialise on one address; with nrep = 0 (few samples) every
@@ -128,7 +131,7 @@ __device__ __forceinline__ bool draw_sample(const SampleSpec &S, int64_t s, int3
 constexpr int kWarps = kThreads / 32;
 
 template <int D, typename TF, int COLS>
-__global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) k_fused(const FusedSpec P) {
+__global__ void __launch_bounds__(kThreads, fused_min_blocks(D, COLS)) k_fused(const FusedSpec P) {
     constexpr int SW = rec_words_for(D);  // words per staged sample: coordinates, value, replica slots
     constexpr int NQ = COLS / 4;          // quads of columns per lane
     __shared__ __align__(16) int32_t s_slot[2][kWarps][32][SW];
@@ -143,11 +146,16 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
     const int ngrp = 32 >> log2L;
     const unsigned gmask = (L == 32) ? 0xFFFFFFFFu : (((1u << L) - 1u) << (grp * L));
     int col[NQ];
+    bool on[NQ];  // the quad holds columns of the rank, not padding alone
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) col[q] = q * (P.Rp >> 1) + 4 * glane;
+    for (int q = 0; q < NQ; ++q) {
+        col[q] = q * (P.Rp >> 1) + 4 * glane;
+        on[q] = col[q] < P.R;
+    }
     const int p = (int)P.s.p;  // sample counts of one call are below 2^31
     const int S = (int)(P.s.p + P.s.q);
-    const int ntiles = (int)(((int64_t)S + 31) >> 5);  // S may be 2^31 - 1
+    const unsigned TS = P.tile;
+    const int ntiles = (int)(((int64_t)S + TS - 1) / TS);  // S may be 2^31 - 1
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     const int warp0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const TF *__restrict__ F = static_cast<const TF *>(P.F);
@@ -162,10 +170,11 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
     // A1: start the draw of this lane's sample of `tile` into stage `st`;
     // returns the key of a stratified zero candidate (kEmpty otherwise).
     auto issue = [&](int tile, int st) -> uint64_t {
-        if (tile >= ntiles) return kEmpty;
-        const int s = (tile << 5) + lane;
+        if (tile >= ntiles || lane >= (int)TS) return kEmpty;
+        const unsigned us = (unsigned)tile * TS + lane;  // may pass 2^31 - 1 in the last tile
         int32_t *slot = s_slot[st][warp][lane];
-        if (s >= S) return kEmpty;
+        if (us >= (unsigned)S) return kEmpty;
+        const int s = (int)us;
         if (uniform) {
             int32_t idx[D];
             draw_tuple<D>(P.s, kStreamUniform, (uint64_t)s, 0, idx);
@@ -196,8 +205,9 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
 
     // A2: finish the draw of stage `st`; returns whether the sample exists.
     auto finish = [&](int tile, int st, uint64_t key) -> bool {
-        const int s = (tile << 5) + lane;
-        if (s >= S) return false;
+        const unsigned us = (unsigned)tile * TS + lane;
+        if (lane >= (int)TS || us >= (unsigned)S) return false;
+        const int s = (int)us;
         if (key == kEmpty) return true;  // nonzero, semi-stratified or dense draw
         const ulonglong2 lo = *reinterpret_cast<const ulonglong2 *>(&s_bkt[st][warp][lane][0]);
         const ulonglong2 hi = *reinterpret_cast<const ulonglong2 *>(&s_bkt[st][warp][lane][2]);
@@ -247,11 +257,11 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
         // phase B: one sample per group; the group leader keeps FP32 loss
         // sums of the tile, added to the FP64 totals once per tile
         float tf_nz = 0.0f, tf_z = 0.0f;
-        for (int it = 0; it < L; ++it) {
+        for (int it = 0; it * ngrp < (int)TS; ++it) {
             const int src = it * ngrp + grp;
             if (!((okmask >> src) & 1u)) {  // uniform within the group
-                const int sm = (tile << 5) + src;
-                if (P.Yval && glane == 0 && sm < S) {  // no sample: a zero entry at a valid cell
+                const unsigned sm = (unsigned)tile * TS + src;
+                if (P.Yval && glane == 0 && src < (int)TS && sm < (unsigned)S) {  // no sample: a zero entry at a valid cell
 #pragma unroll
                     for (int k = 0; k < D; ++k) P.Ycoord[(int64_t)sm * P.ystride + k] = s_slot[st][warp][src][k];
                     P.Yval[(int64_t)sm * P.vstride] = 0.0f;
@@ -263,7 +273,7 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
 #pragma unroll
             for (int k = 0; k < D; ++k) ii[k] = slot[k];
             const float xs = __int_as_float(slot[D]);
-            const bool is_nz = !uniform && ((tile << 5) + src) < p;
+            const bool is_nz = !uniform && ((unsigned)tile * TS + src) < (unsigned)p;
 
             int off[D];
             float a[D][COLS];
@@ -299,7 +309,7 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
                 tf_z += f;
             if (P.Yval) {  // materialize the gradient tensor entry (non-fused MTTKRP input)
                 if (glane == 0) {
-                    const int sm = (tile << 5) + src;
+                    const int sm = tile * TS + src;
 #pragma unroll
                     for (int k = 0; k < D; ++k) P.Ycoord[(int64_t)sm * P.ystride + k] = ii[k];
                     P.Yval[(int64_t)sm * P.vstride] = ((is_nz || uniform) ? P.w_nz : P.w_z) * df * scale;
@@ -321,7 +331,8 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
                     float *g = hs != kNoSlot ? grep + (int)hs * P.Rp : P.G + off[n];
 #pragma unroll
                     for (int q = 0; q < NQ; ++q)
-                        red_add_v4(g + col[q], pre[4 * q] * suf[n][4 * q], pre[4 * q + 1] * suf[n][4 * q + 1],
+                        if (on[q])
+                            red_add_v4(g + col[q], pre[4 * q] * suf[n][4 * q], pre[4 * q + 1] * suf[n][4 * q + 1],
                                    pre[4 * q + 2] * suf[n][4 * q + 2], pre[4 * q + 3] * suf[n][4 * q + 3]);
 #pragma unroll
                     for (int v = 0; v < COLS; ++v) pre[v] *= a[n][v];
@@ -335,20 +346,20 @@ __global__ void __launch_bounds__(kThreads, (D <= 4 ? (COLS == 4 ? 4 : 3) : 1)) 
     }
     cp_async_wait<0>();
 
-    // block reduction of the FP64 loss sums and attempt counts
-    double att = (double)attempts;
-#pragma unroll
-    for (int o = 16; o > 0; o >>= 1) {
+    // block reduction of the FP64 loss sums (held by the group leaders) and
+    // attempt counts; FP64 adds are slow here (16 cycles of the SM's pipe for
+    // a warp), so only the leaders' steps are taken
+    attempts = __reduce_add_sync(0xFFFFFFFFu, attempts);
+    for (int o = 16; o >= L; o >>= 1) {
         acc_nz += __shfl_xor_sync(0xFFFFFFFFu, acc_nz, o);
         acc_z += __shfl_xor_sync(0xFFFFFFFFu, acc_z, o);
-        att += __shfl_xor_sync(0xFFFFFFFFu, att, o);
     }
     double(*red)[kWarps] = reinterpret_cast<double(*)[kWarps]>(&s_bkt[0][0][0][0]);  // staging is free now
     __syncthreads();
     if (lane == 0) {
         red[0][warp] = acc_nz;
         red[1][warp] = acc_z;
-        red[2][warp] = att;
+        red[2][warp] = (double)attempts;
     }
     __syncthreads();
     if (threadIdx.x < 3) {
@@ -789,10 +800,26 @@ static void launch_fused_d(const FusedSpec &f, bool bf16, int cols, int blocks, 
     }
 }
 
-cudaError_t launch_fused(const FusedSpec &f, bool bf16, int cols, int max_blocks, cudaStream_t st,
+// Samples per warp tile: with r = ceil(S / (32 W)) rounds of tiles over the W
+// resident warps, the smallest tile that still takes r rounds (a multiple of
+// the samples that the warp's groups evaluate at once), so that every warp
+// has the same work: 250,000 samples on 4,864 warps are two rounds of 28
+// instead of one of 32 and 0.6 of another, and small sets spread over all
+// warps.
+static int fused_tile(int64_t S, int log2L, int64_t warps) {
+    const int ngrp = 32 >> log2L;
+    const int64_t rounds = (S + 32 * warps - 1) / (32 * warps);
+    if (rounds < 1) return 32;
+    const int64_t per = (S + warps * rounds - 1) / (warps * rounds);
+    return (int)((per + ngrp - 1) / ngrp * ngrp);
+}
+
+cudaError_t launch_fused(const FusedSpec &spec, bool bf16, int cols, int max_blocks, cudaStream_t st,
                          int *blocks_used) {
+    FusedSpec f = spec;
     const int64_t S = f.s.p + f.s.q;
-    const int64_t ntiles = (S + 31) / 32;
+    f.tile = fused_tile(S, f.log2L, (int64_t)max_blocks * kWarps);
+    const int64_t ntiles = (S + f.tile - 1) / f.tile;
     int64_t want = (ntiles + kWarps - 1) / kWarps;
     if (want < 1) want = 1;
     const int blocks = (int)(want < max_blocks ? want : max_blocks);
@@ -827,8 +854,12 @@ __global__ void __launch_bounds__(kThreads) k_mttkrp_nonfused(const FusedSpec P,
     const TF *__restrict__ F = static_cast<const TF *>(P.F);
     float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (P.nrep - 1)) * P.Htot * P.Rp : nullptr;
     int col[NQ];
+    bool on[NQ];  // the quad holds columns of the rank, not padding alone
 #pragma unroll
-    for (int q = 0; q < NQ; ++q) col[q] = q * (P.Rp >> 1) + 4 * glane;
+    for (int q = 0; q < NQ; ++q) {
+        col[q] = q * (P.Rp >> 1) + 4 * glane;
+        on[q] = col[q] < P.R;
+    }
     for (int s = group; s < S; s += ngroups) {
         const float y = __ldg(P.Yval + (int64_t)s * P.vstride);
         int ii[D], off[D];
@@ -856,7 +887,8 @@ __global__ void __launch_bounds__(kThreads) k_mttkrp_nonfused(const FusedSpec P,
             float *g = hs >= 0 ? grep + hs * P.Rp : P.G + off[n];
 #pragma unroll
             for (int q = 0; q < NQ; ++q)
-                red_add_v4(g + col[q], pre[4 * q] * suf[n][4 * q], pre[4 * q + 1] * suf[n][4 * q + 1],
+                if (on[q])
+                    red_add_v4(g + col[q], pre[4 * q] * suf[n][4 * q], pre[4 * q + 1] * suf[n][4 * q + 1],
                            pre[4 * q + 2] * suf[n][4 * q + 2], pre[4 * q + 3] * suf[n][4 * q + 3]);
 #pragma unroll
             for (int v = 0; v < COLS; ++v) pre[v] *= a[n][v];

@@ -862,3 +862,26 @@ def test_l2_probe_performs_every_row_operation(env):
     total = float(wide.double().sum())
     assert abs(total - expect) <= 1e-4 * expect, (total, expect)
     assert float(wide.view(2048, 64).double().sum(0).min()) > 0.0  # every column was reached
+
+
+@pytest.mark.parametrize("R", [3, 4, 9, 17, 33, 65])
+def test_sample_counts_around_the_tile_rounds(env, R):
+    """The samples per warp tile follow the sample count: counts of one
+    sample, one tile, every resident warp with one tile (and one sample more
+    or fewer), and two rounds of uneven tiles, at one to 32 lanes a sample
+    with padded ranks; loss and gradient against the oracle."""
+    gcp, torch = env
+    dims = [61, 47, 900]
+    coords, vals, factors = problem(dims, 6000, R, "poisson", 711)
+    ctx = gcp.gcp_create(dims, coords, vals, R, "poisson", seed=712)
+    ctx.set_factors(factors)
+    warps = torch.cuda.get_device_properties(0).multi_processor_count * 32
+    for t, (p, q) in enumerate([(1, 0), (0, 1), (17, 16), (2 * warps, 2 * warps - 1), (2 * warps, 2 * warps + 1),
+                                (16 * warps, 16 * warps), (16 * warps, 16 * warps + 1), (40 * warps, 11 * warps + 3)]):
+        Lg, Gg = gpu_grad(gcp, torch, ctx, t, p, q)
+        idx, x, w, _ = oracle.stratified_samples(712, t, p, q, dims, coords, vals)
+        Lo, Go = oracle.sampled_loss_grad(dims, factors, "poisson", idx, x, w)
+        assert abs(Lg - Lo) <= TOL_FP32 * abs(Lo), (t, Lg, Lo)
+        for n, (a, b) in enumerate(zip(split(Gg, dims, R), Go)):
+            assert rel_err(a, b) <= TOL_FP32, (t, n, rel_err(a, b))
+    ctx.close()

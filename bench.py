@@ -35,7 +35,7 @@ WORKLOAD = ("zipf-count 4-way 2000x1500x1000x200, 5e7 nnz Zipf(1.1) coords, 1+Po
 L2_NOTE = ("inputs larger than L2 (1.6 GB records, 2.1 GB hash set); factors and gradient (0.6 MB each) stay "
            "L2-resident across steps as in training")
 CONFIG = {"workload": WORKLOAD, "l2": L2_NOTE}
-KERNEL_SOURCES = ["paper_2605_20353_gb300/csrc/gcp_kernels.cu", "paper_2605_20353_gb300/csrc/gcp_device.cuh"]
+KERNEL_SOURCES = ["paper_2605_20353_gb300/csrc/gcp_fused.cuh", "paper_2605_20353_gb300/csrc/gcp_device.cuh"]
 TRAFFIC_FILE = os.path.join(ROOT, "profiles", "fused_grad_zipf_count_traffic.json")
 
 
@@ -74,21 +74,13 @@ def compulsory_bytes_per_sample(d, R, nnz, M, rows, access_bytes=128, elt_bytes=
     return 0.5 * access_bytes + 0.5 * access_bytes * attempts + rows * R * (elt_bytes + 8) / float(1 << 21)
 
 
-# the fused pass's part of gcp_kernels.cu ends where the replica fold begins
-FUSED_SECTION_END = b"// G(hot row) += sum over replicas"
-
-
 def kernel_source_hash():
-    """Hash of the fused kernel's source: the device header and the part of
-    gcp_kernels.cu up to the replica fold (the whole file if that marker
-    moved), so that edits to other kernels keep the captured counters."""
+    """Hash of the fused kernel's source (its header and the device header),
+    so that edits to other kernels keep the captured counters."""
     h = hashlib.sha256()
     for f in KERNEL_SOURCES:
         with open(os.path.join(ROOT, f), "rb") as fh:
-            text = fh.read()
-        if f.endswith("gcp_kernels.cu") and FUSED_SECTION_END in text:
-            text = text[:text.index(FUSED_SECTION_END)]
-        h.update(text)
+            h.update(fh.read())
     return h.hexdigest()[:16]
 
 

@@ -103,7 +103,7 @@ typedef struct {
     uint64_t seed;        /* Philox key word 0                                             */
     void *stream;         /* cudaStream_t for all work of the context; NULL = default     */
     double hash_max_load; /* nonzero hash set load bound in (0, 0.5]; 0 selects 0.3        */
-    int32_t lane_cols;    /* factor columns per GPU lane: 4 or 8; 0 picks 4 for rank <= 32 */
+    int32_t lane_cols;    /* factor columns per GPU lane: 4 or 8; 0 picks by rank and order  */
     int32_t reserved;
 } gcp_options;
 

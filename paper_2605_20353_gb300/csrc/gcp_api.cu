@@ -175,18 +175,27 @@ gcp_status init_common(gcp_ctx *c, int32_t ndim, const int64_t *dims, int32_t ra
         c->rowoff[k] = c->total_rows;
         c->total_rows += dims[k];
     }
-    // Row length padded to 4 x a power of two.  A lane owns 4 columns when a
-    // row is at most 32 floats (a group's reduction covers the whole
-    // 128-byte row), else 8 (two half rows of >= 128 bytes).
+    // Row length padded to 4 x a power of two, and the columns of it that a
+    // lane owns.  Eight halve the work that each group of lanes repeats
+    // (index arithmetic, loss, shuffles); four let a group's reduction cover
+    // a whole row of up to 128 bytes with one instruction and leave registers
+    // for a fourth block per SM.  A pass without reductions takes eight
+    // wherever there are eight columns, and still fits four blocks (2^19
+    // samples of the 4-way Zipf tensor, rank 32 BF16: kernel 42.8 -> 35.8 us).
+    // A gradient pass takes eight from rank 33 on (2^20 samples of 2 to 8
+    // modes at ranks 33 to 65: 12 to 27% faster), and at a padded rank of 32
+    // where few of the second half's columns are in use (rank 20, 2 to 5
+    // modes: 4 to 18% faster; rank 24 the same, rank 32 slower by 12%) or
+    // there are two modes (12%).
     int Rp = 4;
     while (Rp < rank) Rp <<= 1;
     c->Rp = Rp;
-    c->cols = Rp >= 64 ? 8 : 4;
-    if (c->opt.lane_cols == 4 || (c->opt.lane_cols == 8 && Rp >= 8)) c->cols = c->opt.lane_cols;
+    c->cols = Rp >= 64 || (Rp == 32 && (ndim == 2 || (rank <= 20 && ndim <= 5))) ? 8 : 4;
+    c->eval_cols = Rp >= 8 ? 8 : 4;
+    if (c->opt.lane_cols == 4 || (c->opt.lane_cols == 8 && Rp >= 8)) c->cols = c->eval_cols = c->opt.lane_cols;
     else if (c->opt.lane_cols != 0) return fail(nullptr, GCP_ERR_ARG, "lane_cols must be 0, 4 or 8");
-    int L = Rp / c->cols, log2L = 0;
-    while ((1 << log2L) < L) ++log2L;
-    c->log2L = log2L;
+    while ((c->cols << c->log2L) < Rp) ++c->log2L;
+    while ((c->eval_cols << c->eval_log2L) < Rp) ++c->eval_log2L;
     if ((double)c->total_rows * c->Rp >= 2147483647.0)
         return fail(nullptr, GCP_ERR_ARG, "sum of mode sizes x padded rank must be < 2^31");
 
@@ -298,7 +307,8 @@ gcpk::FusedSpec gcpk_make_spec(const gcp_ctx *c, uint64_t iter, int64_t p, int64
     f.G = grad ? c->G : nullptr;
     f.Rp = c->Rp;
     f.R = c->R;
-    f.log2L = c->log2L;
+    f.log2L = grad ? c->log2L : c->eval_log2L;
+    f.tile = gcpk::fused_tile(p + q, c->log2L, c->max_blocks);
     for (int k = 0; k < c->d; ++k) f.rowoff[k] = (int)c->rowoff[k];
     f.loss = c->loss;
     f.w_nz = (float)w_nz;
@@ -412,12 +422,16 @@ gcp_status run_fused(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, bool grad,
         m.Yval = c->nf_val;
         m.ystride = c->d;
         m.vstride = 1;
-        GCP_CUDA(c, gcpk::launch_fused(m, c->Abf != nullptr, c->cols, c->max_blocks, c->st, &blocks));
+        m.log2L = c->eval_log2L;
+        GCP_CUDA(c, gcpk::launch_fused_eval(m, c->Abf != nullptr, c->eval_cols, c->max_blocks, c->st, &blocks));
         m.G = c->G;  // pass 2: MTTKRP of the stored gradient tensor
+        m.log2L = c->log2L;
         GCP_CUDA(c, gcpk::launch_mttkrp_nonfused(m, f.nrep ? c->hot_slot : nullptr, c->Abf != nullptr, c->cols,
                                                  c->max_blocks, c->st));
-    } else {
+    } else if (grad) {
         GCP_CUDA(c, gcpk::launch_fused(f, c->Abf != nullptr, c->cols, c->max_blocks, c->st, &blocks));
+    } else {
+        GCP_CUDA(c, gcpk::launch_fused_eval(f, c->Abf != nullptr, c->eval_cols, c->max_blocks, c->st, &blocks));
     }
     if (stop) GCP_CUDA(c, cudaEventRecord(stop, c->st));
     bool copy_loss = false;

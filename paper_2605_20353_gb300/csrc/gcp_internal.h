@@ -36,9 +36,9 @@ struct FusedSpec {
     SampleSpec s;
     const void *F;                  // factors the kernels read (FP32 or BF16), row stride Rp
     float *G;                       // gradient, row stride Rp; null = loss only
-    int Rp;                         // padded row length: cols x lanes per sample (power of 2)
+    int Rp;                         // padded row length: columns per lane x lanes per sample (power of 2)
     int R;                          // rank: columns R .. Rp - 1 hold zeros
-    int tile;                       // samples per warp tile, at most 32 (launch_fused)
+    int tile;                       // samples per warp tile, at most 32 (fused_tile)
     int log2L;                      // log2(lanes per sample); each lane owns cols = 4 or 8 columns
     int rowoff[GCP_MAX_NDIM];       // first row of each mode in F and G
     int loss;
@@ -118,8 +118,14 @@ cudaError_t launch_build_records(const int32_t *coords, const float *vals, int64
                                  cudaStream_t st);
 cudaError_t launch_sample(const SampleSpec &s, int32_t *idx_out, float *x_out, float *w_out, float w_nz,
                           float w_z, cudaStream_t st);
+// The fused pass with reductions into f.G, and without (f.log2L to match cols).
+// Both run on the blocks and tiles of the gradient pass, so that their loss
+// partials agree bit for bit.
 cudaError_t launch_fused(const FusedSpec &f, bool bf16, int cols, int max_blocks, cudaStream_t st,
                          int *blocks_used);
+cudaError_t launch_fused_eval(const FusedSpec &f, bool bf16, int cols, int max_blocks, cudaStream_t st,
+                              int *blocks_used);
+int fused_tile(int64_t S, int log2L, int max_blocks);
 cudaError_t launch_grad_finish(const GradOutSpec &p, cudaStream_t st);
 cudaError_t launch_mttkrp_nonfused(const FusedSpec &f, const int *hot_slot, bool bf16, int cols, int max_blocks,
                                    cudaStream_t st);
@@ -140,7 +146,9 @@ struct gcp_ctx {
     uint64_t stride[GCP_MAX_NDIM] = {0};
     int64_t rowoff[GCP_MAX_NDIM] = {0};
     int64_t total_rows = 0;
-    int R = 0, Rp = 0, log2L = 0, cols = 4;
+    int R = 0, Rp = 0;
+    int log2L = 0, cols = 4;            // log2 of the lanes per sample and columns per lane of gradient passes
+    int eval_log2L = 0, eval_cols = 4;  // the same of passes without reductions (loss, gradient tensor)
     int loss = 0;
     int64_t nnz = 0;
     double M = 0;  // number of cells (exact below 2^53, used for weights)

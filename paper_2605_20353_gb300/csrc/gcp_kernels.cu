@@ -1,76 +1,22 @@
-// gcp_kernels.cu -- the fused stochastic GCP gradient on sm_103a.
-//
-// One pass per sample set (the fused Sampling-MTTKRP of Sec. 3.1.2, here with
-// stratified sampling and hash rejection):
-//   phase A, one sample per lane: Philox4x64-10 counters -> nonzero record
-//            load, or zero candidates probed against the nonzero hash set
-//            until one is absent (Sec. 3.1.1);
-//   phase B, one sample per group of L = Rp / (16 B / elt) lanes: each lane
-//            gathers a 16-byte slice of the d factor rows, forms the CP model
-//            entry m (Eq. cp) with a shuffle reduction over the group,
-//            evaluates f and f', and scatters w f' prod_{k!=n} A_k(i_k,:)
-//            into every mode's gradient row with FP32 vector reductions
-//            (Eq. gcp-gradient, atomic MTTKRP of Sec. 3.1.2).
-// The sampled loss is accumulated in FP64 per lane, reduced per block into
-// a partials array and finished by a single-block kernel in fixed order.
+// gcp_kernels.cu -- the kernels around the fused pass (gcp_fused.cuh): the
+// sample writer, the epilogues of a gradient call and of a training step,
+// Adam, nonzero records, and the non-fused MTTKRP.
 #include <cuda_bf16.h>
 
 #include "gcp_device.cuh"
 #include "gcp_epilogue.cuh"
+#include "gcp_fused.cuh"
 #include "gcp_internal.h"
 
 using namespace gcpdev;
 
 namespace gcpk {
 
-constexpr int kThreads = 256;
-
 static int elementwise_blocks(int64_t n);
-static int num_sms();
 
 struct RowOffsets {
     int64_t off[GCP_MAX_NDIM];
 };
-
-template <int D>
-__device__ __forceinline__ void draw_tuple(const SampleSpec &S, uint64_t stream, uint64_t j, uint64_t sub0,
-                                           int32_t (&idx)[D]) {
-#pragma unroll
-    for (int b = 0; 4 * b < D; ++b) {
-        const U64x4 w = philox4x64_10(j, sub0 + (uint64_t)b, S.iter, 0, S.seed, stream);
-#pragma unroll
-        for (int k = 4 * b; k < D && k < 4 * b + 4; ++k)
-            idx[k] = (int32_t)map_range(w.v[k - 4 * b], (uint64_t)S.dims[k]);
-    }
-}
-
-template <int D>
-__device__ __forceinline__ uint64_t linear_of(const SampleSpec &S, const int32_t (&idx)[D]) {
-    uint64_t L = 0;
-#pragma unroll
-    for (int k = 0; k < D; ++k) L += (uint64_t)idx[k] * S.stride[k];
-    return L;
-}
-
-template <int D>
-__device__ __forceinline__ void load_record(const int32_t *__restrict__ rec, uint64_t e, int32_t (&idx)[D],
-                                            float &x) {
-    constexpr int NV = (D + 4) / 4;  // 16-byte vectors holding D coordinates + value
-    constexpr int RW = rec_words_for(D);
-    const int4 *r = reinterpret_cast<const int4 *>(rec + e * RW);
-    int w[4 * NV];
-#pragma unroll
-    for (int v = 0; v < NV; ++v) {
-        const int4 t = __ldg(r + v);
-        w[4 * v] = t.x;
-        w[4 * v + 1] = t.y;
-        w[4 * v + 2] = t.z;
-        w[4 * v + 3] = t.w;
-    }
-#pragma unroll
-    for (int k = 0; k < D; ++k) idx[k] = w[k];
-    x = __int_as_float(w[D]);
-}
 
 // Draw sample s of the set.  Returns false when the sample does not exist
 // (exhausted zero draw); idx then holds the last candidate.
@@ -108,265 +54,6 @@ __device__ __forceinline__ bool draw_sample(const SampleSpec &S, int64_t s, int3
     attempts += S.max_attempts;
     atomicOr(S.status, kErrExhausted);
     return false;
-}
-
-// ------------------------------------------------------------ fused pass
-// Per warp and per tile of P.tile <= 32 consecutive samples (fused_tile):
-//   A1 (tile t+1, one sample per lane): Philox draw; the nonzero record, the
-//      dense value or the first hash bucket of the zero candidate is copied
-//      into shared memory with cp.async while tile t is processed;
-//   A2 (tile t): finish the draw -- a zero candidate found in its bucket is
-//      rejected and redrawn with direct probes (rare: 1/(1-N/M) attempts);
-//   B  (tile t, one sample per group of L = Rp/COLS lanes): lane g owns
-//      COLS columns as COLS/4 quads (4g..4g+3, and Rp/2+4g.. when COLS = 8),
-//      so a group's loads and vector reductions cover whole 32-byte sectors
-//      and, for rows up to 128 bytes, one whole row per instruction.  Quads
-//      beyond the rank hold zeros and are not reduced; they are loaded, as
-//      a test around the loads costs more than the sectors (orders 2 to 8,
-//      ranks 20 to 65, 2^20 samples: 0 to 15% slower with it).
-// Gradient rows that many samples hit go to one of the call's nrep replicas
-// (chosen by warp), folded into G afterwards, so that the reductions of hot
-// rows do not serialise on one address; with nrep = 0 (few samples) every
-// row is added to G itself.
-constexpr int kWarps = kThreads / 32;
-
-template <int D, typename TF, int COLS>
-__global__ void __launch_bounds__(kThreads, fused_min_blocks(D, COLS)) k_fused(const FusedSpec P) {
-    constexpr int SW = rec_words_for(D);  // words per staged sample: coordinates, value, replica slots
-    constexpr int NQ = COLS / 4;          // quads of columns per lane
-    __shared__ __align__(16) int32_t s_slot[2][kWarps][32][SW];
-    __shared__ __align__(16) uint64_t s_bkt[2][kWarps][32][4];
-
-    const int lane = threadIdx.x & 31;
-    const int warp = threadIdx.x >> 5;
-    const int log2L = P.log2L;
-    const int L = 1 << log2L;
-    const int glane = lane & (L - 1);
-    const int grp = lane >> log2L;
-    const int ngrp = 32 >> log2L;
-    const unsigned gmask = (L == 32) ? 0xFFFFFFFFu : (((1u << L) - 1u) << (grp * L));
-    int col[NQ];
-    bool on[NQ];  // the quad holds columns of the rank, not padding alone
-#pragma unroll
-    for (int q = 0; q < NQ; ++q) {
-        col[q] = q * (P.Rp >> 1) + 4 * glane;
-        on[q] = col[q] < P.R;
-    }
-    const int p = (int)P.s.p;  // sample counts of one call are below 2^31
-    const int S = (int)(P.s.p + P.s.q);
-    const unsigned TS = P.tile;
-    const int ntiles = (int)(((int64_t)S + TS - 1) / TS);  // S may be 2^31 - 1
-    const int nwarps = (gridDim.x * blockDim.x) >> 5;
-    const int warp0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const TF *__restrict__ F = static_cast<const TF *>(P.F);
-    const float scale = P.dscale ? __ldg(P.dscale) : 1.0f;
-    const bool semi = P.s.sampling == GCP_SAMPLING_SEMI_STRATIFIED;
-    const bool uniform = P.s.sampling == GCP_SAMPLING_UNIFORM;
-    float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (P.nrep - 1)) * P.Htot * P.Rp : nullptr;
-
-    double acc_nz = 0.0, acc_z = 0.0;
-    int attempts = 0;
-
-    // A1: start the draw of this lane's sample of `tile` into stage `st`;
-    // returns the key of a stratified zero candidate (kEmpty otherwise).
-    auto issue = [&](int tile, int st) -> uint64_t {
-        if (tile >= ntiles || lane >= (int)TS) return kEmpty;
-        const unsigned us = (unsigned)tile * TS + lane;  // may pass 2^31 - 1 in the last tile
-        int32_t *slot = s_slot[st][warp][lane];
-        if (us >= (unsigned)S) return kEmpty;
-        const int s = (int)us;
-        if (uniform) {
-            int32_t idx[D];
-            draw_tuple<D>(P.s, kStreamUniform, (uint64_t)s, 0, idx);
-#pragma unroll
-            for (int k = 0; k < D; ++k) slot[k] = idx[k];
-            cp_async4(slot + D, P.s.dense + linear_of<D>(P.s, idx));
-            return kEmpty;
-        }
-        if (s < p) {
-            const U64x4 w = philox4x64_10((uint64_t)s, 0, P.s.iter, 0, P.s.seed, kStreamNonzero);
-            const int32_t *rec = P.s.rec + map_range(w.v[0], (uint64_t)P.s.nnz) * SW;
-#pragma unroll
-            for (int v = 0; v < SW / 4; ++v) cp_async16(slot + 4 * v, rec + 4 * v);
-            return kEmpty;
-        }
-        int32_t idx[D];
-        draw_tuple<D>(P.s, semi ? kStreamSemiZero : kStreamZero, (uint64_t)(s - p), 0, idx);
-#pragma unroll
-        for (int k = 0; k < D; ++k) slot[k] = idx[k];
-        slot[D] = 0;  // x = 0.0f
-        if (semi) return kEmpty;
-        const uint64_t key = linear_of<D>(P.s, idx);
-        const uint64_t *b = P.s.hkeys + 4 * (mix64(key) & P.s.hbmask);
-        cp_async16(&s_bkt[st][warp][lane][0], b);
-        cp_async16(&s_bkt[st][warp][lane][2], b + 2);
-        return key;
-    };
-
-    // A2: finish the draw of stage `st`; returns whether the sample exists.
-    auto finish = [&](int tile, int st, uint64_t key) -> bool {
-        const unsigned us = (unsigned)tile * TS + lane;
-        if (lane >= (int)TS || us >= (unsigned)S) return false;
-        const int s = (int)us;
-        if (key == kEmpty) return true;  // nonzero, semi-stratified or dense draw
-        const ulonglong2 lo = *reinterpret_cast<const ulonglong2 *>(&s_bkt[st][warp][lane][0]);
-        const ulonglong2 hi = *reinterpret_cast<const ulonglong2 *>(&s_bkt[st][warp][lane][2]);
-        int h = bucket_decide(lo, hi, key);
-        if (h == 2)
-            h = hash_contains_from(P.s.hkeys, P.s.hbmask, key, ((mix64(key) & P.s.hbmask) + 1) & P.s.hbmask, 1);
-        if (h == 0) {
-            attempts += 1;
-            return true;
-        }
-        // rejected: redraw until a candidate is absent (Sec. 3.1.1)
-        int32_t *slot = s_slot[st][warp][lane];
-        const uint64_t j = (uint64_t)(s - p);
-        for (int a = 1; h == 1 && a < P.s.max_attempts; ++a) {
-            int32_t idx[D];
-            draw_tuple<D>(P.s, kStreamZero, j, 4 * (uint64_t)a, idx);
-            h = hash_contains(P.s.hkeys, P.s.hbmask, linear_of<D>(P.s, idx));
-            if (h == 0) {
-#pragma unroll
-                for (int k = 0; k < D; ++k) slot[k] = idx[k];
-                attempts += a + 1;
-                return true;
-            }
-        }
-        if (h < 0) {
-            atomicOr(P.s.status, kErrHashFull);
-        } else {
-            attempts += P.s.max_attempts;
-            atomicOr(P.s.status, kErrExhausted);
-        }
-        return false;
-    };
-
-    int tile = warp0;
-    uint64_t key_next = issue(tile, 0);
-    cp_async_commit();
-    for (int st = 0; tile < ntiles; tile += nwarps, st ^= 1) {
-        const uint64_t key = key_next;
-        __syncwarp();  // stage st^1 is free: the previous tile's phase B is done
-        key_next = issue(tile + nwarps, st ^ 1);
-        cp_async_commit();
-        cp_async_wait<1>();  // this lane's copies into stage st have landed
-        const bool ok = finish(tile, st, key);
-        const unsigned okmask = __ballot_sync(0xFFFFFFFFu, ok);
-        __syncwarp();  // every lane's staged sample is visible to the warp
-
-        // phase B: one sample per group; the group leader keeps FP32 loss
-        // sums of the tile, added to the FP64 totals once per tile
-        float tf_nz = 0.0f, tf_z = 0.0f;
-        for (int it = 0; it * ngrp < (int)TS; ++it) {
-            const int src = it * ngrp + grp;
-            if (!((okmask >> src) & 1u)) {  // uniform within the group
-                const unsigned sm = (unsigned)tile * TS + src;
-                if (P.Yval && glane == 0 && src < (int)TS && sm < (unsigned)S) {  // no sample: a zero entry at a valid cell
-#pragma unroll
-                    for (int k = 0; k < D; ++k) P.Ycoord[(int64_t)sm * P.ystride + k] = s_slot[st][warp][src][k];
-                    P.Yval[(int64_t)sm * P.vstride] = 0.0f;
-                }
-                continue;
-            }
-            const int32_t *slot = s_slot[st][warp][src];
-            int32_t ii[D];
-#pragma unroll
-            for (int k = 0; k < D; ++k) ii[k] = slot[k];
-            const float xs = __int_as_float(slot[D]);
-            const bool is_nz = !uniform && ((unsigned)tile * TS + src) < (unsigned)p;
-
-            int off[D];
-            float a[D][COLS];
-#pragma unroll
-            for (int k = 0; k < D; ++k) {
-                off[k] = (P.rowoff[k] + ii[k]) * P.Rp;
-#pragma unroll
-                for (int q = 0; q < NQ; ++q) Quad<TF>::load(F + off[k] + col[q], a[k] + 4 * q);
-            }
-            float suf[D][COLS];  // suf[k] = prod_{j>k} a_j
-#pragma unroll
-            for (int v = 0; v < COLS; ++v) suf[D - 1][v] = 1.0f;
-#pragma unroll
-            for (int k = D - 2; k >= 0; --k)
-#pragma unroll
-                for (int v = 0; v < COLS; ++v) suf[k][v] = suf[k + 1][v] * a[k + 1][v];
-            float m = 0.0f;
-#pragma unroll
-            for (int v = 0; v < COLS; ++v) m = fmaf(a[0][v], suf[0][v], m);
-            for (int o = L >> 1; o > 0; o >>= 1) m += __shfl_xor_sync(gmask, m, o);
-
-            float f, df;
-            loss_eval(P.loss, xs, m, f, df);
-            if (semi && is_nz) {
-                float f0, df0;
-                loss_eval(P.loss, 0.0f, m, f0, df0);
-                f -= f0;
-                df -= df0;
-            }
-            if (is_nz || uniform)
-                tf_nz += f;
-            else
-                tf_z += f;
-            if (P.Yval) {  // materialize the gradient tensor entry (non-fused MTTKRP input)
-                if (glane == 0) {
-                    const int sm = tile * TS + src;
-#pragma unroll
-                    for (int k = 0; k < D; ++k) P.Ycoord[(int64_t)sm * P.ystride + k] = ii[k];
-                    P.Yval[(int64_t)sm * P.vstride] = ((is_nz || uniform) ? P.w_nz : P.w_z) * df * scale;
-                }
-            } else if (P.G) {
-                const float y = ((is_nz || uniform) ? P.w_nz : P.w_z) * df * scale;
-                float pre[COLS];
-#pragma unroll
-                for (int v = 0; v < COLS; ++v) pre[v] = y;
-#pragma unroll
-                for (int n = 0; n < D; ++n) {
-                    // replica slot: stored in a nonzero's record; for drawn
-                    // cells, rows of fully replicated modes only
-                    unsigned hs;
-                    if (is_nz && grep)
-                        hs = ((unsigned)slot[D + 1 + n / 2] >> (16 * (n & 1))) & 0xFFFFu;
-                    else
-                        hs = P.small_base[n] >= 0 ? (unsigned)(P.small_base[n] + ii[n]) : kNoSlot;
-                    float *g = hs != kNoSlot ? grep + (int)hs * P.Rp : P.G + off[n];
-#pragma unroll
-                    for (int q = 0; q < NQ; ++q)
-                        if (on[q])
-                            red_add_v4(g + col[q], pre[4 * q] * suf[n][4 * q], pre[4 * q + 1] * suf[n][4 * q + 1],
-                                   pre[4 * q + 2] * suf[n][4 * q + 2], pre[4 * q + 3] * suf[n][4 * q + 3]);
-#pragma unroll
-                    for (int v = 0; v < COLS; ++v) pre[v] *= a[n][v];
-                }
-            }
-        }
-        if (glane == 0) {
-            acc_nz += (double)tf_nz;
-            acc_z += (double)tf_z;
-        }
-    }
-    cp_async_wait<0>();
-
-    // block reduction of the FP64 loss sums (held by the group leaders) and
-    // attempt counts; FP64 adds are slow here (16 cycles of the SM's pipe for
-    // a warp), so only the leaders' steps are taken
-    attempts = __reduce_add_sync(0xFFFFFFFFu, attempts);
-    for (int o = 16; o >= L; o >>= 1) {
-        acc_nz += __shfl_xor_sync(0xFFFFFFFFu, acc_nz, o);
-        acc_z += __shfl_xor_sync(0xFFFFFFFFu, acc_z, o);
-    }
-    double(*red)[kWarps] = reinterpret_cast<double(*)[kWarps]>(&s_bkt[0][0][0][0]);  // staging is free now
-    __syncthreads();
-    if (lane == 0) {
-        red[0][warp] = acc_nz;
-        red[1][warp] = acc_z;
-        red[2][warp] = (double)attempts;
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        double t = 0.0;
-        for (int w = 0; w < kWarps; ++w) t += red[threadIdx.x][w];
-        P.partials[4 * blockIdx.x + threadIdx.x] = t;
-    }
 }
 
 // ------------------------------------------------- loss, fold, gradient out
@@ -700,16 +387,6 @@ __global__ void k_to_bf16(int64_t n, const float *__restrict__ A, __nv_bfloat16 
 }
 
 // --------------------------------------------------------------- launches
-static int num_sms() {
-    static int sms = 0;
-    if (!sms) {
-        int dev = 0;
-        cudaGetDevice(&dev);
-        cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-    }
-    return sms;
-}
-
 static int elementwise_blocks(int64_t n) {
     const int64_t want = (n + kThreads - 1) / kThreads;
     const int64_t cap = (int64_t)num_sms() * 8;
@@ -752,88 +429,6 @@ cudaError_t launch_sample(const SampleSpec &s, int32_t *idx_out, float *x_out, f
 #define GCP_LAUNCH_SAMPLE(D) k_sample<D><<<blocks, kThreads, 0, st>>>(s, idx_out, x_out, w_out, w_nz, w_z)
     GCP_DISPATCH_D(s.d, GCP_LAUNCH_SAMPLE)
 #undef GCP_LAUNCH_SAMPLE
-    return cudaGetLastError();
-}
-
-template <int D, typename TF, int COLS>
-static int occupancy_blocks() {
-    static int nb = -1;
-    if (nb < 0) {
-        int per_sm = 0;
-        cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k_fused<D, TF, COLS>, kThreads, 0);
-        nb = (per_sm < 1 ? 1 : per_sm) * num_sms();
-    }
-    return nb;
-}
-
-template <int D>
-static int occupancy_of(bool bf16, int cols) {
-    if (bf16) return cols == 8 ? occupancy_blocks<D, __nv_bfloat16, 8>() : occupancy_blocks<D, __nv_bfloat16, 4>();
-    return cols == 8 ? occupancy_blocks<D, float, 8>() : occupancy_blocks<D, float, 4>();
-}
-
-int fused_max_blocks(int d, bool bf16, int cols) {
-    switch (d) {
-    case 2: return occupancy_of<2>(bf16, cols);
-    case 3: return occupancy_of<3>(bf16, cols);
-    case 4: return occupancy_of<4>(bf16, cols);
-    case 5: return occupancy_of<5>(bf16, cols);
-    case 6: return occupancy_of<6>(bf16, cols);
-    case 7: return occupancy_of<7>(bf16, cols);
-    case 8: return occupancy_of<8>(bf16, cols);
-    default: return num_sms();
-    }
-}
-
-template <int D>
-static void launch_fused_d(const FusedSpec &f, bool bf16, int cols, int blocks, cudaStream_t st) {
-    if (bf16) {
-        if (cols == 8)
-            k_fused<D, __nv_bfloat16, 8><<<blocks, kThreads, 0, st>>>(f);
-        else
-            k_fused<D, __nv_bfloat16, 4><<<blocks, kThreads, 0, st>>>(f);
-    } else {
-        if (cols == 8)
-            k_fused<D, float, 8><<<blocks, kThreads, 0, st>>>(f);
-        else
-            k_fused<D, float, 4><<<blocks, kThreads, 0, st>>>(f);
-    }
-}
-
-// Samples per warp tile: with r = ceil(S / (32 W)) rounds of tiles over the W
-// resident warps, the smallest tile that still takes r rounds (a multiple of
-// the samples that the warp's groups evaluate at once), so that every warp
-// has the same work: 250,000 samples on 4,864 warps are two rounds of 28
-// instead of one of 32 and 0.6 of another, and small sets spread over all
-// warps.
-static int fused_tile(int64_t S, int log2L, int64_t warps) {
-    const int ngrp = 32 >> log2L;
-    const int64_t rounds = (S + 32 * warps - 1) / (32 * warps);
-    if (rounds < 1) return 32;
-    const int64_t per = (S + warps * rounds - 1) / (warps * rounds);
-    return (int)((per + ngrp - 1) / ngrp * ngrp);
-}
-
-cudaError_t launch_fused(const FusedSpec &spec, bool bf16, int cols, int max_blocks, cudaStream_t st,
-                         int *blocks_used) {
-    FusedSpec f = spec;
-    const int64_t S = f.s.p + f.s.q;
-    f.tile = fused_tile(S, f.log2L, (int64_t)max_blocks * kWarps);
-    const int64_t ntiles = (S + f.tile - 1) / f.tile;
-    int64_t want = (ntiles + kWarps - 1) / kWarps;
-    if (want < 1) want = 1;
-    const int blocks = (int)(want < max_blocks ? want : max_blocks);
-    *blocks_used = blocks;
-    switch (f.s.d) {
-    case 2: launch_fused_d<2>(f, bf16, cols, blocks, st); break;
-    case 3: launch_fused_d<3>(f, bf16, cols, blocks, st); break;
-    case 4: launch_fused_d<4>(f, bf16, cols, blocks, st); break;
-    case 5: launch_fused_d<5>(f, bf16, cols, blocks, st); break;
-    case 6: launch_fused_d<6>(f, bf16, cols, blocks, st); break;
-    case 7: launch_fused_d<7>(f, bf16, cols, blocks, st); break;
-    case 8: launch_fused_d<8>(f, bf16, cols, blocks, st); break;
-    default: return cudaErrorInvalidValue;
-    }
     return cudaGetLastError();
 }
 

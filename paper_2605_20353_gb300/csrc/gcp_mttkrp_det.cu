@@ -735,7 +735,8 @@ gcp_status gcpk_det_grad(gcp_ctx *c, const gcpk::FusedSpec &f0, int *blocks) {
     f.Yval = reinterpret_cast<float *>(recs + c->d);
     f.ystride = rw;
     f.vstride = rw;
-    DET_CUDA(gcpk::launch_fused(f, c->Abf != nullptr, c->cols, c->max_blocks, st, blocks));
+    f.log2L = c->eval_log2L;
+    DET_CUDA(gcpk::launch_fused_eval(f, c->Abf != nullptr, c->eval_cols, c->max_blocks, st, blocks));
     if (S == 0) return GCP_OK;
 
     // 2a. the first pass of every mode: counted and scanned once

@@ -28,7 +28,7 @@ __device__ __forceinline__ void draw_tuple_b(const gcpk::SampleSpec &S, uint64_t
         const U64x4 w = philox4x64_10(j, sub0 + (uint64_t)b, S.iter, 0, S.seed, stream);
 #pragma unroll
         for (int k = 4 * b; k < D && k < 4 * b + 4; ++k)
-            idx[k] = (int32_t)map_range(w.v[k - 4 * b], (uint64_t)S.dims[k]);
+            idx[k] = (int32_t)map_range32(w.v[k - 4 * b], (uint32_t)S.dims[k]);
     }
 }
 

@@ -54,6 +54,12 @@ __device__ __forceinline__ U64x4 philox4x64_10(uint64_t c0, uint64_t c1, uint64_
 // floor(u * n / 2^64): exact map of a 64-bit word onto [0, n).
 __device__ __forceinline__ uint64_t map_range(uint64_t u, uint64_t n) { return __umul64hi(u, n); }
 
+// The same for n below 2^32 (a mode size): two 32-bit products instead of four.
+__device__ __forceinline__ uint32_t map_range32(uint64_t u, uint32_t n) {
+    const uint64_t lo = (uint64_t)(uint32_t)u * n;
+    return (uint32_t)(((u >> 32) * n + (lo >> 32)) >> 32);
+}
+
 // --------------------------------------------------------------- hash set
 // Open addressing over buckets of four uint64 keys (one 32-byte sector),
 // linear probing bucket by bucket; slots of a bucket fill in order and are
@@ -190,6 +196,29 @@ template <int N>
 __device__ __forceinline__ void cp_async_wait() {
     asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory");
 }
+
+// Four entries through the coherent path, for factors that an earlier grid may
+// still be writing when this kernel starts (programmatic dependent launch).
+__device__ __forceinline__ void load_quad_coherent(const float *p, float *o) {
+    const float4 v = *reinterpret_cast<const float4 *>(p);
+    o[0] = v.x;
+    o[1] = v.y;
+    o[2] = v.z;
+    o[3] = v.w;
+}
+__device__ __forceinline__ void load_quad_coherent(const __nv_bfloat16 *p, float *o) {
+    const uint2 v = *reinterpret_cast<const uint2 *>(p);
+    o[0] = __uint_as_float(v.x << 16);
+    o[1] = __uint_as_float(v.x & 0xFFFF0000u);
+    o[2] = __uint_as_float(v.y << 16);
+    o[3] = __uint_as_float(v.y & 0xFFFF0000u);
+}
+
+// Programmatic dependent launch: wait until the grids this one depends on
+// have finished and their writes are visible (returns at once in a grid
+// launched without the attribute), and let dependent grids be scheduled.
+__device__ __forceinline__ void grid_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void grid_trigger() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Fire-and-forget FP32 vector reduction into global memory (sm_90+).
 __device__ __forceinline__ void red_add_v4(float *p, float a, float b, float c, float d) {

@@ -47,7 +47,7 @@ __device__ __forceinline__ void draw_tuple(const SampleSpec &S, uint64_t stream,
         const U64x4 w = philox4x64_10(j, sub0 + (uint64_t)b, S.iter, 0, S.seed, stream);
 #pragma unroll
         for (int k = 4 * b; k < D && k < 4 * b + 4; ++k)
-            idx[k] = (int32_t)map_range(w.v[k - 4 * b], (uint64_t)S.dims[k]);
+            idx[k] = (int32_t)map_range32(w.v[k - 4 * b], (uint32_t)S.dims[k]);
     }
 }
 
@@ -145,8 +145,7 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
     const int ntiles = (int)(((int64_t)S + TS - 1) / TS);  // S may be 2^31 - 1
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     const int warp0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const TF *__restrict__ F = static_cast<const TF *>(P.F);
-    const float scale = P.dscale ? __ldg(P.dscale) : 1.0f;
+    const TF *F = static_cast<const TF *>(P.F);
     const bool semi = P.s.sampling == GCP_SAMPLING_SEMI_STRATIFIED;
     const bool uniform = P.s.sampling == GCP_SAMPLING_UNIFORM;
     [[maybe_unused]] float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (P.nrep - 1)) * P.Htot * P.Rp : nullptr;
@@ -231,6 +230,12 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
     int tile = warp0;
     uint64_t key_next = issue(tile, 0);
     cp_async_commit();
+    // the draws need only what never changes; everything else (factors, G,
+    // replicas, the incoming scale, the partials) waits for the grids before.
+    // Dependents are let in only then, so that theirs wait for ours alone.
+    grid_wait();
+    grid_trigger();
+    const float scale = P.dscale ? *P.dscale : 1.0f;
     for (int st = 0; tile < ntiles; tile += nwarps, st ^= 1) {
         const uint64_t key = key_next;
         __syncwarp();  // stage st^1 is free: the previous tile's phase B is done
@@ -266,7 +271,7 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
             for (int k = 0; k < D; ++k) {
                 off[k] = (P.rowoff[k] + ii[k]) * P.Rp;
 #pragma unroll
-                for (int q = 0; q < NQ; ++q) Quad<TF>::load(F + off[k] + col[q], a[k] + 4 * q);
+                for (int q = 0; q < NQ; ++q) load_quad_coherent(F + off[k] + col[q], a[k] + 4 * q);
             }
             float suf[D][COLS];  // suf[k] = prod_{j>k} a_j
 #pragma unroll
@@ -376,19 +381,20 @@ int fused_occupancy_d(bool bf16, int cols) {
     return cols == 8 ? fused_occupancy<D, float, 8, EVAL>() : fused_occupancy<D, float, 4, EVAL>();
 }
 
+template <int D, typename TF, int COLS, bool EVAL>
+cudaError_t launch_fused_k(const FusedSpec &f, int blocks, cudaStream_t st) {
+    if (f.dependent) return launch_dependent(k_fused<D, TF, COLS, EVAL>, blocks, kThreads, st, f);
+    k_fused<D, TF, COLS, EVAL><<<blocks, kThreads, 0, st>>>(f);
+    return cudaGetLastError();
+}
+
 template <int D, bool EVAL>
-void launch_fused_d(const FusedSpec &f, bool bf16, int cols, int blocks, cudaStream_t st) {
-    if (bf16) {
-        if (cols == 8)
-            k_fused<D, __nv_bfloat16, 8, EVAL><<<blocks, kThreads, 0, st>>>(f);
-        else
-            k_fused<D, __nv_bfloat16, 4, EVAL><<<blocks, kThreads, 0, st>>>(f);
-    } else {
-        if (cols == 8)
-            k_fused<D, float, 8, EVAL><<<blocks, kThreads, 0, st>>>(f);
-        else
-            k_fused<D, float, 4, EVAL><<<blocks, kThreads, 0, st>>>(f);
-    }
+cudaError_t launch_fused_d(const FusedSpec &f, bool bf16, int cols, int blocks, cudaStream_t st) {
+    if (bf16)
+        return cols == 8 ? launch_fused_k<D, __nv_bfloat16, 8, EVAL>(f, blocks, st)
+                         : launch_fused_k<D, __nv_bfloat16, 4, EVAL>(f, blocks, st);
+    return cols == 8 ? launch_fused_k<D, float, 8, EVAL>(f, blocks, st)
+                     : launch_fused_k<D, float, 4, EVAL>(f, blocks, st);
 }
 
 template <bool EVAL>
@@ -401,16 +407,15 @@ cudaError_t launch_fused_any(const FusedSpec &f, bool bf16, int cols, int max_bl
     const int blocks = (int)(want < max_blocks ? want : max_blocks);
     *blocks_used = blocks;
     switch (f.s.d) {
-    case 2: launch_fused_d<2, EVAL>(f, bf16, cols, blocks, st); break;
-    case 3: launch_fused_d<3, EVAL>(f, bf16, cols, blocks, st); break;
-    case 4: launch_fused_d<4, EVAL>(f, bf16, cols, blocks, st); break;
-    case 5: launch_fused_d<5, EVAL>(f, bf16, cols, blocks, st); break;
-    case 6: launch_fused_d<6, EVAL>(f, bf16, cols, blocks, st); break;
-    case 7: launch_fused_d<7, EVAL>(f, bf16, cols, blocks, st); break;
-    case 8: launch_fused_d<8, EVAL>(f, bf16, cols, blocks, st); break;
+    case 2: return launch_fused_d<2, EVAL>(f, bf16, cols, blocks, st);
+    case 3: return launch_fused_d<3, EVAL>(f, bf16, cols, blocks, st);
+    case 4: return launch_fused_d<4, EVAL>(f, bf16, cols, blocks, st);
+    case 5: return launch_fused_d<5, EVAL>(f, bf16, cols, blocks, st);
+    case 6: return launch_fused_d<6, EVAL>(f, bf16, cols, blocks, st);
+    case 7: return launch_fused_d<7, EVAL>(f, bf16, cols, blocks, st);
+    case 8: return launch_fused_d<8, EVAL>(f, bf16, cols, blocks, st);
     default: return cudaErrorInvalidValue;
     }
-    return cudaGetLastError();
 }
 
 }  // namespace gcpk

@@ -38,6 +38,7 @@ struct FusedSpec {
     float *G;                       // gradient, row stride Rp; null = loss only
     int Rp;                         // padded row length: columns per lane x lanes per sample (power of 2)
     int R;                          // rank: columns R .. Rp - 1 hold zeros
+    bool dependent;                 // launched beside the end of the grid before (launch_dependent)
     int tile;                       // samples per warp tile, at most 32 (fused_tile)
     int log2L;                      // log2(lanes per sample); each lane owns cols = 4 or 8 columns
     int rowoff[GCP_MAX_NDIM];       // first row of each mode in F and G
@@ -110,6 +111,23 @@ __host__ __device__ constexpr int fused_min_blocks(int d, int cols) {
     return d <= 4 ? (cols == 4 ? 4 : 3) : (cols == 4 && d <= 7 ? 3 : 2);
 }
 
+// A launch that may start while the grid before it on the stream still runs
+// (programmatic dependent launch); the kernel calls gcpdev::grid_wait before
+// it touches what that grid writes.
+template <typename... Params, typename... Args>
+cudaError_t launch_dependent(void (*k)(Params...), int blocks, int threads, cudaStream_t st, Args... args) {
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchConfig_t cfg{};
+    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.stream = st;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+    return cudaLaunchKernelEx(&cfg, k, args...);
+}
+
 // ---------------------------------------------------------------- kernels
 // All launches are asynchronous on `st`; device errors go to the status word.
 cudaError_t launch_build_records(const int32_t *coords, const float *vals, int64_t nnz, int d,
@@ -130,6 +148,7 @@ cudaError_t launch_grad_finish(const GradOutSpec &p, cudaStream_t st);
 cudaError_t launch_mttkrp_nonfused(const FusedSpec &f, const int *hot_slot, bool bf16, int cols, int max_blocks,
                                    cudaStream_t st);
 cudaError_t launch_finish_loss(const LossSpec &l, cudaStream_t st);
+cudaError_t launch_clear(float *x, int64_t n, cudaStream_t st);  // n a multiple of 4, x 16-byte aligned
 cudaError_t launch_adam(int64_t n, int Rp, int R, float *A, float *B, float *C, const float *G, float lr,
                         float beta1, float beta2, float c1inv, float c2inv, float eps, float lower,
                         void *Abf, cudaStream_t st);

@@ -88,7 +88,11 @@ __device__ __forceinline__ void finish_loss_block(const LossSpec &l) {
     }
 }
 
-__global__ void __launch_bounds__(kThreads) k_finish_loss(const LossSpec l) { finish_loss_block(l); }
+__global__ void __launch_bounds__(kThreads) k_finish_loss(const LossSpec l) {
+    grid_wait();
+    grid_trigger();
+    finish_loss_block(l);
+}
 
 // The epilogue of a gradient call after the fused pass, in one launch:
 //  - the last block finishes the FP64 loss (and hands it to the caller's
@@ -109,6 +113,8 @@ __global__ void __launch_bounds__(kThreads) k_finish_loss(const LossSpec l) { fi
 // samples 52.2 -> 41.0 us.
 template <int NREP, int V>
 __global__ void __launch_bounds__(kThreads) k_grad_finish(const GradOutSpec P, int ncold) {
+    grid_wait();
+    grid_trigger();
     if (blockIdx.x == gridDim.x - 1) {
         finish_loss_block(P.loss);
         return;
@@ -273,6 +279,8 @@ constexpr int kPostUnroll = 1;
 
 template <int NREP>
 __global__ void __launch_bounds__(kThreads) k_post_step(PostSpec P, int ncold) {
+    grid_wait();
+    grid_trigger();  // the next step's pass may draw its samples beside this grid
     if (blockIdx.x == gridDim.x - 1) {  // the last block only finishes the loss
         finish_loss_block(P.loss);
         return;
@@ -367,8 +375,8 @@ static cudaError_t launch_post_step_r(const PostSpec &p, cudaStream_t st) {
         constexpr int per = kThreads / gcpe::hot_lanes<NREP>();  // hot quads of a block
         nhot = (int)(((int64_t)p.Htot * (p.Rp >> 2) + per - 1) / per);
     }
-    k_post_step<NREP><<<ncold + nhot + 1, kThreads, 0, st>>>(p, ncold);  // + the loss block
-    return cudaGetLastError();
+    const int blocks = ncold + nhot + 1;  // + the loss block
+    return launch_dependent(k_post_step<NREP>, blocks, kThreads, st, p, ncold);
 }
 
 cudaError_t launch_post_step(const PostSpec &p, cudaStream_t st) {
@@ -535,8 +543,8 @@ static cudaError_t launch_grad_finish_rv(const GradOutSpec &p, cudaStream_t st) 
         constexpr int per = kThreads / gcpe::hot_lanes<NREP>();  // hot quads of a block
         nhot = (int)(((int64_t)p.Htot * (p.Rp >> 2) + per - 1) / per);
     }
-    k_grad_finish<NREP, V><<<ncold + nhot + 1, kThreads, 0, st>>>(p, ncold);  // + the loss block
-    return cudaGetLastError();
+    const int blocks = ncold + nhot + 1;  // + the loss block
+    return launch_dependent(k_grad_finish<NREP, V>, blocks, kThreads, st, p, ncold);
 }
 
 template <int NREP>
@@ -556,8 +564,20 @@ cudaError_t launch_grad_finish(const GradOutSpec &p, cudaStream_t st) {
 }
 
 cudaError_t launch_finish_loss(const LossSpec &l, cudaStream_t st) {
-    k_finish_loss<<<1, kThreads, 0, st>>>(l);
-    return cudaGetLastError();
+    return launch_dependent(k_finish_loss, 1, kThreads, st, l);
+}
+
+// x = 0 before a gradient pass, as a kernel and not a memset so that the pass
+// may start beside it.
+__global__ void __launch_bounds__(kThreads) k_clear(float4 *x, int64_t nq) {
+    grid_wait();
+    grid_trigger();
+    for (int64_t q = (int64_t)blockIdx.x * kThreads + threadIdx.x; q < nq; q += (int64_t)gridDim.x * kThreads)
+        x[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+}
+
+cudaError_t launch_clear(float *x, int64_t n, cudaStream_t st) {
+    return launch_dependent(k_clear, elementwise_blocks(n >> 2), kThreads, st, reinterpret_cast<float4 *>(x), n >> 2);
 }
 
 cudaError_t launch_adam(int64_t n, int Rp, int R, float *A, float *B, float *C, const float *G, float lr,

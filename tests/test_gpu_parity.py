@@ -906,3 +906,65 @@ def test_loss_bits_do_not_depend_on_the_pass(env, dims, R, loss, dtype):
             L.setdefault((p, q), set()).update({ctx.loss_value(1, p, q), ctx.grad(1, p, q)[0]})
         ctx.close()
     assert all(len(v) == 1 for v in L.values()), L
+
+
+@pytest.mark.parametrize("p,q", [(40, 33), (3000, 2800), (300000, 300000)])
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+def test_back_to_back_calls_wait_for_one_another(env, p, q, dtype):
+    """The kernels of consecutive calls overlap at their edges (a pass draws
+    its first samples while the epilogue before it runs; small and large
+    sample counts are launched differently).  A long run of steps, gradients
+    and losses issued without a wait, in that order and captured in a CUDA
+    graph, must leave what the same calls leave with a wait after each one:
+    factors within 1e-5 (the atomics' order is free), losses within 1e-5."""
+    gcp, torch = env
+    dims, R = [61, 47, 900], 10
+    coords, vals, factors = problem(dims, 6000, R, "poisson", 911)
+    prm = gcp.AdamParams(lr=1e-2, beta1=0.9, beta2=0.99, eps=1e-8, lower=0.05)
+    stream = torch.cuda.Stream()
+
+    def make():
+        with torch.cuda.stream(stream):
+            ctx = gcp.gcp_create(dims, coords, vals, R, "poisson", seed=912, dtype=dtype)
+            ctx.set_factors(factors)
+        return ctx
+
+    def calls(ctx, loss, G, wait):
+        lib = gcp.load()
+        for t in range(12):
+            ctx.step(t, p, q, prm, t + 1, dloss=loss[3 * t:])
+            if wait:
+                torch.cuda.synchronize()
+            ctx.loss_async(t, p, q, loss[3 * t + 1:])
+            if wait:
+                torch.cuda.synchronize()
+            ctx.grad_async(t, p, q, G_out=G, dloss=loss[3 * t + 2:])
+            if wait:
+                torch.cuda.synchronize()
+
+    out = {}
+    for how in ("wait", "run", "graph"):
+        ctx = make()
+        loss = torch.zeros(36, dtype=torch.float64, device="cuda")
+        G = torch.zeros(ctx.num_params, device="cuda")
+        if how == "graph":
+            with torch.cuda.stream(stream):
+                ctx.step(0, p, q, prm, 1)  # first calls outside the capture; undone below
+                ctx.grad_async(0, p, q, G_out=G)
+            torch.cuda.synchronize()
+            ctx.set_factors(factors)
+            ctx.reset_adam()
+            graph = torch.cuda.CUDAGraph()
+            with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+                calls(ctx, loss, G, False)
+            torch.cuda.synchronize()
+            graph.replay()
+        else:
+            torch.cuda.synchronize()
+            calls(ctx, loss, G, how == "wait")
+        torch.cuda.synchronize()
+        out[how] = (np.concatenate([a.ravel() for a in ctx.get_factors()]), loss.cpu().numpy(), G.cpu().numpy())
+        ctx.close()
+    for how in ("run", "graph"):
+        for a, b in zip(out[how], out["wait"]):
+            assert rel_err(a, b) <= 1e-5, (how, rel_err(a, b))

@@ -276,7 +276,9 @@ gcp_status check_counts(gcp_ctx *c, int64_t p, int64_t q) {
 // replicas are taken until the chain is under 6% of the pass's row traffic
 // (2 x 4 B x D Rp per sample at about 9 TB/s) or under 4 us, less than the
 // latency of the shortest pass, rounded up to a count the folds are built
-// for.  Measured per call with 0 / 4 / 16 / 64 replicas: benchmark step 900 /
+// for; and until no row sums more than about 256 terms one after another in
+// FP32 (25,777 samples on six modes of 33 to 91 rows, 781 terms a row: 6.7e-7
+// from the FP64 gradient without replicas, 1.2e-7 with 64).  Measured per call with 0 / 4 / 16 / 64 replicas: benchmark step 900 /
 // 487 / 278 / 247 us (rule: 64); dense 5-way gradient, 2^22 samples 1916 /
 // 852 / 421 / 367 us (64); 172 x 25,000 x 300, rank 50, 2^16 samples 48.5 /
 // 52.3 / 52.3 / 54.3 us (0); 211 x 187 x 95 x 24, rank 10, 10^4 samples 18.7 /
@@ -287,8 +289,10 @@ int replicas_for(const gcp_ctx *c, int64_t p, int64_t q) {
     const double cell = std::min(1.0, c->share_cell * line);
     const bool uniform = c->opt.sampling == GCP_SAMPLING_UNIFORM;
     const double hits = uniform ? (double)p * cell : (double)p * c->share_nz + (double)q * cell;
+    const double terms = uniform ? (double)p * c->share_cell
+                                 : (double)p * c->share_nz + (double)q * c->share_cell;
     const double pass = (double)(p + q) * 8.0 * c->d * c->Rp / 9000.0;  // ns
-    const double want = hits * 4.7 / std::max(0.06 * pass, 4000.0);
+    const double want = std::max(hits * 4.7 / std::max(0.06 * pass, 4000.0), terms / 256.0);
     return want <= 1.0 ? 0 : (want <= 4.0 ? 4 : (want <= 16.0 ? 16 : gcpk::kReplicas));
 }
 

@@ -328,8 +328,9 @@ const char *gcp_batch_last_error(const gcp_batch *batch);
  * the graph at the next gcp_batch_local_steps. */
 gcp_status gcp_batch_tune(gcp_batch *batch, int32_t lane_cols, int32_t blocks);
 
-/* Tuning knob of the multi-client fused kernel: samples per warp tile (16,
- * 32 or 64; 0 = 32).  A warp stages a tile's samples (one, or for 64 two,
+/* Tuning knob of the multi-client fused kernel: samples per warp tile at most
+ * (16, 32 or 64; 0 = 32; fewer where the last round of tiles would be mostly
+ * empty).  A warp stages a tile's samples (one, or for 64 two,
  * per lane; for 16 only half its lanes) and then evaluates them; smaller
  * tiles spread a step over more warps, larger ones keep more sample loads
  * in flight per warp.  The grid size follows the new tile size's occupancy
@@ -342,8 +343,9 @@ gcp_status gcp_batch_tune_tile(gcp_batch *batch, int32_t samples_per_warp);
  * iter0 + k and applies Adam step t0 + k + 1 (Alg. 1) with prm.  Each client
  * ends with the same state as tau rounds of gcp_grad + gcp_adam_step on its
  * own context, up to the summation order of the atomic MTTKRP.  A step is
- * four launches in the graph: gradients cleared, the multi-client fused
- * pass, one epilogue (loss finish, replica fold, Adam) and a counter advance.
+ * two launches in the graph: the multi-client fused pass and one epilogue
+ * (loss finish, replica fold, Adam, gradients cleared); the first step, and
+ * every step of a batch larger than L2, clears the gradients in a third.
  * Asynchronous on the clients' stream; back-to-back calls need no sync. */
 gcp_status gcp_batch_local_steps(gcp_batch *batch, int32_t tau, const gcp_adam_params *prm, uint64_t iter0,
                                  int64_t t0);

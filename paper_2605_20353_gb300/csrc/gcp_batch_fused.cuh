@@ -54,17 +54,20 @@ __device__ __forceinline__ int client_of(const int *__restrict__ tile_start, int
 
 // Multi-client fused sampled gradient.  Each client's FusedSpec (stored as
 // kSpecWords 16-byte words) gives its tensor, model, gradient and weights;
-// the iteration number is step[0].  A tile holds TS consecutive samples of
-// one client (TS = 16, 32 or 64 samples per warp, a tuning knob): in phase
-// A, lane l stages the samples at positions l, l + 32, ... of the tile
-// (for TS = 16 lanes 16..31 stage nothing); in phase B the warp's groups
+// the iteration number is step[0] + k.  A tile holds `tile_n` <= TS
+// consecutive samples of one client (TS = 16, 32 or 64 samples per warp, a
+// tuning knob; tile_n evens out the rounds, batch_tiles): in phase
+// A, lane l stages the samples at positions l, l + 32, ... of the tile;
+// in phase B the warp's groups
 // take the tile's samples in turn.  Per tile, the FP32 loss sums (nonzero,
-// zero) go to tile_loss[tile].
+// zero) go to tile_loss[tile].  The first tile is drawn beside the end of the
+// grid before; the factors, which that grid may write, are read after it.
 template <int D, typename TF, int COLS, int TS>
 __global__ void __launch_bounds__(kThreads, gcpk::fused_min_blocks(D, COLS)) k_batch_fused(const int4 *__restrict__ specs,
                                                          const int *__restrict__ tile_start, int nclients,
-                                                         int total_tiles, int log2L, int Rp,
-                                                         const uint64_t *__restrict__ step, float2 *tile_loss) {
+                                                         int total_tiles, int tile_n, int log2L, int Rp,
+                                                         const uint64_t *__restrict__ step, int k_step,
+                                                         float2 *tile_loss) {
     constexpr int SW = gcpk::rec_words_for(D);
     constexpr int NQ = COLS / 4;
     constexpr int SPL = TS >= 32 ? TS / 32 : 1;  // tile positions a lane stages
@@ -89,7 +92,7 @@ __global__ void __launch_bounds__(kThreads, gcpk::fused_min_blocks(D, COLS)) k_b
     for (int q = 0; q < NQ; ++q) col[q] = q * (Rp >> 1) + 4 * glane;
     const int nwarps = (gridDim.x * blockDim.x) >> 5;
     const int warp0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
-    const uint64_t iter = __ldg(step);
+    const uint64_t iter = __ldg(step) + (uint64_t)k_step;
     int cur_client[2] = {-1, -1};
 
     auto spec_of = [&](int st) -> const gcpk::FusedSpec & {
@@ -118,13 +121,14 @@ __global__ void __launch_bounds__(kThreads, gcpk::fused_min_blocks(D, COLS)) k_b
         const int c = stage_spec(tile, st);
         const gcpk::FusedSpec &P = spec_of(st);
         const int p = (int)P.s.p, S = (int)(P.s.p + P.s.q);
-        const int base = (tile - __ldg(tile_start + c)) * TS;
+        const int base = (tile - __ldg(tile_start + c)) * tile_n;
         const bool semi = P.s.sampling == GCP_SAMPLING_SEMI_STRATIFIED;
 #pragma unroll
         for (int j = 0; j < SPL; ++j) {
             const int pos = lane + 32 * j;
-            const int s = base + pos;
-            if (pos >= TS || s >= S) continue;
+            const unsigned us = (unsigned)base + pos;  // may pass 2^31 - 1 in the last tile
+            if (pos >= tile_n || us >= (unsigned)S) continue;
+            const int s = (int)us;
             int32_t *slot = s_slot[st][warp][pos];
             if (s < p) {
                 const U64x4 w = philox4x64_10((uint64_t)s, 0, P.s.iter, 0, P.s.seed, kStreamNonzero);
@@ -150,8 +154,9 @@ __global__ void __launch_bounds__(kThreads, gcpk::fused_min_blocks(D, COLS)) k_b
     auto finish = [&](int tile, int st, uint64_t key, int pos) -> bool {
         const gcpk::FusedSpec &P = spec_of(st);
         const int p = (int)P.s.p, S = (int)(P.s.p + P.s.q);
-        const int s = (tile - __ldg(tile_start + cur_client[st])) * TS + pos;
-        if (pos >= TS || s >= S) return false;
+        const unsigned us = (unsigned)(tile - __ldg(tile_start + cur_client[st])) * tile_n + pos;
+        if (pos >= tile_n || us >= (unsigned)S) return false;
+        const int s = (int)us;
         if (key == kEmpty) return true;
         const ulonglong2 lo = *reinterpret_cast<const ulonglong2 *>(&s_bkt[st][warp][pos][0]);
         const ulonglong2 hi = *reinterpret_cast<const ulonglong2 *>(&s_bkt[st][warp][pos][2]);
@@ -179,6 +184,8 @@ __global__ void __launch_bounds__(kThreads, gcpk::fused_min_blocks(D, COLS)) k_b
     uint64_t key_next[SPL];
     issue(tile, 0, key_next);
     cp_async_commit();
+    grid_wait();
+    grid_trigger();
     for (int st = 0; tile < total_tiles; tile += nwarps, st ^= 1) {
         uint64_t key[SPL];
 #pragma unroll
@@ -194,28 +201,28 @@ __global__ void __launch_bounds__(kThreads, gcpk::fused_min_blocks(D, COLS)) k_b
         __syncwarp();
 
         const gcpk::FusedSpec &P = spec_of(st);
-        const TF *__restrict__ F = static_cast<const TF *>(P.F);
+        const TF *F = static_cast<const TF *>(P.F);
         const int p = (int)P.s.p;
-        const int tbase = (tile - __ldg(tile_start + cur_client[st])) * TS;
+        const int tbase = (tile - __ldg(tile_start + cur_client[st])) * tile_n;
         const bool semi = P.s.sampling == GCP_SAMPLING_SEMI_STRATIFIED;
         float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (P.nrep - 1)) * P.Htot * Rp : nullptr;
         float tf_nz = 0.0f, tf_z = 0.0f;
-        for (int it = 0; it * ngrp < TS; ++it) {
+        for (int it = 0; it * ngrp < tile_n; ++it) {
             const int src = it * ngrp + grp;
-            if (src >= TS || !((okmask >> src) & 1ull)) continue;  // uniform within the group
+            if (src >= tile_n || !((okmask >> src) & 1ull)) continue;  // uniform within the group
             const int32_t *slot = s_slot[st][warp][src];
             int32_t ii[D];
 #pragma unroll
             for (int k = 0; k < D; ++k) ii[k] = slot[k];
             const float xs = __int_as_float(slot[D]);
-            const bool is_nz = (tbase + src) < p;
+            const bool is_nz = (unsigned)tbase + src < (unsigned)p;
             int off[D];
             float a[D][COLS];
 #pragma unroll
             for (int k = 0; k < D; ++k) {
                 off[k] = (P.rowoff[k] + ii[k]) * Rp;
 #pragma unroll
-                for (int q = 0; q < NQ; ++q) Quad<TF>::load(F + off[k] + col[q], a[k] + 4 * q);
+                for (int q = 0; q < NQ; ++q) load_quad_coherent(F + off[k] + col[q], a[k] + 4 * q);
             }
             float suf[D][COLS];
 #pragma unroll
@@ -279,7 +286,7 @@ constexpr size_t batch_fused_smem(int d, int ts) {
            (size_t)2 * kWarps * kSpecWords * sizeof(int4);
 }
 
-using FusedKernel = void (*)(const int4 *, const int *, int, int, int, int, const uint64_t *, float2 *);
+using FusedKernel = void (*)(const int4 *, const int *, int, int, int, int, int, const uint64_t *, int, float2 *);
 
 // The instantiation for (dtype, cols); with `allow`, its dynamic shared
 // memory limit is raised to what it needs (a host call made before any
@@ -302,14 +309,13 @@ cudaError_t fused_kernel_ts(bool bf16, int cols, FusedKernel *k, bool allow) {
 
 template <int D, int TS>
 cudaError_t launch_fused_ts(bool bf16, int cols, int blocks, const int4 *specs, const int *tile_start, int n,
-                            int total_tiles, int log2L, int Rp, const uint64_t *step, float2 *tile_loss,
-                            cudaStream_t st) {
+                            int total_tiles, int tile_n, int log2L, int Rp, const uint64_t *step, int k_step,
+                            float2 *tile_loss, cudaStream_t st) {
     FusedKernel k = nullptr;
     cudaError_t e = fused_kernel_ts<D, TS>(bf16, cols, &k, false);
     if (e != cudaSuccess) return e;
-    k<<<blocks, kThreads, batch_fused_smem(D, TS), st>>>(specs, tile_start, n, total_tiles, log2L, Rp, step,
-                                                          tile_loss);
-    return cudaGetLastError();
+    return gcpk::launch_dependent(k, blocks, kThreads, batch_fused_smem(D, TS), st, specs, tile_start, n, total_tiles,
+                                  tile_n, log2L, Rp, step, k_step, tile_loss);
 }
 
 template <int D, int TS>
@@ -338,10 +344,10 @@ int occupancy_ts(bool bf16, int cols) {
 
 template <int TS>
 cudaError_t batch_fused_launch(int d, bool bf16, int cols, int blocks, const int4 *specs, const int *tile_start,
-                               int n, int total_tiles, int log2L, int Rp, const uint64_t *step, float2 *tile_loss,
-                               cudaStream_t st) {
-    GCPB_FOR_D(d, return (launch_fused_ts<D, TS>(bf16, cols, blocks, specs, tile_start, n, total_tiles, log2L, Rp,
-                                                 step, tile_loss, st)))
+                               int n, int total_tiles, int tile_n, int log2L, int Rp, const uint64_t *step,
+                               int k_step, float2 *tile_loss, cudaStream_t st) {
+    GCPB_FOR_D(d, return (launch_fused_ts<D, TS>(bf16, cols, blocks, specs, tile_start, n, total_tiles, tile_n, log2L,
+                                                 Rp, step, k_step, tile_loss, st)))
     return cudaErrorInvalidValue;
 }
 

@@ -4,8 +4,8 @@
 
 namespace gcpb {
 
-template cudaError_t batch_fused_launch<16>(int, bool, int, int, const int4 *, const int *, int, int, int, int,
-                                            const uint64_t *, float2 *, cudaStream_t);
+template cudaError_t batch_fused_launch<16>(int, bool, int, int, const int4 *, const int *, int, int, int, int, int,
+                                            const uint64_t *, int, float2 *, cudaStream_t);
 template cudaError_t batch_fused_allow<16>(int, bool, int);
 template int batch_fused_occupancy<16>(int, bool, int);
 

@@ -383,7 +383,7 @@ int fused_occupancy_d(bool bf16, int cols) {
 
 template <int D, typename TF, int COLS, bool EVAL>
 cudaError_t launch_fused_k(const FusedSpec &f, int blocks, cudaStream_t st) {
-    if (f.dependent) return launch_dependent(k_fused<D, TF, COLS, EVAL>, blocks, kThreads, st, f);
+    if (f.dependent) return launch_dependent(k_fused<D, TF, COLS, EVAL>, blocks, kThreads, 0, st, f);
     k_fused<D, TF, COLS, EVAL><<<blocks, kThreads, 0, st>>>(f);
     return cudaGetLastError();
 }

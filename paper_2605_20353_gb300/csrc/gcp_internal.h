@@ -115,13 +115,14 @@ __host__ __device__ constexpr int fused_min_blocks(int d, int cols) {
 // (programmatic dependent launch); the kernel calls gcpdev::grid_wait before
 // it touches what that grid writes.
 template <typename... Params, typename... Args>
-cudaError_t launch_dependent(void (*k)(Params...), int blocks, int threads, cudaStream_t st, Args... args) {
+cudaError_t launch_dependent(void (*k)(Params...), dim3 blocks, int threads, size_t smem, cudaStream_t st, Args... args) {
     cudaLaunchAttribute at{};
     at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
     at.val.programmaticStreamSerializationAllowed = 1;
     cudaLaunchConfig_t cfg{};
-    cfg.gridDim = dim3((unsigned)blocks);
+    cfg.gridDim = blocks;
     cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem;
     cfg.stream = st;
     cfg.attrs = &at;
     cfg.numAttrs = 1;

@@ -376,7 +376,7 @@ static cudaError_t launch_post_step_r(const PostSpec &p, cudaStream_t st) {
         nhot = (int)(((int64_t)p.Htot * (p.Rp >> 2) + per - 1) / per);
     }
     const int blocks = ncold + nhot + 1;  // + the loss block
-    return launch_dependent(k_post_step<NREP>, blocks, kThreads, st, p, ncold);
+    return launch_dependent(k_post_step<NREP>, blocks, kThreads, 0, st, p, ncold);
 }
 
 cudaError_t launch_post_step(const PostSpec &p, cudaStream_t st) {
@@ -544,7 +544,7 @@ static cudaError_t launch_grad_finish_rv(const GradOutSpec &p, cudaStream_t st) 
         nhot = (int)(((int64_t)p.Htot * (p.Rp >> 2) + per - 1) / per);
     }
     const int blocks = ncold + nhot + 1;  // + the loss block
-    return launch_dependent(k_grad_finish<NREP, V>, blocks, kThreads, st, p, ncold);
+    return launch_dependent(k_grad_finish<NREP, V>, blocks, kThreads, 0, st, p, ncold);
 }
 
 template <int NREP>
@@ -564,7 +564,7 @@ cudaError_t launch_grad_finish(const GradOutSpec &p, cudaStream_t st) {
 }
 
 cudaError_t launch_finish_loss(const LossSpec &l, cudaStream_t st) {
-    return launch_dependent(k_finish_loss, 1, kThreads, st, l);
+    return launch_dependent(k_finish_loss, 1, kThreads, 0, st, l);
 }
 
 // x = 0 before a gradient pass, as a kernel and not a memset so that the pass
@@ -577,7 +577,7 @@ __global__ void __launch_bounds__(kThreads) k_clear(float4 *x, int64_t nq) {
 }
 
 cudaError_t launch_clear(float *x, int64_t n, cudaStream_t st) {
-    return launch_dependent(k_clear, elementwise_blocks(n >> 2), kThreads, st, reinterpret_cast<float4 *>(x), n >> 2);
+    return launch_dependent(k_clear, elementwise_blocks(n >> 2), kThreads, 0, st, reinterpret_cast<float4 *>(x), n >> 2);
 }
 
 cudaError_t launch_adam(int64_t n, int Rp, int R, float *A, float *B, float *C, const float *G, float lr,

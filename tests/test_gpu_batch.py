@@ -423,3 +423,42 @@ def test_batch_orders_and_tiles_match_clients_alone(env, ndim, rank, tile):
     b.close()
     for c in ref + bat:
         c.close()
+
+
+@pytest.mark.parametrize("nrows", [700, 400000])
+@pytest.mark.parametrize("tile", [16, 32, 64])
+def test_batch_tiles_rounds_and_gradient_clearing(env, tile, nrows):
+    """Sample counts that leave the last round of tiles mostly empty (so that
+    the batch takes smaller ones), one that fits in a single tile and an empty
+    client, with the gradients cleared by the epilogue (small models) or
+    before each pass (models beyond L2): three local steps, twice, leave every
+    client where its own gcp_step calls do."""
+    gcp, torch = env
+    dims, R = [31, 41, nrows], 9
+    warps = torch.cuda.get_device_properties(0).multi_processor_count * 32
+    counts = [(9 * warps, 8 * warps + 1), (5, 6), (0, 0), (11 * warps + 7, 0), (700, 913)]
+    prm = gcp.AdamParams(lr=1e-2, beta1=0.9, beta2=0.99, eps=1e-8, lower=0.05)
+    made = []
+    for i in range(len(counts)):
+        coords, vals = synth.uniform_sparse(dims, 3000, 740 + i, lam=2.0)
+        fac = synth.factors_uniform(dims, R, 750 + i, lo=0.1, hi=1.0)
+        pair = []
+        for _ in range(2):
+            c = gcp.gcp_create(dims, coords, vals, R, "poisson", seed=760 + i)
+            c.set_factors(fac)
+            pair.append(c)
+        made.append(pair)
+    b = gcp.GcpBatch([a for a, _ in made], [p for p, _ in counts], [q for _, q in counts])
+    b.tune(samples_per_warp=tile)
+    for call in range(2):
+        b.local_steps(3, prm, 10 * call, 3 * call)
+        losses = b.losses()
+        for (a, alone), (p, q), L in zip(made, counts, losses):
+            dl = torch.zeros(1, dtype=torch.float64, device="cuda")
+            for k in range(3):
+                alone.step(10 * call + k, p, q, prm, 3 * call + k + 1, dloss=dl)
+            ref = np.concatenate([x.ravel() for x in alone.get_factors()])
+            got = np.concatenate([x.ravel() for x in a.get_factors()])
+            assert L == pytest.approx(dl.item(), rel=1e-5, abs=0.0)
+            assert rel_err(got, ref) <= 1e-5, (call, p, q, rel_err(got, ref))
+    b.close()

@@ -80,9 +80,9 @@ typedef enum {
                                      grows a scratch buffer for the largest sample count
                                      S = p + q seen: a 16, 32 or 64 B record per sample, 16 B
                                      per sample and mode for the modes sorted side by side
-                                     (as many as fit 1 GiB, at least one), 8 x padded rank B
-                                     per 64 samples, and small counts; GCP_ERR_OOM if it
-                                     cannot.  It also creates a second stream for its sort
+                                     (as many as fit 1 GiB, at least one), for each of them
+                                     8 x padded rank B per 64 samples, and small counts;
+                                     GCP_ERR_OOM if it cannot.  It also creates a second stream for its sort
                                      on first use, so make the first call with the largest
                                      sample count outside stream capture */
     GCP_MTTKRP_NONFUSED = 2       /* sampling writes the gradient tensor, then a separate

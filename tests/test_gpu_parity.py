@@ -968,3 +968,36 @@ def test_back_to_back_calls_wait_for_one_another(env, p, q, dtype):
     for how in ("run", "graph"):
         for a, b in zip(out[how], out["wait"]):
             assert rel_err(a, b) <= 1e-5, (how, rel_err(a, b))
+
+
+@pytest.mark.parametrize("dims,R,dtype", [([100, 256, 40], 6, "fp32"), ([10000, 700, 200], 64, "fp32"),
+                                          ([40000, 128, 129], 5, "bf16"), ([100000, 300, 9000], 16, "fp32"),
+                                          ([1024, 1025], 33, "fp32"), ([5, 16384, 16385, 3], 20, "fp32")])
+def test_deterministic_mttkrp_digit_widths_and_long_runs(env, dims, R, dtype):
+    """Modes that sort in one to three passes of 7, 8 and 10 bits, side by
+    side, and skewed nonzeros: a third of them share one row of every mode, so
+    that row's run covers hundreds of chunks and is summed by a whole block,
+    beside runs inside a chunk and across a few.  Against the oracle, and bit
+    for bit the same from call to call."""
+    gcp, torch = env
+    rng = np.random.default_rng(1000 + R)
+    n = 6000
+    coords = np.stack([rng.integers(0, I, n) for I in dims], 1).astype(np.int32)
+    for k in range(len(dims)):
+        coords[rng.random(n) < 0.33, k] = dims[k] // 3
+    coords = np.unique(coords, axis=0).astype(np.int32)
+    vals = (1 + rng.poisson(2.0, len(coords))).astype(np.float32)
+    factors = synth.factors_uniform(dims, R, 1001, lo=0.1, hi=1.0)
+    ctx = gcp.gcp_create(dims, coords, vals, R, "poisson", seed=1002, dtype=dtype, mttkrp="deterministic")
+    ctx.set_factors(factors)
+    fac = [bf16_round(a) for a in factors] if dtype == "bf16" else factors
+    for p, q in [(60001, 30000), (1, 1), (4100, 0), (63, 65)]:
+        idx, x, w, _ = oracle.stratified_samples(1002, 3, p, q, dims, coords, vals)
+        Lo, Go = oracle.sampled_loss_grad(dims, fac, "poisson", idx, x, w)
+        Lg, Gg = gpu_grad(gcp, torch, ctx, 3, p, q)
+        Lh, Gh = gpu_grad(gcp, torch, ctx, 3, p, q)
+        assert Lg == Lh and np.array_equal(Gg.view(np.uint32), Gh.view(np.uint32))
+        assert abs(Lg - Lo) <= TOL_FP32 * abs(Lo)
+        for m, (a, b) in enumerate(zip(split(Gg, dims, R), Go)):
+            assert rel_err(a, b) <= TOL_FP32, (p, q, m, rel_err(a, b))
+    ctx.close()

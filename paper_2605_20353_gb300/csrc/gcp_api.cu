@@ -11,6 +11,7 @@
 #include <string>
 #include <vector>
 
+#include "gcp_device.cuh"
 #include "gcp_internal.h"
 
 namespace {
@@ -48,6 +49,8 @@ gcp_status cuda_fail(gcp_ctx *c, cudaError_t e, const char *what) {
         cudaError_t e_ = (call);                                 \
         if (e_ != cudaSuccess) return cuda_fail(ctx, e_, #call); \
     } while (0)
+
+constexpr int64_t kStageBytes = 8 << 20;  // rows_out, rows_in
 
 uint64_t next_pow2(uint64_t v) {
     uint64_t p = 1;
@@ -92,6 +95,7 @@ void destroy_buffers(gcp_ctx *c) {
     cudaFree(c->hkeys);
     cudaFree(c->X);
     cudaFree(c->A);
+    cudaFree(c->stage);
     cudaFree(c->Abf);
     cudaFree(c->G);
     cudaFree(c->B);
@@ -206,6 +210,11 @@ gcp_status init_common(gcp_ctx *c, int32_t ndim, const int64_t *dims, int32_t ra
         (e = cudaMalloc(&c->dloss, 4 * sizeof(double))) || (e = cudaMalloc(&c->status, sizeof(int))) ||
         (e = cudaMallocHost(&c->h_status, sizeof(int))) || (e = cudaMallocHost(&c->h_loss, 4 * sizeof(double))))
         return cuda_fail(nullptr, e, "allocating model buffers");
+    if (c->R != c->Rp) {
+        c->stage_rows = std::min<int64_t>(c->total_rows, std::max<int64_t>(1, kStageBytes / (4 * c->R)));
+        if ((e = cudaMalloc(&c->stage, (size_t)c->stage_rows * c->R * 4)))
+            return cuda_fail(nullptr, e, "allocating the staging rows");
+    }
     if (c->opt.factor_dtype == GCP_BF16 && (e = cudaMalloc(&c->Abf, nparam * 2)))
         return cuda_fail(nullptr, e, "allocating BF16 factors");
     c->max_blocks = gcpk::fused_max_blocks(ndim, c->opt.factor_dtype == GCP_BF16, c->cols);
@@ -555,24 +564,51 @@ __global__ void k_check_dense(const float *X, int64_t n, int loss, int *status) 
     if (bad) atomicOr(status, bad);
 }
 
-// Every mode's factor matrix (src.A[k], I_k x R row-major, device memory)
-// copied into the context's padded flat layout in one launch; padding
-// columns are written as zero and the BF16 copy, if any, is refreshed.
+// Factor matrices (src.A[k], I_k x R row-major, device memory) of the modes
+// whose rows are row0 .. row0 + rows - 1 copied into the context's padded flat
+// layout in one launch, one 16-byte quad of a padded row per thread; padding
+// columns are written as zero and the BF16 copy, if any, is refreshed.  VEC:
+// R and every pointer allow 16-byte loads.
 struct FactorSrc {
     const float *A[GCP_MAX_NDIM];
     int64_t rowoff[GCP_MAX_NDIM + 1];  // first row of each mode, then the total
 };
 
-__global__ void k_stage_factors(FactorSrc src, int d, int R, int log2Rp, int64_t n, float *__restrict__ A,
-                                __nv_bfloat16 *__restrict__ Abf) {
-    for (int64_t e = (int64_t)blockIdx.x * blockDim.x + threadIdx.x; e < n; e += (int64_t)gridDim.x * blockDim.x) {
-        const int64_t row = e >> log2Rp;
-        const int col = (int)(e & ((1 << log2Rp) - 1));
-        int k = 0;
-        while (k + 1 < d && row >= src.rowoff[k + 1]) ++k;
-        const float v = col < R ? __ldg(src.A[k] + (row - src.rowoff[k]) * R + col) : 0.0f;
-        A[e] = v;
-        if (Abf) Abf[e] = __float2bfloat16_rn(v);
+template <bool VEC>
+__global__ void __launch_bounds__(256) k_stage_factors(FactorSrc src, int d, int R, int log2Rp, int64_t row0,
+                                                       int64_t rows, float *A, __nv_bfloat16 *Abf) {
+    gcpdev::grid_wait();  // the matrices and the context's factors may be in use by the grid before
+    gcpdev::grid_trigger();
+    const int log2Q = log2Rp - 2;
+    const int64_t nq = rows << log2Q;
+    for (int64_t e = (int64_t)blockIdx.x * 256 + threadIdx.x; e < nq; e += (int64_t)gridDim.x * 256) {
+        const int64_t row = row0 + (e >> log2Q);
+        const int col = (int)(e & ((1 << log2Q) - 1)) << 2;
+        const float *base = src.A[0];
+        int64_t first = 0;
+#pragma unroll
+        for (int k = 1; k < GCP_MAX_NDIM; ++k)  // constant indices only
+            if (k < d && row >= src.rowoff[k]) {
+                base = src.A[k];
+                first = src.rowoff[k];
+            }
+        const float *a = base + (row - first) * R + col;
+        float4 v = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+        if (VEC) {
+            if (col < R) v = *reinterpret_cast<const float4 *>(a);
+        } else {
+            if (col < R) v.x = a[0];
+            if (col + 1 < R) v.y = a[1];
+            if (col + 2 < R) v.z = a[2];
+            if (col + 3 < R) v.w = a[3];
+        }
+        const int64_t q = (row << log2Q) + (col >> 2);
+        reinterpret_cast<float4 *>(A)[q] = v;
+        if (Abf) {
+            const __nv_bfloat162 lo = __floats2bfloat162_rn(v.x, v.y), hi = __floats2bfloat162_rn(v.z, v.w);
+            reinterpret_cast<uint2 *>(Abf)[q] = make_uint2(*reinterpret_cast<const unsigned *>(&lo),
+                                                           *reinterpret_cast<const unsigned *>(&hi));
+        }
     }
 }
 
@@ -602,32 +638,118 @@ __global__ void k_sumsq_blocks(const float *__restrict__ x, int64_t n, double *p
     if (threadIdx.x == 0) partial[blockIdx.x] = sh[0];
 }
 
-// out[0] = sqrt(sum of the block partials), summed in block order; a
+// out[0] = sqrt(sum of the block partials), a fixed tree over one block; a
 // non-finite result sets the status word.
-__global__ void k_sumsq_finish(const double *__restrict__ partial, int nblocks, double *out, int *status) {
-    if (threadIdx.x != 0 || blockIdx.x != 0) return;
+__global__ void __launch_bounds__(256) k_sumsq_finish(const double *__restrict__ partial, int nblocks, double *out,
+                                                      int *status) {
+    __shared__ double sh[256];
     double t = 0.0;
-    for (int b = 0; b < nblocks; ++b) t += partial[b];
-    out[0] = sqrt(t);
-    if (!isfinite(t)) atomicOr(status, 1 << GCP_ERR_NONFINITE);
+    for (int b = threadIdx.x; b < nblocks; b += 256) t += partial[b];
+    sh[threadIdx.x] = t;
+    __syncthreads();
+    for (int h = 128; h > 0; h >>= 1) {
+        if ((int)threadIdx.x < h) sh[threadIdx.x] += sh[threadIdx.x + h];
+        __syncthreads();
+    }
+    if (threadIdx.x != 0) return;
+    out[0] = sqrt(sh[0]);
+    if (!isfinite(sh[0])) atomicOr(status, 1 << GCP_ERR_NONFINITE);
 }
 
-// Copy `rows` rows of `width` bytes between arrays whose rows are dpitch
-// and spitch bytes apart.  With equal pitches and no padding the rows are
-// one contiguous block and go as one plain copy (the strided form moves
-// each row separately).
-static cudaError_t copy_rows(void *dst, size_t dpitch, const void *src, size_t spitch, size_t width, size_t rows,
-                      cudaStream_t st) {
-    if (dpitch == width && spitch == width)
-        return cudaMemcpyAsync(dst, src, width * rows, cudaMemcpyDefault, st);
-    return cudaMemcpy2DAsync(dst, dpitch, src, spitch, width, rows, cudaMemcpyDefault, st);
-}
+// Rows row0 .. row0 + rows - 1 of padded device memory (row stride Rp) copied
+// out to `out` (unpadded rows of R floats).  Device memory that kernels can
+// write takes one kernel, except unpadded rows of 32 MB and more, where a
+// plain copy is faster (486 MB: 164 against 174 us).  Host memory, and
+// anything else, takes plain copies: of the rows as they are where there is
+// no padding, else of unpadded rows staged kStageBytes at a time.  A strided
+// copy moves each row by itself, about 2 ns a row out and 10 ns in: 10^6 rows
+// of 10 floats 1.9 ms out and 10.5 ms in, against 0.29 ms staged; it stays for
+// few rows, where it saves a launch (120 rows: 11 against 16 us out with the
+// synchronisation, 3.4 against 9.2 us in).
+constexpr int64_t kPlainBytes = 32 << 20, kStridedOut = 2048, kStridedIn = 512;
 
-gcp_status copy_grad_out(gcp_ctx *c, float *G_out) {
-    GCP_CUDA(c, copy_rows(G_out, (size_t)c->R * 4, c->G, (size_t)c->Rp * 4, (size_t)c->R * 4,
-                                  (size_t)c->total_rows, c->st));
+gcp_status rows_out(gcp_ctx *c, const float *src, int64_t row0, int64_t rows, float *out) {
+    const float *p = src + row0 * c->Rp;
+    const size_t row = (size_t)c->R * 4;
+    if (!(c->R == c->Rp && rows * (int64_t)row >= kPlainBytes) && kernel_writable(c, out, sizeof(float))) {
+        GCP_CUDA(c, gcpk::launch_unpad(p, c->Rp, c->R, rows, out, c->st));
+        return GCP_OK;
+    }
+    if (c->R != c->Rp && rows <= kStridedOut) {
+        GCP_CUDA(c, cudaMemcpy2DAsync(out, row, p, (size_t)c->Rp * 4, row, (size_t)rows, cudaMemcpyDefault, c->st));
+        return GCP_OK;
+    }
+    if (c->R == c->Rp) {
+        GCP_CUDA(c, cudaMemcpyAsync(out, p, row * rows, cudaMemcpyDefault, c->st));
+        return GCP_OK;
+    }
+    for (int64_t r = 0; r < rows; r += c->stage_rows) {
+        const int64_t n = std::min(c->stage_rows, rows - r);
+        GCP_CUDA(c, gcpk::launch_unpad(p + r * c->Rp, c->Rp, c->R, n, c->stage, c->st));
+        GCP_CUDA(c, cudaMemcpyAsync(reinterpret_cast<char *>(out) + r * row, c->stage, row * n, cudaMemcpyDefault,
+                                    c->st));
+    }
     return GCP_OK;
 }
+
+// Rows row0 .. row0 + rows - 1 of the factors (and of their BF16 copy) from
+// the matrices src.A of the modes they span, device memory.
+gcp_status stage_factors(gcp_ctx *c, const FactorSrc &src, int64_t row0, int64_t rows) {
+    int log2Rp = 0;
+    while ((1 << log2Rp) < c->Rp) ++log2Rp;
+    bool vec = c->R % 4 == 0;
+    for (int k = 0; k < c->d; ++k) vec = vec && (reinterpret_cast<uintptr_t>(src.A[k]) & 15) == 0;
+    const int64_t want = (rows * (c->Rp / 4) + 255) / 256;
+    const dim3 grid((unsigned)(want < 8192 ? want : 8192));
+    auto *bf = static_cast<__nv_bfloat16 *>(c->Abf);
+    if (vec)
+        GCP_CUDA(c, gcpk::launch_dependent(k_stage_factors<true>, grid, 256, 0, c->st, src, c->d, c->R, log2Rp, row0,
+                                           rows, c->A, bf));
+    else
+        GCP_CUDA(c, gcpk::launch_dependent(k_stage_factors<false>, grid, 256, 0, c->st, src, c->d, c->R, log2Rp, row0,
+                                           rows, c->A, bf));
+    return GCP_OK;
+}
+
+// The same from the unpadded rows at `in` (host or device): see rows_out.
+gcp_status rows_in(gcp_ctx *c, int64_t row0, int64_t rows, const float *in) {
+    FactorSrc src{};  // the modes' matrices as the kernel reads them, were all rows at `at`
+    auto from = [&](const float *at, int64_t first) {
+        for (int k = 0; k < c->d; ++k) {
+            src.A[k] = at + (c->rowoff[k] - first) * c->R;
+            src.rowoff[k] = c->rowoff[k];
+        }
+        src.rowoff[c->d] = c->total_rows;
+    };
+    const size_t row = (size_t)c->R * 4;
+    const bool plain = c->R == c->Rp && !c->Abf && rows * (int64_t)row >= kPlainBytes;
+    if (!plain && kernel_writable(c, in, sizeof(float))) {
+        from(in, row0);
+        return stage_factors(c, src, row0, rows);
+    }
+    if (c->R == c->Rp || rows <= kStridedIn) {
+        if (c->R == c->Rp)
+            GCP_CUDA(c, cudaMemcpyAsync(c->A + row0 * c->Rp, in, row * rows, cudaMemcpyDefault, c->st));
+        else
+            GCP_CUDA(c, cudaMemcpy2DAsync(c->A + row0 * c->Rp, (size_t)c->Rp * 4, in, row, row, (size_t)rows,
+                                          cudaMemcpyDefault, c->st));
+        if (c->Abf)
+            GCP_CUDA(c, gcpk::launch_to_bf16(rows * c->Rp, c->A + row0 * c->Rp,
+                                             static_cast<__nv_bfloat16 *>(c->Abf) + row0 * c->Rp, c->st));
+        return GCP_OK;
+    }
+    for (int64_t r = 0; r < rows; r += c->stage_rows) {
+        const int64_t n = std::min(c->stage_rows, rows - r);
+        GCP_CUDA(c, cudaMemcpyAsync(c->stage, reinterpret_cast<const char *>(in) + r * row, row * n,
+                                    cudaMemcpyDefault, c->st));
+        from(c->stage, row0 + r);
+        gcp_status s = stage_factors(c, src, row0 + r, n);
+        if (s) return s;
+    }
+    return GCP_OK;
+}
+
+gcp_status copy_grad_out(gcp_ctx *c, float *G_out) { return rows_out(c, c->G, 0, c->total_rows, G_out); }
 
 gcp_status refresh_bf16(gcp_ctx *c) {
     if (!c->Abf) return GCP_OK;
@@ -643,8 +765,8 @@ gcp_status refresh_bf16(gcp_ctx *c) {
 // first.  A nonzero record stores the slots of its rows.
 gcp_status setup_hot_rows(gcp_ctx *c, const std::vector<int64_t> &counts) {
     std::vector<int> slot((size_t)c->total_rows, -1), row;
-    for (int64_t n : counts) c->share_nz = std::max(c->share_nz, (double)n / (double)c->nnz);
     for (int k = 0; k < c->d; ++k) c->share_cell = std::max(c->share_cell, 1.0 / (double)c->dims[k]);
+    int64_t most = 0;  // nonzeros of the fullest row
     for (int k = 0; k < c->d; ++k) {
         c->small_base[k] = -1;
         if (c->dims[k] > 512) continue;
@@ -652,15 +774,20 @@ gcp_status setup_hot_rows(gcp_ctx *c, const std::vector<int64_t> &counts) {
         for (int64_t i = 0; i < c->dims[k]; ++i) {
             slot[(size_t)(c->rowoff[k] + i)] = (int)row.size();
             row.push_back((int)(c->rowoff[k] + i));
+            if (!counts.empty()) most = std::max(most, counts[(size_t)(c->rowoff[k] + i)]);
         }
     }
+    const int64_t floor_hot = (c->nnz + 511) / 512;  // the fewest nonzeros that are 1/512 of all
     for (int k = 0; k < c->d && !counts.empty(); ++k) {
         if (c->dims[k] <= 512) continue;
         std::vector<std::pair<int64_t, int>> hot;
+        const int64_t *at = counts.data() + c->rowoff[k];
+        int64_t fullest = 0;
         for (int64_t i = 0; i < c->dims[k]; ++i) {
-            const int64_t n = counts[(size_t)(c->rowoff[k] + i)];
-            if ((double)n * 512.0 >= (double)c->nnz) hot.push_back({n, (int)(c->rowoff[k] + i)});
+            fullest = std::max(fullest, at[i]);
+            if (at[i] >= floor_hot) hot.push_back({at[i], (int)(c->rowoff[k] + i)});
         }
+        most = std::max(most, fullest);
         std::stable_sort(hot.begin(), hot.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
         if (hot.size() > 256) hot.resize(256);
         for (const auto &h : hot) {
@@ -668,6 +795,7 @@ gcp_status setup_hot_rows(gcp_ctx *c, const std::vector<int64_t> &counts) {
             row.push_back(h.second);
         }
     }
+    c->share_nz = counts.empty() ? 0.0 : (double)most / (double)c->nnz;
     c->Htot = (int)row.size();
     if (c->Htot == 0) return GCP_OK;
     const size_t rep_bytes = (size_t)gcpk::kReplicas * c->Htot * c->Rp * 4;
@@ -853,18 +981,14 @@ int64_t gcp_num_params(const gcp_ctx *c) { return c ? c->total_rows * c->R : 0; 
 gcp_status gcp_set_factors(gcp_ctx *c, const float *A) {
     if (!c || !A) return fail(c, GCP_ERR_ARG, "NULL argument");
     DeviceGuard g(c->device);
-    GCP_CUDA(c, copy_rows(c->A, (size_t)c->Rp * 4, A, (size_t)c->R * 4, (size_t)c->R * 4,
-                                  (size_t)c->total_rows, c->st));
-    return refresh_bf16(c);
+    return rows_in(c, 0, c->total_rows, A);
 }
 
 gcp_status gcp_set_factor(gcp_ctx *c, int32_t mode, const float *A_mode) {
     if (!c || !A_mode) return fail(c, GCP_ERR_ARG, "NULL argument");
     if (mode < 0 || mode >= c->d) return fail(c, GCP_ERR_ARG, "mode out of range");
     DeviceGuard g(c->device);
-    GCP_CUDA(c, copy_rows(c->A + c->rowoff[mode] * c->Rp, (size_t)c->Rp * 4, A_mode, (size_t)c->R * 4,
-                                  (size_t)c->R * 4, (size_t)c->dims[mode], c->st));
-    return refresh_bf16(c);
+    return rows_in(c, c->rowoff[mode], c->dims[mode], A_mode);
 }
 
 gcp_status gcp_set_factor_list(gcp_ctx *c, const float *const *A_modes) {
@@ -872,17 +996,27 @@ gcp_status gcp_set_factor_list(gcp_ctx *c, const float *const *A_modes) {
     for (int k = 0; k < c->d; ++k)
         if (!A_modes[k]) return fail(c, GCP_ERR_ARG, "NULL factor pointer");
     DeviceGuard g(c->device);
-    for (int k = 0; k < c->d; ++k)
-        GCP_CUDA(c, copy_rows(c->A + c->rowoff[k] * c->Rp, (size_t)c->Rp * 4, A_modes[k], (size_t)c->R * 4,
-                                      (size_t)c->R * 4, (size_t)c->dims[k], c->st));
-    return refresh_bf16(c);
+    FactorSrc src{};
+    bool device = true;
+    for (int k = 0; k < c->d; ++k) {
+        device = device && kernel_writable(c, A_modes[k], sizeof(float));
+        src.A[k] = A_modes[k];
+        src.rowoff[k] = c->rowoff[k];
+    }
+    src.rowoff[c->d] = c->total_rows;
+    if (device) return stage_factors(c, src, 0, c->total_rows);
+    for (int k = 0; k < c->d; ++k) {
+        gcp_status s = rows_in(c, c->rowoff[k], c->dims[k], A_modes[k]);
+        if (s) return s;
+    }
+    return GCP_OK;
 }
 
 gcp_status gcp_get_factors(gcp_ctx *c, float *A_out) {
     if (!c || !A_out) return fail(c, GCP_ERR_ARG, "NULL argument");
     DeviceGuard g(c->device);
-    GCP_CUDA(c, copy_rows(A_out, (size_t)c->R * 4, c->A, (size_t)c->Rp * 4, (size_t)c->R * 4,
-                                  (size_t)c->total_rows, c->st));
+    gcp_status s = rows_out(c, c->A, 0, c->total_rows, A_out);
+    if (s) return s;
     return collect(c);
 }
 
@@ -971,13 +1105,7 @@ gcp_status gcp_grad_factors_async(gcp_ctx *c, const float *const *A_modes, uint6
     DeviceGuard g(c->device);
     gcp_status s = check_counts(c, p, q);
     if (s) return s;
-    const int64_t n = c->total_rows * c->Rp;
-    int log2Rp = 0;
-    while ((1 << log2Rp) < c->Rp) ++log2Rp;
-    const int64_t want = (n + 255) / 256;
-    k_stage_factors<<<(unsigned)(want < 8192 ? want : 8192), 256, 0, c->st>>>(
-        src, c->d, c->R, log2Rp, n, c->A, static_cast<__nv_bfloat16 *>(c->Abf));
-    GCP_CUDA(c, cudaGetLastError());
+    if ((s = stage_factors(c, src, 0, c->total_rows))) return s;
     Outputs out;
     out.G = G_out;
     out.dloss = dloss_out;
@@ -1019,7 +1147,7 @@ gcp_status gcp_grad_norm(gcp_ctx *c, double *norm_out) {
     const int nb = (int)std::max<int64_t>(1, std::min<int64_t>(want, 4 * (int64_t)c->max_blocks));
     // the loss partials are free once the gradient's loss is finished (stream order)
     k_sumsq_blocks<<<nb, 256, 0, c->st>>>(c->G, n, c->partials);
-    k_sumsq_finish<<<1, 32, 0, c->st>>>(c->partials, nb, c->dloss + 2, c->status);
+    k_sumsq_finish<<<1, 256, 0, c->st>>>(c->partials, nb, c->dloss + 2, c->status);
     GCP_CUDA(c, cudaGetLastError());
     GCP_CUDA(c, cudaMemcpyAsync(c->h_loss + 2, c->dloss + 2, sizeof(double), cudaMemcpyDeviceToHost, c->st));
     const gcp_status s = collect(c);  // synchronises

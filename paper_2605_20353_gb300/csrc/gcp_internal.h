@@ -149,6 +149,8 @@ cudaError_t launch_grad_finish(const GradOutSpec &p, cudaStream_t st);
 cudaError_t launch_mttkrp_nonfused(const FusedSpec &f, const int *hot_slot, bool bf16, int cols, int max_blocks,
                                    cudaStream_t st);
 cudaError_t launch_finish_loss(const LossSpec &l, cudaStream_t st);
+// Rows of Rp floats copied to rows of R (device memory).
+cudaError_t launch_unpad(const float *src, int Rp, int R, int64_t rows, float *out, cudaStream_t st);
 cudaError_t launch_clear(float *x, int64_t n, cudaStream_t st);  // n a multiple of 4, x 16-byte aligned
 cudaError_t launch_adam(int64_t n, int Rp, int R, float *A, float *B, float *C, const float *G, float lr,
                         float beta1, float beta2, float c1inv, float c2inv, float eps, float lower,
@@ -214,6 +216,10 @@ struct gcp_ctx {
     int32_t *nf_coord = nullptr;
     float *nf_val = nullptr;
     int64_t nf_cap = 0;
+
+    // rows of host arrays on their way in or out (padded ranks)
+    float *stage = nullptr;
+    int64_t stage_rows = 0;
 
     // gcp_fit: last accepted factors and moments
     float *bk_A = nullptr, *bk_B = nullptr, *bk_C = nullptr;

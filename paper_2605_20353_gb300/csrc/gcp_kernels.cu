@@ -94,12 +94,30 @@ __global__ void __launch_bounds__(kThreads) k_finish_loss(const LossSpec l) {
     finish_loss_block(l);
 }
 
+// Rows of Rp floats copied to rows of R, V columns per thread (V = 4 where R
+// and the address of `out` allow 16-byte stores), by the first `nblocks`
+// blocks; rows with a slot in `skip` (if given) are left out.
+template <int V>
+__device__ __forceinline__ void unpad_rows(const float *src, int Rp, int R, int64_t rows, float *out,
+                                           const int *__restrict__ skip, int nblocks) {
+    const unsigned units = (unsigned)(R / V);  // vectors or columns of a row
+    const int64_t n = rows * units;            // below 2^31
+    for (int64_t e = (int64_t)blockIdx.x * kThreads + threadIdx.x; e < n; e += (int64_t)nblocks * kThreads) {
+        const unsigned row = (unsigned)e / units, u = (unsigned)e - row * units;
+        if (skip && __ldg(skip + row) >= 0) continue;
+        const float *g = src + (int64_t)row * Rp + V * u;
+        if (V == 4)
+            reinterpret_cast<float4 *>(out)[e] = *reinterpret_cast<const float4 *>(g);
+        else
+            out[e] = *g;
+    }
+}
+
 // The epilogue of a gradient call after the fused pass, in one launch:
 //  - the last block finishes the FP64 loss (and hands it to the caller's
 //    device word or the pinned mirrors);
 //  - with a caller's array, the first `ncold` blocks copy the rows of G that
-//    have no replicas into its rows of R columns, V columns per thread (V = 4
-//    where R and the array's address allow 16-byte stores);
+//    have no replicas into its rows of R columns (unpad_rows);
 //  - the blocks between take the quads of hot rows, one per group of NREP / 4
 //    lanes: all replica quads of a hot quad are in flight at once
 //    (gcpe::hot_quad_sum, which clears them for the next call), and the
@@ -154,17 +172,15 @@ __global__ void __launch_bounds__(kThreads) k_grad_finish(const GradOutSpec P, i
             return;
         }
     }
-    const unsigned units = (unsigned)(P.R / V);  // vectors or columns of a row
-    const int64_t n = P.rows * units;            // below 2^31
-    for (int64_t e = (int64_t)blockIdx.x * kThreads + threadIdx.x; e < n; e += (int64_t)ncold * kThreads) {
-        const unsigned row = (unsigned)e / units, u = (unsigned)e - row * units;
-        if (NREP > 0 && __ldg(P.hot_slot + row) >= 0) continue;  // the hot blocks' rows
-        const float *g = P.G + (int64_t)row * P.Rp + V * u;
-        if (V == 4)
-            reinterpret_cast<float4 *>(P.out)[e] = *reinterpret_cast<const float4 *>(g);
-        else
-            P.out[e] = *g;
-    }
+    unpad_rows<V>(P.G, P.Rp, P.R, P.rows, P.out, NREP > 0 ? P.hot_slot : nullptr, ncold);  // not the hot blocks' rows
+}
+
+// The same for a plain copy (factors out).
+template <int V>
+__global__ void __launch_bounds__(kThreads) k_unpad(const float *src, int Rp, int R, int64_t rows, float *out) {
+    grid_wait();
+    grid_trigger();
+    unpad_rows<V>(src, Rp, R, rows, out, nullptr, gridDim.x);
 }
 
 // ------------------------------------------------------------- sampling
@@ -565,6 +581,12 @@ cudaError_t launch_grad_finish(const GradOutSpec &p, cudaStream_t st) {
 
 cudaError_t launch_finish_loss(const LossSpec &l, cudaStream_t st) {
     return launch_dependent(k_finish_loss, 1, kThreads, 0, st, l);
+}
+
+cudaError_t launch_unpad(const float *src, int Rp, int R, int64_t rows, float *out, cudaStream_t st) {
+    if (R % 4 == 0 && (reinterpret_cast<uintptr_t>(out) & 15) == 0)
+        return launch_dependent(k_unpad<4>, elementwise_blocks(rows * (R / 4)), kThreads, 0, st, src, Rp, R, rows, out);
+    return launch_dependent(k_unpad<1>, elementwise_blocks(rows * R), kThreads, 0, st, src, Rp, R, rows, out);
 }
 
 // x = 0 before a gradient pass, as a kernel and not a memset so that the pass

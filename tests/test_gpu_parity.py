@@ -1001,3 +1001,59 @@ def test_deterministic_mttkrp_digit_widths_and_long_runs(env, dims, R, dtype):
         for m, (a, b) in enumerate(zip(split(Gg, dims, R), Go)):
             assert rel_err(a, b) <= TOL_FP32, (p, q, m, rel_err(a, b))
     ctx.close()
+
+
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("dims,R", [([40, 30, 20], 6), ([40, 30, 20], 16), ([2600, 700, 90], 7), ([2600, 700, 90], 20),
+                                    ([2600, 700, 90], 32), ([2600000, 700, 90], 3)])
+def test_factors_in_and_out_by_every_route(env, dims, R, dtype):
+    """Factors set from and read into device, pinned and pageable arrays, on a
+    16-byte boundary and 4 bytes past one, all at once, mode by mode and as a
+    list, with and without padding, few rows (strided copy), many (staged) and
+    more than the staging holds at once: every entry comes back, nothing
+    outside is written, the BF16 copy follows (the loss equals that of a
+    context that was given the same factors another way), and a step after it
+    sees them."""
+    gcp, torch = env
+    coords, vals, factors = problem(dims, 500, R, "poisson", 1101)
+    flat = np.concatenate([a.ravel() for a in factors])
+    n, lib = flat.size, gcp.load()
+    ref = gcp.gcp_create(dims, coords, vals, R, "poisson", seed=1102, dtype=dtype)
+    ref.set_factors(factors)
+    L = ref.loss_value(1, 400, 500)
+    ref.close()
+    ctx = gcp.gcp_create(dims, coords, vals, R, "poisson", seed=1102, dtype=dtype)
+
+    def array(kind, shift, fill):
+        if kind == "device":
+            t = torch.full((n + 8,), float(fill), device="cuda")
+        else:
+            t = torch.full((n + 8,), float(fill), pin_memory=kind == "pinned")
+        return t, t[shift:shift + n]
+
+    zero = np.zeros(n, np.float32)
+    for kind in ("device", "pinned", "pageable"):
+        for shift in (0, 1):
+            ctx.set_factors(zero)
+            whole, part = array(kind, shift, 0.0)
+            part.copy_(torch.from_numpy(flat))
+            if shift == 0:
+                assert lib.gcp_set_factors(ctx.handle, part.data_ptr()) == 0
+            else:  # mode by mode
+                o = 0
+                for k, I in enumerate(dims):
+                    assert lib.gcp_set_factor(ctx.handle, k, part.data_ptr() + 4 * o) == 0
+                    o += I * R
+            assert ctx.loss_value(1, 400, 500) == L, (kind, shift)
+            whole, part = array(kind, shift, 7.0)
+            assert lib.gcp_get_factors(ctx.handle, part.data_ptr()) == 0
+            torch.cuda.synchronize()
+            assert np.array_equal(part.cpu().numpy(), flat), (kind, shift)
+            assert bool((whole[:shift] == 7.0).all()) and bool((whole[shift + n:] == 7.0).all())
+    ctx.set_factors(zero)
+    ctx.set_factors([torch.from_numpy(a).cuda() for a in factors])
+    assert ctx.loss_value(1, 400, 500) == L
+    ctx.set_factors(zero)
+    ctx.set_factors([torch.from_numpy(a).cuda() if k else a for k, a in enumerate(factors)])  # mixed
+    assert ctx.loss_value(1, 400, 500) == L
+    ctx.close()

@@ -375,7 +375,8 @@ gcp_status gcp_batch_server_step(gcp_batch *batch, const gcp_adam_params *prm, i
  * fixed at start-up, such as a host framework that owns every allocation
  * through its own pool, or a long-running service that must not grow its
  * footprint.  The caller passes every input and output; the only scratch
- * (one loss partial per thread block) is a file-scope device array
+ * (one loss partial per thread block, and replicas of the gradient rows that
+ * most of a long list meets in) is a file-scope device array
  * of the library, 128 KB, held by every GPU that loads the library until the
  * process exits.  No cudaMalloc, cudaFree or allocating library routine is
  * called.

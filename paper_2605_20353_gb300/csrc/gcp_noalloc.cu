@@ -6,10 +6,13 @@
 // allocation through its own pool, or a long-running service that must not
 // grow its footprint after start-up).  This entry point takes all of its
 // inputs and outputs from the caller and keeps its only scratch -- one loss
-// partial per block -- in the file-scope device array below.  That array is
-// part of the library image: every GPU that loads the library holds it
-// (8192 slots x 16 bytes = 128 KB) until the
-// process exits.
+// partial per block and a few replicas of the hottest gradient rows -- in the
+// file-scope device array below.  That array is part of the library image:
+// every GPU that loads the library holds it (128 KB) until the process exits.
+//
+// Three launches: the gradient cleared and the hot rows of the list found
+// (k_na_setup), the pass over the samples (k_na_grad), the replicas folded and
+// the loss summed (k_na_finish).
 #include <algorithm>
 #include <mutex>
 
@@ -23,21 +26,112 @@ namespace {
 
 constexpr int kNaThreads = 256;
 constexpr int kNaWarps = kNaThreads / 32;
-constexpr int kNaMaxBlocks = 8192;
+constexpr int kNaMaxBlocks = 2048;
 constexpr int kNaMaxDevices = 64;
+constexpr int kNaHot = 32;               // hot rows of a mode at most
+constexpr int kNaRepFloats = 23 * 1024;  // replica rows, shared out evenly over the modes
 
-// Per-block (loss partial, skipped-sample count), shared by every call on a
-// device.  Each call writes the slots of the blocks it launches before it
-// reads them, so nothing has to start at zero; calls that overlap on the
-// GPU race on these slots.
-__device__ __align__(256) double2 g_na_partials[kNaMaxBlocks];
+// The hot rows of one mode: nrep replicas of n rows each, n | nrep << 8 in one
+// word (read once by whoever uses it, so that the two always belong together).
+struct NaHot {
+    int n_nrep;
+    int row[kNaHot];
+};
+
+// Everything a call keeps on the device, shared by every call on it: loss
+// partials (block loss, skipped samples), the hot rows, their replicas.  Each
+// call writes what it reads later, so nothing has to start at zero; calls
+// that overlap on the GPU race on it.
+struct NaScratch {
+    double2 partials[kNaMaxBlocks];
+    NaHot hot[GCP_MAX_NDIM];
+    alignas(16) float rep[kNaRepFloats];
+};
+static_assert(sizeof(NaScratch) <= 128 * 1024, "the documented size of the scratch");
+__device__ __align__(256) unsigned char g_na_scratch[128 * 1024];
 
 struct NaShape {
     int R;
     int log2L;                       // lanes per sample
+    int d;
+    int hot;                         // whether the list is searched for hot rows
+    int tile;                        // samples per warp tile (fused_tile)
+    int64_t rows;
     int64_t dims[GCP_MAX_NDIM];
     int64_t rowoff[GCP_MAX_NDIM];
 };
+
+// Floats of a replica row, and of one mode's share of the replicas.
+__host__ __device__ constexpr int na_row_floats(int R) { return (R + 3) & ~3; }
+__host__ __device__ constexpr int na_mode_floats(int d) { return (kNaRepFloats / d) & ~3; }
+
+// Blocks k < d (if sh.hot): the hot rows of mode k.  kNaProbe samples spread
+// over the list are counted in a hash table; the rows counted at least T times
+// are hot, T the smallest of 8, 16, 32, ... with which there are at most
+// kNaHot of them and four replicas of each fit the mode's share.  (A row that
+// takes 1/256 of the samples is counted 8 times.)  The mode's replicas are
+// cleared.  The other blocks clear G.
+constexpr int kNaProbe = 2048, kNaTable = 4096;
+
+__global__ void __launch_bounds__(kNaThreads) k_na_setup(const NaShape sh, int64_t n, const int32_t *__restrict__ idx,
+                                                        float *__restrict__ G, NaScratch *__restrict__ S) {
+    const int searchers = sh.hot ? sh.d : 0;
+    if ((int)blockIdx.x >= searchers) {
+        const int64_t total = sh.rows * sh.R, step = (int64_t)(gridDim.x - searchers) * kNaThreads;
+        const int64_t first = (int64_t)(blockIdx.x - searchers) * kNaThreads + threadIdx.x;
+        if ((reinterpret_cast<uintptr_t>(G) & 15) == 0) {
+            for (int64_t e = first; e < (total >> 2); e += step)
+                reinterpret_cast<float4 *>(G)[e] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+            if (first < (total & 3)) G[(total & ~(int64_t)3) + first] = 0.0f;
+        } else {
+            for (int64_t e = first; e < total; e += step) G[e] = 0.0f;
+        }
+        return;
+    }
+    const int k = blockIdx.x;
+    __shared__ int key[kNaTable];
+    __shared__ unsigned count[kNaTable];
+    __shared__ int over[8], slots;
+    for (int i = threadIdx.x; i < kNaTable; i += kNaThreads) {
+        key[i] = -1;
+        count[i] = 0;
+    }
+    if (threadIdx.x < 8) over[threadIdx.x] = 0;
+    if (threadIdx.x == 0) slots = 0;
+    __syncthreads();
+    for (int i = threadIdx.x; i < kNaProbe; i += kNaThreads) {
+        const int r = __ldg(idx + (n * i / kNaProbe) * sh.d + k);
+        if (r < 0 || r >= sh.dims[k]) continue;
+        unsigned h = ((unsigned)r * 2654435769u) >> 20;
+        for (int probe = 0; probe < 32; ++probe, h = (h + 1) & (kNaTable - 1)) {  // at most half full
+            const int was = atomicCAS(&key[h], -1, r);
+            if (was == -1 || was == r) {
+                atomicAdd(&count[h], 1u);
+                break;
+            }
+        }
+    }
+    __syncthreads();
+    for (int i = threadIdx.x; i < kNaTable; i += kNaThreads)
+        for (int t = 0; t < 8; ++t)
+            if (count[i] >= (8u << t)) atomicAdd(&over[t], 1);
+    __syncthreads();
+    const int rf = na_row_floats(sh.R), share = na_mode_floats(sh.d);
+    int t = 0;
+    while (t < 7 && (over[t] > kNaHot || 4 * over[t] * rf > share)) ++t;
+    const int hot = over[t] <= kNaHot && 4 * over[t] * rf <= share ? over[t] : 0;
+    int nrep = 0;
+    if (hot) {
+        nrep = 4;
+        while (nrep < 32 && 2 * nrep * hot * rf <= share) nrep *= 2;
+        for (int i = threadIdx.x; i < kNaTable; i += kNaThreads)
+            if (count[i] >= (8u << t)) S->hot[k].row[atomicAdd(&slots, 1)] = key[i];
+    }
+    if (threadIdx.x == 0) {
+        S->hot[k].n_nrep = hot | nrep << 8;
+    }
+    for (int i = threadIdx.x; i < hot * nrep * rf; i += kNaThreads) S->rep[k * share + i] = 0.0f;
+}
 
 // V consecutive columns of a row of A, or added to a row of G: one 16-byte
 // vector (V = 4) or a scalar (V = 1).
@@ -56,7 +150,7 @@ __device__ __forceinline__ void na_add(float *p, const float *c) {
         atomicAdd(p, c[0]);
 }
 
-// Sampled gradient of a sample list.  A warp takes tiles of 32 consecutive
+// Sampled gradient of a sample list.  A warp takes tiles of up to 32 consecutive
 // samples: lane l reads sample l's coordinates, value and weight (the next
 // tile's are in flight while this one is evaluated), then groups of L lanes
 // take the tile's samples in turn, their row offsets, values and weights
@@ -64,17 +158,40 @@ __device__ __forceinline__ void na_add(float *p, const float *c) {
 // V (g + L q) + V - 1 for q < NQ; those past the rank are skipped, so rows
 // need no padding.  Each lane keeps its own sample's loss and adds it in
 // FP64 once per tile (three FP64 instructions per 32 samples).
+// Reductions of a hot row go to one of its replicas (chosen by warp), folded
+// afterwards; a lane looks its sample's rows up in a small table in shared
+// memory.
 // Bound by the row traffic through L2 (d rows gathered, d rows reduced per
-// sample) and, on skewed data, by the reductions that meet in one row: the
-// entry point has no scratch for replicas.  2^18 samples of the 2000 x 1500
+// sample).  2^18 samples of the 2000 x 1500
 // x 1000 x 200 Zipf tensor at rank 32, drawn with gcp_sample and passed
-// here: 156 us a pass, against 745 us with one warp per sample walking 256
-// samples one after another on 128 blocks.
+// here: 106 us a pass, this kernel 42; 156 us with every reduction added to G itself (the ones
+// that meet in one row are applied one after another, about 4.7 ns each);
+// 745 us with one warp per sample walking 256 samples one after another on
+// 128 blocks.
 template <int D, int V, int NQ>
-__global__ void __launch_bounds__(kNaThreads, (D <= 4 ? 3 : 1))
+__global__ void __launch_bounds__(kNaThreads, (D <= 4 ? 3 : 2))
     k_na_grad(const NaShape sh, int loss, int64_t n, const int32_t *__restrict__ idx, const float *__restrict__ x,
-              const float *__restrict__ w, const float *__restrict__ A, float *__restrict__ G, double2 *partials) {
+              const float *__restrict__ w, const float *__restrict__ A, float *__restrict__ G,
+              NaScratch *__restrict__ S) {
     constexpr int C = V * NQ;  // columns per lane
+    constexpr int kBuckets = 64;
+    __shared__ int s_row[D][kBuckets];             // -1: empty
+    __shared__ unsigned char s_slot[D][kBuckets];
+    __shared__ int s_hot[D];
+    if (sh.hot) {
+        if (threadIdx.x < D) s_hot[threadIdx.x] = S->hot[threadIdx.x].n_nrep;
+        for (int i = threadIdx.x; i < D * kBuckets; i += kNaThreads) (&s_row[0][0])[i] = -1;
+        __syncthreads();
+        for (int i = threadIdx.x; i < D * kNaHot; i += kNaThreads) {
+            const int k = i / kNaHot, j = i % kNaHot;
+            if (j >= (s_hot[k] & 255)) continue;
+            const int r = S->hot[k].row[j];
+            unsigned h = ((unsigned)r * 2654435769u) >> 26;
+            while (atomicCAS(&s_row[k][h], -1, r) != -1) h = (h + 1) & (kBuckets - 1);  // at most half full
+            s_slot[k][h] = (unsigned char)j;
+        }
+        __syncthreads();
+    }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     const int L = 1 << sh.log2L;
     const int glane = lane & (L - 1), grp = lane >> sh.log2L, ngrp = 32 >> sh.log2L;
@@ -85,13 +202,22 @@ __global__ void __launch_bounds__(kNaThreads, (D <= 4 ? 3 : 1))
         col[q] = V * (glane + L * q);
         on[q] = col[q] < sh.R;
     }
-    const int64_t ntiles = (n + 31) >> 5;
+    const int TS = sh.tile;
+    const int64_t ntiles = (n + TS - 1) / TS;
     const int64_t nwarps = (int64_t)gridDim.x * kNaWarps;
+    const int rf = na_row_floats(sh.R);
+    int rep[D];  // where this warp's replicas of a mode's hot rows start
+#pragma unroll
+    for (int k = 0; k < D; ++k) {
+        rep[k] = k * na_mode_floats(D);
+        if (sh.hot && s_hot[k])
+            rep[k] += (((int)blockIdx.x * kNaWarps + warp) & ((s_hot[k] >> 8) - 1)) * (s_hot[k] & 255) * rf;
+    }
     int32_t ni[D];  // the next tile's sample of this lane
     float nx = 0.0f, nw = 0.0f;
     auto fetch = [&](int64_t tile) {
-        const int64_t s = (tile << 5) + lane;
-        if (s < n) {
+        const int64_t s = tile * TS + lane;
+        if (lane < TS && s < n) {
 #pragma unroll
             for (int k = 0; k < D; ++k) ni[k] = __ldg(idx + s * D + k);
             nx = __ldg(x + s);
@@ -114,16 +240,31 @@ __global__ void __launch_bounds__(kNaThreads, (D <= 4 ? 3 : 1))
             row[k] = (sh.rowoff[k] + ni[k]) * sh.R;
         }
         const float myx = nx, myw = nw;
-        const bool in = (tile << 5) + lane < n;
+        const bool in = lane < TS && tile * TS + lane < n;
         skipped += in && !ok;  // out-of-range coordinates: the sample is skipped and counted
         const unsigned okmask = __ballot_sync(0xFFFFFFFFu, in && ok);
+        unsigned hot[(D + 3) / 4];  // per mode a byte: the row's hot slot, or 255
+#pragma unroll
+        for (int k = 0; k < D; ++k) {
+            unsigned slot = 255u;
+            if (sh.hot)
+                for (unsigned h = ((unsigned)ni[k] * 2654435769u) >> 26;; h = (h + 1) & (kBuckets - 1)) {
+                    const int r = s_row[k][h];  // an empty bucket ends the search
+                    if (r == ni[k]) slot = s_slot[k][h];
+                    if (r == ni[k] || r == -1) break;
+                }
+            hot[k / 4] = (k % 4 ? hot[k / 4] : 0u) | slot << (8 * (k % 4));
+        }
         fetch(tile + nwarps);
         float myf = 0.0f;
-        for (int it = 0; it < L; ++it) {
+        for (int it = 0; it * ngrp < TS; ++it) {
             const int src = it * ngrp + grp;
             const bool live = (okmask >> src) & 1u;  // uniform within the group
             const float xs = __shfl_sync(0xFFFFFFFFu, myx, src), ws = __shfl_sync(0xFFFFFFFFu, myw, src);
             int64_t off[D];
+            unsigned hs[(D + 3) / 4];
+#pragma unroll
+            for (int i = 0; i < (D + 3) / 4; ++i) hs[i] = __shfl_sync(0xFFFFFFFFu, hot[i], src);
             float a[D][C];
 #pragma unroll
             for (int k = 0; k < D; ++k) {
@@ -159,13 +300,15 @@ __global__ void __launch_bounds__(kNaThreads, (D <= 4 ? 3 : 1))
             for (int v = 0; v < C; ++v) pre[v] = ws * df;
 #pragma unroll
             for (int k = 0; k < D; ++k) {
+                const int slot = (int)((hs[k / 4] >> (8 * (k % 4))) & 255u);
+                float *const g = slot == 255 ? G + off[k] : S->rep + rep[k] + slot * rf;
 #pragma unroll
                 for (int q = 0; q < NQ; ++q) {
                     if (!on[q]) continue;
                     float c[V];
 #pragma unroll
                     for (int v = 0; v < V; ++v) c[v] = pre[V * q + v] * suf[k][V * q + v];
-                    na_add<V>(G + off[k] + col[q], c);
+                    na_add<V>(g + col[q], c);
                 }
 #pragma unroll
                 for (int v = 0; v < C; ++v) pre[v] *= a[k][v];
@@ -190,31 +333,49 @@ __global__ void __launch_bounds__(kNaThreads, (D <= 4 ? 3 : 1))
             t.x += red[i].x;
             t.y += red[i].y;
         }
-        partials[blockIdx.x] = t;
+        S->partials[blockIdx.x] = t;
     }
 }
 
-// Fixed-order sum of the block partials: loss_out[0] = loss,
-// loss_out[1] = samples skipped for out-of-range coordinates.
-__global__ void __launch_bounds__(kNaThreads) k_na_sum(const double2 *partials, int nblocks, double *loss_out) {
-    __shared__ double2 sh[kNaThreads];
+// The last block: fixed-order sum of the block partials, loss_out[0] = loss,
+// loss_out[1] = samples skipped for out-of-range coordinates.  The others, one
+// per mode and hot row: the row's replicas added to G.
+__global__ void __launch_bounds__(kNaThreads) k_na_finish(const NaShape sh, float *__restrict__ G, NaScratch *S,
+                                                         int nblocks, double *loss_out) {
+    if (blockIdx.x < gridDim.x - 1) {
+        const int k = blockIdx.x / kNaHot, j = blockIdx.x % kNaHot;
+        const int word = S->hot[k].n_nrep, hot = word & 255, nrep = word >> 8, rf = na_row_floats(sh.R);
+        const int c = threadIdx.x;
+        if (j >= hot || c >= sh.R) return;
+        const float *p = S->rep + k * na_mode_floats(sh.d) + j * rf + c;
+        float t = 0.0f;
+        for (int r = 0; r < nrep; r += 4) {  // 4, 8, 16 or 32
+            float v[4];
+#pragma unroll
+            for (int u = 0; u < 4; ++u) v[u] = p[(r + u) * hot * rf];
+            t += (v[0] + v[1]) + (v[2] + v[3]);
+        }
+        G[(sh.rowoff[k] + S->hot[k].row[j]) * sh.R + c] += t;
+        return;
+    }
+    __shared__ double2 red[kNaThreads];
     double2 t = make_double2(0.0, 0.0);
     for (int b = threadIdx.x; b < nblocks; b += kNaThreads) {
-        t.x += partials[b].x;
-        t.y += partials[b].y;
+        t.x += S->partials[b].x;
+        t.y += S->partials[b].y;
     }
-    sh[threadIdx.x] = t;
+    red[threadIdx.x] = t;
     __syncthreads();
     for (int h = kNaThreads / 2; h > 0; h >>= 1) {
         if (threadIdx.x < h) {
-            sh[threadIdx.x].x += sh[threadIdx.x + h].x;
-            sh[threadIdx.x].y += sh[threadIdx.x + h].y;
+            red[threadIdx.x].x += red[threadIdx.x + h].x;
+            red[threadIdx.x].y += red[threadIdx.x + h].y;
         }
         __syncthreads();
     }
     if (threadIdx.x == 0) {
-        loss_out[0] = sh[0].x;
-        loss_out[1] = sh[0].y;
+        loss_out[0] = red[0].x;
+        loss_out[1] = red[0].y;
     }
 }
 
@@ -236,7 +397,7 @@ NaPlan na_plan(int R, bool aligned) {
 }
 
 using NaKernel = void (*)(NaShape, int, int64_t, const int32_t *, const float *, const float *, const float *, float *,
-                          double2 *);
+                          NaScratch *);
 
 template <int D>
 NaKernel na_kernel_d(const NaPlan &p) {
@@ -256,14 +417,14 @@ NaKernel na_kernel(int d, const NaPlan &p) {
     }
 }
 
-// Device address of g_na_partials, looked up once per device.  In host
+// Device address of g_na_scratch, looked up once per device.  In host
 // code the array's name is only a host-side stand-in, so the kernel must be
 // given the address that cudaGetSymbolAddress returns for the current
 // device.
 std::mutex g_na_mutex;
-double2 *g_na_addr[kNaMaxDevices] = {nullptr};
+NaScratch *g_na_addr[kNaMaxDevices] = {nullptr};
 
-cudaError_t scratch_for_current_device(double2 **out) {
+cudaError_t scratch_for_current_device(NaScratch **out) {
     int dev = 0;
     cudaError_t e = cudaGetDevice(&dev);
     if (e != cudaSuccess) return e;
@@ -271,9 +432,9 @@ cudaError_t scratch_for_current_device(double2 **out) {
     std::lock_guard<std::mutex> lock(g_na_mutex);
     if (!g_na_addr[dev]) {
         void *p = nullptr;
-        e = cudaGetSymbolAddress(&p, g_na_partials);
+        e = cudaGetSymbolAddress(&p, g_na_scratch);
         if (e != cudaSuccess) return e;
-        g_na_addr[dev] = static_cast<double2 *>(p);
+        g_na_addr[dev] = static_cast<NaScratch *>(p);
     }
     *out = g_na_addr[dev];
     return cudaSuccess;
@@ -310,12 +471,19 @@ extern "C" gcp_status gcp_grad_samples_noalloc(int32_t ndim, const int64_t *dims
         sh.rowoff[k] = rows;
         rows += dims[k];
     }
-    double2 *scratch = nullptr;
+    NaScratch *scratch = nullptr;
     cudaError_t e = scratch_for_current_device(&scratch);
     if (e != cudaSuccess) return na_fail(GCP_ERR_CUDA, cudaGetErrorString(e));
     cudaStream_t st = static_cast<cudaStream_t>(stream);
-    if ((e = cudaMemsetAsync(G, 0, (size_t)rows * rank * sizeof(float), st)) != cudaSuccess)
-        return na_fail(GCP_ERR_CUDA, cudaGetErrorString(e));
+    // A hot row needs that many reductions in one line to matter: 2^14
+    // samples of which a fifth meet in one row are 15 us, less than two
+    // launches; from there on the list is searched.
+    sh.d = ndim;
+    sh.rows = rows;
+    sh.hot = nsamples >= 1 << 14;
+    const int64_t clear = (rows * rank / 4 + kNaThreads - 1) / kNaThreads;
+    k_na_setup<<<(sh.hot ? ndim : 0) + (int)std::max<int64_t>(1, std::min<int64_t>(clear, 1216)), kNaThreads, 0, st>>>(
+        sh, nsamples, idx, G, scratch);
     int nblocks = 0;
     if (nsamples > 0) {
         // a grid of at most the blocks that fit on the GPU at once; fewer
@@ -326,11 +494,13 @@ extern "C" gcp_status gcp_grad_samples_noalloc(int32_t ndim, const int64_t *dims
             (e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev)) != cudaSuccess ||
             (e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, k, kNaThreads, 0)) != cudaSuccess)
             return na_fail(GCP_ERR_CUDA, cudaGetErrorString(e));
-        const int64_t want = ((nsamples + 31) / 32 + kNaWarps - 1) / kNaWarps;
-        nblocks = (int)std::min<int64_t>(want, std::min<int64_t>((int64_t)std::max(1, per_sm) * sms, kNaMaxBlocks));
+        const int most = std::min(std::max(1, per_sm) * sms, kNaMaxBlocks);
+        sh.tile = gcpk::fused_tile(nsamples, plan.log2L, most);
+        const int64_t ntiles = (nsamples + sh.tile - 1) / sh.tile;
+        nblocks = (int)std::min<int64_t>((ntiles + kNaWarps - 1) / kNaWarps, most);
         k<<<nblocks, kNaThreads, 0, st>>>(sh, loss, nsamples, idx, x, w, A, G, scratch);
     }
-    k_na_sum<<<1, kNaThreads, 0, st>>>(scratch, nblocks, loss_out);
+    k_na_finish<<<(sh.hot ? ndim * kNaHot : 0) + 1, kNaThreads, 0, st>>>(sh, G, scratch, nblocks, loss_out);
     if ((e = cudaGetLastError()) != cudaSuccess) return na_fail(GCP_ERR_CUDA, cudaGetErrorString(e));
     return GCP_OK;
 }

@@ -153,3 +153,42 @@ def test_noalloc_ranks_alignments_and_ragged_counts(env, ndim, R, shift):
         assert rel_err(G.cpu().numpy(), np.concatenate([g.ravel() for g in Go])) <= TOL, n
         rest = torch.cat([buf[:shift], buf[shift + flat.size:]])
         assert bool((rest == 7.0).all())
+
+
+@pytest.mark.parametrize("dims,R,shift", [([200, 3000, 50, 700], 32, 0), ([7, 900, 40000], 128, 0), ([7, 900, 40000], 30, 1),
+                                          ([3, 5, 2000, 60, 4, 9], 12, 0), ([31, 2, 100, 40, 50, 6, 7, 8], 5, 0),
+                                          ([50000, 60000], 100, 0)])
+def test_noalloc_skewed_lists_use_and_clear_the_replicas(env, dims, R, shift):
+    """Long lists whose samples meet in few rows (replicas of the hottest
+    rows, as many as the scratch holds at this rank and order), then a short
+    and a uniform one on the same scratch, with some coordinates out of range:
+    loss, skipped count and gradient against the FP64 oracle each time."""
+    import oracle
+
+    gcp, torch = env
+    rng = np.random.default_rng(1200 + R)
+    factors = synth.factors_uniform(dims, R, 1201, lo=0.1, hi=1.0)
+    flat = np.concatenate([a.ravel() for a in factors])
+    A = torch.zeros(flat.size + 4, device="cuda")[shift:shift + flat.size]
+    A.copy_(torch.from_numpy(flat))
+    for n, zipf in ((40000, True), (16384, True), (500, True), (30001, False)):
+        cols = []
+        for I in dims:
+            c = rng.zipf(1.3, n) - 1 if zipf else rng.integers(0, I, n)
+            cols.append(np.where(c < I, c, rng.integers(0, I, n)))
+        idx = np.stack(cols, 1).astype(np.int32)
+        bad = rng.choice(n, 7, replace=False)
+        idx[bad, 0] = [-1, -1, dims[0], -5, 2**31 - 1, -2**31, dims[0] + 1]
+        x = rng.poisson(2.0, n).astype(np.float32)
+        w = rng.uniform(0.5, 2.0, n).astype(np.float32)
+        G = torch.full((flat.size + 4,), float("nan"), device="cuda")[shift:shift + flat.size]
+        out = torch.full((2,), float("nan"), dtype=torch.float64, device="cuda")
+        gcp.gcp_grad_samples_noalloc(dims, R, "poisson", torch.from_numpy(idx).cuda(), torch.from_numpy(x).cuda(),
+                                     torch.from_numpy(w).cuda(), A, G, out)
+        L, skipped = out.cpu().numpy()
+        keep = np.setdiff1d(np.arange(n), bad)
+        Lo, Go = oracle.sampled_loss_grad(dims, factors, "poisson", idx[keep], x[keep].astype(np.float64),
+                                          w[keep].astype(np.float64))
+        assert skipped == len(bad)
+        assert abs(L - Lo) <= TOL * abs(Lo), (n, L, Lo)
+        assert rel_err(G.cpu().numpy(), np.concatenate([g.ravel() for g in Go])) <= TOL, n

@@ -287,11 +287,17 @@ __global__ void k_adam(int64_t n, int Rp, int R, float *__restrict__ A, float *_
 // The streaming blocks run at the copy rate on models larger than L2; the
 // hot quads cost one memory round trip each instead of one per group of
 // replica loads.
-// Quads per streaming thread and iteration.  One quad per thread at full
-// occupancy streamed the HBM-resident epilogue (121.6M parameters) at
-// 6.0 TB/s; two or four per thread, with fewer resident warps, at 3.6 and
-// 4.1 TB/s.
+// Quads per streaming thread and iteration, and waves of resident streaming
+// blocks at most.  One quad per thread streamed the HBM-resident epilogue
+// (121.6M parameters) at 6.0 TB/s; two or four per thread, with fewer
+// resident warps, at 3.6 and 4.1 TB/s.  With one wave of blocks striding over
+// the arrays the rate hangs on how the eight streams fall on the memory
+// banks: a step of that model took 2.77, 2.31, 2.22, 2.27 and 2.24 ms on 304,
+// 608, 700, 760 and 912 blocks, and 4.2 ms when the compiler chose a few
+// registers more; with 13 to 40 waves, which the hardware hands out as blocks
+// finish, 2.14 ms (the epilogue at 6.6 TB/s).
 constexpr int kPostUnroll = 1;
+constexpr int kPostWaves = 16;
 
 template <int NREP>
 __global__ void __launch_bounds__(kThreads) k_post_step(PostSpec P, int ncold) {
@@ -385,7 +391,8 @@ static cudaError_t launch_post_step_r(const PostSpec &p, cudaStream_t st) {
         resident = (per_sm < 1 ? 1 : per_sm) * num_sms();
     }
     const int64_t want = ((p.n >> 2) + (int64_t)kThreads * kPostUnroll - 1) / ((int64_t)kThreads * kPostUnroll);
-    const int ncold = (int)(want < 1 ? 1 : (want > resident ? resident : want));
+    const int64_t cap = (int64_t)kPostWaves * resident;
+    const int ncold = (int)(want < 1 ? 1 : (want > cap ? cap : want));
     int nhot = 0;
     if constexpr (NREP > 0) {
         constexpr int per = kThreads / gcpe::hot_lanes<NREP>();  // hot quads of a block
@@ -605,7 +612,9 @@ cudaError_t launch_clear(float *x, int64_t n, cudaStream_t st) {
 cudaError_t launch_adam(int64_t n, int Rp, int R, float *A, float *B, float *C, const float *G, float lr,
                         float beta1, float beta2, float c1inv, float c2inv, float eps, float lower, void *Abf,
                         cudaStream_t st) {
-    k_adam<<<elementwise_blocks(n), kThreads, 0, st>>>(n, Rp, R, A, B, C, G, lr, beta1, beta2, c1inv, c2inv, eps,
+    // many blocks per SM, as in k_post_step: 121.6M parameters 540 -> 496 us
+    const int64_t want = ((n >> 2) + kThreads - 1) / kThreads, cap = (int64_t)num_sms() * 64;
+    k_adam<<<(int)(want < 1 ? 1 : (want < cap ? want : cap)), kThreads, 0, st>>>(n, Rp, R, A, B, C, G, lr, beta1, beta2, c1inv, c2inv, eps,
                                                         lower, static_cast<__nv_bfloat16 *>(Abf));
     return cudaGetLastError();
 }

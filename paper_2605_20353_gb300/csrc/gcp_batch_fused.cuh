@@ -36,7 +36,7 @@ template <int D>
 __device__ __forceinline__ uint64_t linear_b(const gcpk::SampleSpec &S, const int32_t (&idx)[D]) {
     uint64_t L = 0;
 #pragma unroll
-    for (int k = 0; k < D; ++k) L += (uint64_t)idx[k] * S.stride[k];
+    for (int k = 0; k < D; ++k) L += (uint64_t)(uint32_t)idx[k] * S.stride[k];
     return L;
 }
 
@@ -131,14 +131,14 @@ __global__ void __launch_bounds__(kThreads, gcpk::fused_min_blocks(D, COLS)) k_b
             const int s = (int)us;
             int32_t *slot = s_slot[st][warp][pos];
             if (s < p) {
-                const U64x4 w = philox4x64_10((uint64_t)s, 0, P.s.iter, 0, P.s.seed, kStreamNonzero);
+                const U64x4 w = philox4x64_10((uint64_t)(uint32_t)s, 0, P.s.iter, 0, P.s.seed, kStreamNonzero);
                 const int32_t *rec = P.s.rec + map_range(w.v[0], (uint64_t)P.s.nnz) * SW;
 #pragma unroll
                 for (int v = 0; v < SW / 4; ++v) cp_async16(slot + 4 * v, rec + 4 * v);
                 continue;
             }
             int32_t idx[D];
-            draw_tuple_b<D>(P.s, semi ? kStreamSemiZero : kStreamZero, (uint64_t)(s - p), 0, idx);
+            draw_tuple_b<D>(P.s, semi ? kStreamSemiZero : kStreamZero, (uint64_t)(uint32_t)(s - p), 0, idx);
 #pragma unroll
             for (int k = 0; k < D; ++k) slot[k] = idx[k];
             slot[D] = 0;
@@ -165,7 +165,7 @@ __global__ void __launch_bounds__(kThreads, gcpk::fused_min_blocks(D, COLS)) k_b
             h = hash_contains_from(P.s.hkeys, P.s.hbmask, key, ((mix64(key) & P.s.hbmask) + 1) & P.s.hbmask, 1);
         if (h == 0) return true;
         int32_t *slot = s_slot[st][warp][pos];
-        const uint64_t j = (uint64_t)(s - p);
+        const uint64_t j = (uint64_t)(uint32_t)(s - p);
         for (int a = 1; h == 1 && a < P.s.max_attempts; ++a) {
             int32_t idx[D];
             draw_tuple_b<D>(P.s, kStreamZero, j, 4 * (uint64_t)a, idx);

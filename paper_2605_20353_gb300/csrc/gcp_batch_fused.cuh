@@ -253,12 +253,15 @@ __global__ void __launch_bounds__(kThreads, gcpk::fused_min_blocks(D, COLS)) k_b
             for (int v = 0; v < COLS; ++v) pre[v] = y;
 #pragma unroll
             for (int n = 0; n < D; ++n) {
-                unsigned hs;
-                if (is_nz && grep)
-                    hs = ((unsigned)slot[D + 1 + n / 2] >> (16 * (n & 1))) & 0xFFFFu;
-                else
-                    hs = P.small_base[n] >= 0 ? (unsigned)(P.small_base[n] + ii[n]) : gcpk::kNoSlot;
-                float *g = hs != gcpk::kNoSlot ? grep + (int)hs * Rp : P.G + off[n];
+                float *g = P.G + off[n];
+                if (D > 4 || grep) {  // as in k_fused
+                    unsigned hs;
+                    if (is_nz && (D <= 4 || grep))
+                        hs = ((unsigned)slot[D + 1 + n / 2] >> (16 * (n & 1))) & 0xFFFFu;
+                    else
+                        hs = P.small_base[n] >= 0 ? (unsigned)(P.small_base[n] + ii[n]) : gcpk::kNoSlot;
+                    if (hs != gcpk::kNoSlot) g = grep + (int)hs * Rp;
+                }
 #pragma unroll
                 for (int q = 0; q < NQ; ++q)
                     red_add_v4(g + col[q], pre[4 * q] * suf[n][4 * q], pre[4 * q + 1] * suf[n][4 * q + 1],

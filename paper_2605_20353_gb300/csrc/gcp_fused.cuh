@@ -314,13 +314,29 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
 #pragma unroll
                 for (int n = 0; n < D; ++n) {
                     // replica slot: stored in a nonzero's record; for drawn
-                    // cells, rows of fully replicated modes only
-                    unsigned hs;
-                    if (is_nz && grep)
-                        hs = ((unsigned)slot[D + 1 + n / 2] >> (16 * (n & 1))) & 0xFFFFu;
-                    else
-                        hs = P.small_base[n] >= 0 ? (unsigned)(P.small_base[n] + ii[n]) : kNoSlot;
-                    float *g = hs != kNoSlot ? grep + (int)hs * P.Rp : P.G + off[n];
+                    // cells, rows of fully replicated modes only.  Passes
+                    // without replicas skip the search up to order 4 (rank
+                    // 20, 250,000 samples: 27.7 -> 27.1 us); at order 5 the
+                    // branch costs registers (dense 5-way: 325 -> 335 us)
+                    float *g;
+                    if constexpr (D > 4) {
+                        unsigned hs;
+                        if (is_nz && grep)
+                            hs = ((unsigned)slot[D + 1 + n / 2] >> (16 * (n & 1))) & 0xFFFFu;
+                        else
+                            hs = P.small_base[n] >= 0 ? (unsigned)(P.small_base[n] + ii[n]) : kNoSlot;
+                        g = hs != kNoSlot ? grep + (int)hs * P.Rp : P.G + off[n];
+                    } else {
+                        g = P.G + off[n];
+                        if (grep) {
+                            unsigned hs;
+                            if (is_nz)
+                                hs = ((unsigned)slot[D + 1 + n / 2] >> (16 * (n & 1))) & 0xFFFFu;
+                            else
+                                hs = P.small_base[n] >= 0 ? (unsigned)(P.small_base[n] + ii[n]) : kNoSlot;
+                            if (hs != kNoSlot) g = grep + (int)hs * P.Rp;
+                        }
+                    }
 #pragma unroll
                     for (int q = 0; q < NQ; ++q)
                         if (on[q])

@@ -75,6 +75,7 @@ constexpr int kNaProbe = 2048, kNaTable = 4096;
 
 __global__ void __launch_bounds__(kNaThreads) k_na_setup(const NaShape sh, int64_t n, const int32_t *__restrict__ idx,
                                                         float *__restrict__ G, NaScratch *__restrict__ S) {
+    grid_trigger();
     const int searchers = sh.hot ? sh.d : 0;
     if ((int)blockIdx.x >= searchers) {
         const int64_t total = sh.rows * sh.R, step = (int64_t)(gridDim.x - searchers) * kNaThreads;
@@ -164,7 +165,7 @@ __device__ __forceinline__ void na_add(float *p, const float *c) {
 // Bound by the row traffic through L2 (d rows gathered, d rows reduced per
 // sample).  2^18 samples of the 2000 x 1500
 // x 1000 x 200 Zipf tensor at rank 32, drawn with gcp_sample and passed
-// here: 106 us a pass, this kernel 42; 156 us with every reduction added to G itself (the ones
+// here: 99 us a pass, this kernel 42; 156 us with every reduction added to G itself (the ones
 // that meet in one row are applied one after another, about 4.7 ns each);
 // 745 us with one warp per sample walking 256 samples one after another on
 // 128 blocks.
@@ -178,6 +179,8 @@ __global__ void __launch_bounds__(kNaThreads, (D <= 4 ? 3 : 2))
     __shared__ int s_row[D][kBuckets];             // -1: empty
     __shared__ unsigned char s_slot[D][kBuckets];
     __shared__ int s_hot[D];
+    grid_wait();  // G is cleared and the hot rows are known
+    grid_trigger();
     if (sh.hot) {
         if (threadIdx.x < D) s_hot[threadIdx.x] = S->hot[threadIdx.x].n_nrep;
         for (int i = threadIdx.x; i < D * kBuckets; i += kNaThreads) (&s_row[0][0])[i] = -1;
@@ -342,6 +345,7 @@ __global__ void __launch_bounds__(kNaThreads, (D <= 4 ? 3 : 2))
 // per mode and hot row: the row's replicas added to G.
 __global__ void __launch_bounds__(kNaThreads) k_na_finish(const NaShape sh, float *__restrict__ G, NaScratch *S,
                                                          int nblocks, double *loss_out) {
+    grid_wait();
     if (blockIdx.x < gridDim.x - 1) {
         const int k = blockIdx.x / kNaHot, j = blockIdx.x % kNaHot;
         const int word = S->hot[k].n_nrep, hot = word & 255, nrep = word >> 8, rf = na_row_floats(sh.R);
@@ -498,9 +502,12 @@ extern "C" gcp_status gcp_grad_samples_noalloc(int32_t ndim, const int64_t *dims
         sh.tile = gcpk::fused_tile(nsamples, plan.log2L, most);
         const int64_t ntiles = (nsamples + sh.tile - 1) / sh.tile;
         nblocks = (int)std::min<int64_t>((ntiles + kNaWarps - 1) / kNaWarps, most);
-        k<<<nblocks, kNaThreads, 0, st>>>(sh, loss, nsamples, idx, x, w, A, G, scratch);
+        e = gcpk::launch_dependent(k, nblocks, kNaThreads, 0, st, sh, loss, nsamples, idx, x, w, A, G, scratch);
+        if (e != cudaSuccess) return na_fail(GCP_ERR_CUDA, cudaGetErrorString(e));
     }
-    k_na_finish<<<(sh.hot ? ndim * kNaHot : 0) + 1, kNaThreads, 0, st>>>(sh, G, scratch, nblocks, loss_out);
+    e = gcpk::launch_dependent(k_na_finish, (sh.hot ? ndim * kNaHot : 0) + 1, kNaThreads, 0, st, sh, G, scratch, nblocks,
+                               loss_out);
+    if (e != cudaSuccess) return na_fail(GCP_ERR_CUDA, cudaGetErrorString(e));
     if ((e = cudaGetLastError()) != cudaSuccess) return na_fail(GCP_ERR_CUDA, cudaGetErrorString(e));
     return GCP_OK;
 }

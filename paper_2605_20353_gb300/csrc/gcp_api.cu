@@ -274,6 +274,17 @@ gcp_status check_counts(gcp_ctx *c, int64_t p, int64_t q) {
     return GCP_OK;
 }
 
+// Whether single rows take far more of the nonzeros than a uniform tensor's.
+// Then the reductions gather in few lines, and where those lie counts: with
+// the replicas of a row in consecutive 128-byte lines of their own they spread
+// evenly over the L2 slices, while replicas a whole plane of hot rows apart
+// fell on them as the number of hot rows had it (2^21 samples at rank 32 on
+// 4-way Zipf tensors 216 to 249 us; now 216 to 236).  Without skew the planes,
+// compact per warp, are the better layout (100 x 90 x 80 x 70 at rank 32 215
+// against 217 us), and above order 4, where a row's stride other than Rp costs
+// registers (dense 5-way gradient 326 against 334 us), they are kept always.
+bool skewed(const gcp_ctx *c) { return c->d <= 4 && c->share_nz > 2.0 * c->share_cell; }
+
 // Replicas of the hot rows for a sample set.  The reductions that meet in one
 // 128-byte line are applied one after another, about 4.7 ns each (with no
 // replicas the benchmark's step takes 0.90 ms and the dense 5-way gradient
@@ -340,6 +351,8 @@ gcpk::FusedSpec gcpk_make_spec(const gcp_ctx *c, uint64_t iter, int64_t p, int64
     for (int k = 0; k < c->d; ++k) f.small_base[k] = f.nrep ? c->small_base[k] : -1;
     f.Grep = f.nrep ? c->Grep : nullptr;
     f.Htot = f.nrep ? c->Htot : 0;
+    f.rplane = skewed(c) ? std::max(c->Rp, 32) : c->Htot * c->Rp;
+    f.rstride = skewed(c) ? f.nrep * f.rplane : c->Rp;
     if (w_nz_out) *w_nz_out = w_nz;
     if (w_z_out) *w_z_out = w_z;
     return f;
@@ -467,6 +480,8 @@ gcp_status run_fused(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, bool grad,
         go.G = c->G;
         if (c->opt.mttkrp != GCP_MTTKRP_DETERMINISTIC && f.nrep) {
             go.Htot = f.Htot;
+            go.rstride = f.rstride;
+            go.rplane = f.rplane;
             go.nrep = f.nrep;
             go.Grep = f.Grep;
             go.hot_slot = c->hot_slot;
@@ -525,6 +540,8 @@ gcp_status do_step(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, const gcp_ad
     ps.Rp = c->Rp;
     ps.R = c->R;
     ps.Htot = f.Htot;
+    ps.rstride = f.rstride;
+    ps.rplane = f.rplane;
     ps.nrep = f.nrep;
     ps.G = c->G;
     ps.Grep = f.Grep;
@@ -798,7 +815,7 @@ gcp_status setup_hot_rows(gcp_ctx *c, const std::vector<int64_t> &counts) {
     c->share_nz = counts.empty() ? 0.0 : (double)most / (double)c->nnz;
     c->Htot = (int)row.size();
     if (c->Htot == 0) return GCP_OK;
-    const size_t rep_bytes = (size_t)gcpk::kReplicas * c->Htot * c->Rp * 4;
+    const size_t rep_bytes = (size_t)gcpk::kReplicas * c->Htot * (skewed(c) ? std::max(c->Rp, 32) : c->Rp) * 4;
     cudaError_t e;
     if ((e = cudaMalloc(&c->hot_slot, slot.size() * 4)) || (e = cudaMalloc(&c->hot_row, row.size() * 4)) ||
         (e = cudaMalloc(&c->Grep, rep_bytes)) ||

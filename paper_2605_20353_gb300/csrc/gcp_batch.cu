@@ -54,6 +54,7 @@ struct ClientAux {
     void *Abf;
     const int *hot_row;   // replica slot -> row
     const int *hot_slot;  // row -> replica slot, or -1; null without replicas
+    int rstride, rplane;  // as in FusedSpec
     int Htot, nrep;       // replicated rows and replicas of the client's sample count (both 0: none)
     int64_t nparam;  // total_rows * Rp
     int R, Rp;
@@ -192,8 +193,9 @@ __device__ __forceinline__ void post_hot_chunk(const ClientAux &a, int64_t h0, c
         c4 = reinterpret_cast<const float4 *>(a.C)[q];
         x4 = reinterpret_cast<const float4 *>(a.A)[q];
     }
-    const float4 t = gcpe::hot_quad_sum<NREP>(reinterpret_cast<float4 *>(a.Grep), ((int64_t)a.Htot * a.Rp) >> 2, hq,
-                                              gcpe::hot_group_mask<NREP>());
+    const float4 t =
+        gcpe::hot_quad_sum<NREP>(reinterpret_cast<float4 *>(a.Grep + (int64_t)slot * a.rstride) + cq, a.rplane >> 2,
+                                 gcpe::hot_group_mask<NREP>());
     const int col = cq << 2;
     if (!lead || col >= a.R) return;
     if (clear) reinterpret_cast<float4 *>(a.G)[q] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
@@ -572,6 +574,8 @@ gcp_status gcp_batch_create(int32_t nclients, gcp_ctx *const *clients, const int
         a.hot_row = c->hot_row;
         a.hot_slot = f.nrep ? c->hot_slot : nullptr;
         a.Htot = f.Htot;
+        a.rstride = f.rstride;
+        a.rplane = f.rplane;
         a.nrep = f.nrep;
         a.nparam = c->total_rows * c->Rp;
         a.R = c->R;

@@ -205,7 +205,7 @@ __global__ void __launch_bounds__(kThreads, gcpk::fused_min_blocks(D, COLS)) k_b
         const int p = (int)P.s.p;
         const int tbase = (tile - __ldg(tile_start + cur_client[st])) * tile_n;
         const bool semi = P.s.sampling == GCP_SAMPLING_SEMI_STRATIFIED;
-        float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (P.nrep - 1)) * P.Htot * Rp : nullptr;
+        float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (P.nrep - 1)) * P.rplane : nullptr;
         float tf_nz = 0.0f, tf_z = 0.0f;
         for (int it = 0; it * ngrp < tile_n; ++it) {
             const int src = it * ngrp + grp;
@@ -260,7 +260,7 @@ __global__ void __launch_bounds__(kThreads, gcpk::fused_min_blocks(D, COLS)) k_b
                         hs = ((unsigned)slot[D + 1 + n / 2] >> (16 * (n & 1))) & 0xFFFFu;
                     else
                         hs = P.small_base[n] >= 0 ? (unsigned)(P.small_base[n] + ii[n]) : gcpk::kNoSlot;
-                    if (hs != gcpk::kNoSlot) g = grep + (int)hs * Rp;
+                    if (hs != gcpk::kNoSlot) g = grep + (int)hs * P.rstride;
                 }
 #pragma unroll
                 for (int q = 0; q < NQ; ++q)

@@ -2,8 +2,8 @@
 // (k_post_step for one context, k_batch_post for a batch of clients).
 //
 // The fused pass sends the gradient reductions of rows that many samples hit
-// to NREP replicas (planes of Htot x Rp floats); the epilogue adds them into
-// the row's gradient before Adam.  A hot quad (four columns of a hot row) has
+// to NREP replicas of each; the epilogue adds them into the row's gradient
+// before Adam.  A hot quad (four columns of a hot row) has
 // NREP replica quads; loaded one after another they cost a memory round trip
 // per group, so instead a group of NREP / 4 lanes takes one hot quad, four
 // replicas a lane, and every replica load is in flight at once.
@@ -19,7 +19,7 @@ __host__ __device__ constexpr int hot_lanes() {  // lanes that fold one hot quad
     return NREP / 4;
 }
 
-// Sum of the NREP replica quads R4[r * plane4 + o], r = 0..NREP-1, over a
+// Sum of the NREP replica quads at R4, R4 + step, R4 + 2 step, ... over a
 // group of H = NREP / 4 lanes: lane l of the group loads replicas l, l + H,
 // l + 2 H, l + 3 H, adds them in that order, then the group sums its lanes
 // with a butterfly (offsets H/2, ..., 1).  The order is fixed, so the result
@@ -27,13 +27,13 @@ __host__ __device__ constexpr int hot_lanes() {  // lanes that fold one hot quad
 // clears the replicas it loaded.  All lanes of the group must call it
 // together (gmask = the group's lanes).
 template <int NREP>
-__device__ __forceinline__ float4 hot_quad_sum(float4 *__restrict__ R4, int64_t plane4, int64_t o, unsigned gmask) {
+__device__ __forceinline__ float4 hot_quad_sum(float4 *__restrict__ R4, int step, unsigned gmask) {
     constexpr int H = hot_lanes<NREP>();
     static_assert(4 * H == NREP && H <= 32, "four replicas a lane");
     const int l = threadIdx.x & (H - 1);
     float4 v[4];
 #pragma unroll
-    for (int i = 0; i < 4; ++i) v[i] = R4[(int64_t)(l + H * i) * plane4 + o];
+    for (int i = 0; i < 4; ++i) v[i] = R4[(l + H * i) * step];
     float4 t = v[0];
 #pragma unroll
     for (int i = 1; i < 4; ++i) {
@@ -43,7 +43,7 @@ __device__ __forceinline__ float4 hot_quad_sum(float4 *__restrict__ R4, int64_t 
         t.w += v[i].w;
     }
 #pragma unroll
-    for (int i = 0; i < 4; ++i) R4[(int64_t)(l + H * i) * plane4 + o] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
+    for (int i = 0; i < 4; ++i) R4[(l + H * i) * step] = make_float4(0.0f, 0.0f, 0.0f, 0.0f);
 #pragma unroll
     for (int off = H / 2; off > 0; off >>= 1) {
         t.x += __shfl_xor_sync(gmask, t.x, off);

@@ -148,7 +148,7 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
     const TF *F = static_cast<const TF *>(P.F);
     const bool semi = P.s.sampling == GCP_SAMPLING_SEMI_STRATIFIED;
     const bool uniform = P.s.sampling == GCP_SAMPLING_UNIFORM;
-    [[maybe_unused]] float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (P.nrep - 1)) * P.Htot * P.Rp : nullptr;
+    [[maybe_unused]] float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (P.nrep - 1)) * P.rplane : nullptr;
 
     double acc_nz = 0.0, acc_z = 0.0;
     int attempts = 0;
@@ -325,6 +325,7 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
                             hs = ((unsigned)slot[D + 1 + n / 2] >> (16 * (n & 1))) & 0xFFFFu;
                         else
                             hs = P.small_base[n] >= 0 ? (unsigned)(P.small_base[n] + ii[n]) : kNoSlot;
+                        // orders above 4 keep the replicas in planes: rstride is Rp
                         g = hs != kNoSlot ? grep + (int)hs * P.Rp : P.G + off[n];
                     } else {
                         g = P.G + off[n];
@@ -334,7 +335,7 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
                                 hs = ((unsigned)slot[D + 1 + n / 2] >> (16 * (n & 1))) & 0xFFFFu;
                             else
                                 hs = P.small_base[n] >= 0 ? (unsigned)(P.small_base[n] + ii[n]) : kNoSlot;
-                            if (hs != kNoSlot) g = grep + (int)hs * P.Rp;
+                            if (hs != kNoSlot) g = grep + (int)hs * P.rstride;
                         }
                     }
 #pragma unroll

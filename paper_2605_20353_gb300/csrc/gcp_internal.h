@@ -48,9 +48,10 @@ struct FusedSpec {
     double *partials;               // per block: sum f over nonzero / zero samples, attempts, -
     int small_base[GCP_MAX_NDIM];   // replica slot of row 0 of a mode whose rows all have
                                     // slots (contiguous), else -1; used for drawn cells
-    float *Grep;                    // nrep x Htot x Rp replica rows (zero between calls), or null:
+    float *Grep;                    // replica rows (zero between calls), or null:
                                     // every row is added to G itself
     int Htot;                       // replicated rows
+    int rstride, rplane;            // floats from one hot row to the next, and from replica to replica
     int nrep;                       // replicas this call uses: 0 (Grep null), 4, 16 or 64
     int32_t *Ycoord;                // materialize mode (G null): per-sample coordinates
     float *Yval;                    //   and gradient-tensor values w f' scale (0 if no sample):
@@ -60,7 +61,9 @@ struct FusedSpec {
 // Rows that many samples hit (Zipf heads, rows of small modes) are
 // accumulated in up to this many global replicas, then folded into G.  A
 // call uses as many as its sample count and the hottest row's share call for
-// (replicas_for): none, 4, 16 or all 64.
+// (replicas_for): none, 4, 16 or all 64.  Replica r of hot row `slot` starts at
+// slot * rstride + r * rplane floats: planes of Htot rows, or each row's
+// replicas in consecutive lines (skewed in gcp_api.cu).
 constexpr int kReplicas = 64;
 
 // Where a call's sampled loss goes once the block partials are summed: the
@@ -83,6 +86,7 @@ struct GradOutSpec {
     LossSpec loss;
     int64_t rows;
     int Rp, R, Htot, nrep;          // nrep 0: no replicas (Htot 0, hot_slot null)
+    int rstride, rplane;            // as in FusedSpec
     float *G, *Grep;
     const int *hot_slot, *hot_row;
     float *out;                     // rows x R, or null
@@ -94,6 +98,7 @@ struct PostSpec {
     LossSpec loss;
     int64_t n;                      // total_rows * Rp
     int Rp, R, Htot, nrep;          // nrep 0: no replicas (Htot 0, hot_slot null)
+    int rstride, rplane;            // as in FusedSpec
     float *G, *Grep, *A, *B, *C;
     void *Abf;
     const int *hot_slot;            // row -> replica slot, or -1
@@ -201,7 +206,7 @@ struct gcp_ctx {
     int *hot_slot = nullptr;      // [total_rows] row -> replica slot or -1
     int *hot_row = nullptr;       // [Htot] slot -> row
     int small_base[GCP_MAX_NDIM] = {0};
-    float *Grep = nullptr;        // [kReplicas x Htot x Rp]
+    float *Grep = nullptr;        // replica rows, room for kReplicas of each
     int Htot = 0;
     double share_nz = 0.0;        // largest share of the nonzeros in one row
     double share_cell = 0.0;      // the same of all cells: 1 / the smallest mode size

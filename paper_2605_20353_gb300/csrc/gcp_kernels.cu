@@ -150,8 +150,9 @@ __global__ void __launch_bounds__(kThreads) k_grad_finish(const GradOutSpec P, i
             const bool lead = (threadIdx.x & (H - 1)) == 0;
             float4 g;
             if (lead) g = G4[q];
-            const float4 t = gcpe::hot_quad_sum<NREP>(reinterpret_cast<float4 *>(P.Grep),
-                                                      ((int64_t)P.Htot * P.Rp) >> 2, hq, gcpe::hot_group_mask<NREP>());
+            const float4 t = gcpe::hot_quad_sum<NREP>(
+                reinterpret_cast<float4 *>(P.Grep + (int64_t)slot * P.rstride) + cq, P.rplane >> 2,
+                gcpe::hot_group_mask<NREP>());
             if (!lead) return;
             g.x += t.x;
             g.y += t.y;
@@ -329,8 +330,9 @@ __global__ void __launch_bounds__(kThreads) k_post_step(PostSpec P, int ncold) {
                 b = B4[q];
                 c = C4[q];
             }
-            const float4 t = gcpe::hot_quad_sum<NREP>(reinterpret_cast<float4 *>(P.Grep),
-                                                      ((int64_t)P.Htot * P.Rp) >> 2, hq, gcpe::hot_group_mask<NREP>());
+            const float4 t = gcpe::hot_quad_sum<NREP>(
+                reinterpret_cast<float4 *>(P.Grep + (int64_t)slot * P.rstride) + cq, P.rplane >> 2,
+                gcpe::hot_group_mask<NREP>());
             if (!lead) return;
             g.x += t.x;
             g.y += t.y;
@@ -478,7 +480,7 @@ __global__ void __launch_bounds__(kThreads) k_mttkrp_nonfused(const FusedSpec P,
     const int ngroups = (gridDim.x * blockDim.x) >> P.log2L;
     const int warp0 = (blockIdx.x * blockDim.x + threadIdx.x) >> 5;
     const TF *__restrict__ F = static_cast<const TF *>(P.F);
-    float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (P.nrep - 1)) * P.Htot * P.Rp : nullptr;
+    float *const grep = P.Grep ? P.Grep + (size_t)(warp0 & (P.nrep - 1)) * P.rplane : nullptr;
     int col[NQ];
     bool on[NQ];  // the quad holds columns of the rank, not padding alone
 #pragma unroll
@@ -510,7 +512,7 @@ __global__ void __launch_bounds__(kThreads) k_mttkrp_nonfused(const FusedSpec P,
 #pragma unroll
         for (int n = 0; n < D; ++n) {
             const int hs = hot_slot ? __ldg(hot_slot + P.rowoff[n] + ii[n]) : -1;
-            float *g = hs >= 0 ? grep + hs * P.Rp : P.G + off[n];
+            float *g = hs >= 0 ? grep + hs * P.rstride : P.G + off[n];
 #pragma unroll
             for (int q = 0; q < NQ; ++q)
                 if (on[q])

@@ -766,6 +766,58 @@ def test_replica_counts_in_turn_on_one_context(env, mttkrp):
     ctx.close()
 
 
+def one_heavy_row(dims, nnz, heavy, seed):
+    """Distinct cells of a 3-way tensor, `heavy` of them in row 5 of the last
+    mode: there the hottest row holds several times a uniform tensor's share,
+    so its replicas lie in consecutive lines of their own."""
+    rng = np.random.default_rng(seed)
+    cells = rng.choice(dims[0] * dims[1], heavy, replace=False) * dims[2] + 5
+    rest = rng.choice(dims[0] * dims[1] * dims[2], 2 * nnz, replace=False)
+    cells = np.concatenate([cells, rest[rest % dims[2] != 5][:nnz - heavy]])
+    coords = np.stack(np.unravel_index(cells, dims), axis=1)
+    return coords.astype(synth.uniform_sparse(dims, 8, 1)[0].dtype), rng.integers(1, 6, nnz).astype(np.float32)
+
+
+@pytest.mark.parametrize("R", [3, 6, 32, 40])
+@pytest.mark.parametrize("mttkrp", ["atomic", "nonfused"])
+def test_replica_lines_of_skewed_tensors(env, mttkrp, R):
+    """Replicas in lines of their own (a row with a sixth of the nonzeros;
+    ranks below, at and above the 32 floats of a line): sample counts that
+    take none, 4, 16 and 64 of them mixed on one context, so every call must
+    find cleared what calls with another replica stride used."""
+    gcp, torch = env
+    dims = [40, 300, 700]
+    coords, vals = one_heavy_row(dims, 6000, 1000, 621)
+    factors = synth.factors_uniform(dims, R, 622, lo=0.1, hi=1.0)
+    ctx = gcp.gcp_create(dims, coords, vals, R, "poisson", seed=623, mttkrp=mttkrp)
+    for t, (p, q) in enumerate([(60000, 50000), (150, 130), (3000, 700), (7000, 6001), (3000, 700), (60000, 1)]):
+        idx, x, w, _ = oracle.stratified_samples(623, t, p, q, dims, coords, vals)
+        Lo, Go = oracle.sampled_loss_grad(dims, factors, "poisson", idx, x, w)
+        ctx.set_factors(factors)
+        Lg, Gg = gpu_grad(gcp, torch, ctx, t, p, q)
+        assert abs(Lg - Lo) <= TOL_FP32 * abs(Lo), (t, Lg, Lo)
+        for n, (a, b) in enumerate(zip(split(Gg, dims, R), Go)):
+            assert rel_err(a, b) <= TOL_FP32, (t, n, rel_err(a, b))
+        G = step_gradient(gcp, ctx, factors, t, p, q, max(np.abs(g).max() for g in Go))
+        for n, (a, b) in enumerate(zip(split(G, dims, R), Go)):
+            assert rel_err(a, b) <= TOL_FP32, (t, n, rel_err(a, b))
+    if mttkrp == "atomic":  # a batch folds the same replicas
+        b = gcp.GcpBatch([ctx], [7000], [6001])
+        idx, x, w, _ = oracle.stratified_samples(623, 9, 7000, 6001, dims, coords, vals)
+        _, Go = oracle.sampled_loss_grad(dims, factors, "poisson", idx, x, w)
+        from adam_readout import flat, readout_params, recover_gradient
+        prm = readout_params(gcp, max(np.abs(g).max() for g in Go))
+        ctx.set_factors(factors)
+        ctx.reset_adam()
+        b.local_steps(1, prm, 9, 0)
+        b.losses()
+        G = recover_gradient(flat(factors), flat(ctx.get_factors()), prm)
+        for n, (a, g) in enumerate(zip(split(G, dims, R), Go)):
+            assert rel_err(a, g) <= TOL_FP32, (n, rel_err(a, g))
+        b.close()
+    ctx.close()
+
+
 def test_fit_with_tuned_preset_on_count_data(env):
     """gcp_fit with the paper's tuned GCP-SGD hyperparameters on a Poisson
     count tensor: the objective estimate falls, at most max_fails epochs

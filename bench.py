@@ -482,7 +482,7 @@ def batched_variant(gcp, torch, stream, steps=20, with_oracle=True):
         c.close()
     # 64 sequential single-client steps: gcp_step (fused pass + one epilogue,
     # two launches per client, the best single-client path) and gradient +
-    # Adam as separate calls (five launches per client)
+    # Adam as separate calls (four launches per client)
     nseq = max(2, steps // 4)
     for form in ("step", "grad_adam"):
         for dtype in ("bf16", "fp32"):
@@ -507,7 +507,7 @@ def batched_variant(gcp, torch, stream, steps=20, with_oracle=True):
             ms = e0.elapsed_time(e1)
             key = f"sequential_{form}_{dtype}"
             res[key] = {"value": samples_per_step * tau * nseq / (ms / 1e3), "unit": "samples/s",
-                        "launches_per_client_step": 2 if form == "step" else 5}
+                        "launches_per_client_step": 2 if form == "step" else 4}
             for c in clients:
                 c.close()
     for key in [k for k in res if k.startswith("sequential_")]:

@@ -94,7 +94,13 @@ __device__ __forceinline__ void load_record(const int32_t *__restrict__ rec, uin
 //      a test around the loads costs more than the sectors (orders 2 to 8,
 //      ranks 20 to 65, 2^20 samples: 0 to 15% slower with it).
 // The loss: the group's first lane leaves f in the sample's slot; after the
-// tile each lane takes its own sample's f, a butterfly sums the tile in
+// tile each lane takes its own sample's f.  Without reductions (EVAL) no lane
+// of the group needs f', so the group leaves m there instead and each lane
+// evaluates its own sample: one evaluation per tile instead of one per group
+// round, and the gradient tensor's entries written by neighbouring lanes
+// (2^19 samples of the 4-way Zipf counts in BF16, a loss call: 48.1 -> 45.3
+// us; deterministic gradient of 2^21 samples at rank 64: 531 -> 501 us).
+// Then a butterfly sums the tile in
 // FP32 (nonzero and other samples apart), and the warp adds the sum to its
 // FP64 totals.  (FP64 adds are slow here, 16 cycles of the SM's pipe for a
 // warp: a lane's own FP64 totals, reduced over the warp at the end, cost 2 us
@@ -227,6 +233,20 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
         return false;
     };
 
+    // loss and derivative of one sample
+    auto sample_loss = [&](float x, float m, bool is_nz, float &f, float &df) {
+        float f1, d1;
+        loss_eval(P.loss, x, m, f1, d1);
+        if (semi && is_nz) {
+            float f0, d0;
+            loss_eval(P.loss, 0.0f, m, f0, d0);
+            f1 -= f0;
+            d1 -= d0;
+        }
+        f = f1;
+        df = d1;
+    };
+
     int tile = warp0;
     uint64_t key_next = issue(tile, 0);
     cp_async_commit();
@@ -244,26 +264,18 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
         cp_async_wait<1>();  // this lane's copies into stage st have landed
         const bool ok = finish(tile, st, key);
         const unsigned okmask = __ballot_sync(0xFFFFFFFFu, ok);
+        [[maybe_unused]] float xl = 0.0f;  // EVAL: this lane's own value, as m takes its place
+        if (EVAL && ok) xl = __int_as_float(s_slot[st][warp][lane][D]);
         __syncwarp();  // every lane's staged sample is visible to the warp
 
         // phase B: one sample per group
         for (int it = 0; it * ngrp < (int)TS; ++it) {
             const int src = it * ngrp + grp;
-            if (!((okmask >> src) & 1u)) {  // uniform within the group
-                const unsigned sm = (unsigned)tile * TS + src;
-                if (EVAL && P.Yval && glane == 0 && src < (int)TS && sm < (unsigned)S) {  // no sample: a zero entry at a valid cell
-#pragma unroll
-                    for (int k = 0; k < D; ++k) P.Ycoord[(int64_t)sm * P.ystride + k] = s_slot[st][warp][src][k];
-                    P.Yval[(int64_t)sm * P.vstride] = 0.0f;
-                }
-                continue;
-            }
+            if (!((okmask >> src) & 1u)) continue;  // uniform within the group
             int32_t *slot = s_slot[st][warp][src];
             int32_t ii[D];
 #pragma unroll
             for (int k = 0; k < D; ++k) ii[k] = slot[k];
-            const float xs = __int_as_float(slot[D]);
-            const bool is_nz = !uniform && ((unsigned)tile * TS + src) < (unsigned)p;
 
             int off[D];
             float a[D][COLS];
@@ -290,23 +302,14 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
             float m = NQ == 2 ? mq[0] + mq[NQ - 1] : mq[0];
             for (int o = L >> 1; o > 0; o >>= 1) m += __shfl_xor_sync(gmask, m, o);
 
-            float f, df;
-            loss_eval(P.loss, xs, m, f, df);
-            if (semi && is_nz) {
-                float f0, df0;
-                loss_eval(P.loss, 0.0f, m, f0, df0);
-                f -= f0;
-                df -= df0;
-            }
-            if (glane == 0) slot[D] = __float_as_int(f);  // the group has read the value
-            if constexpr (EVAL) {
-                if (P.Yval && glane == 0) {  // the gradient tensor entry (non-fused MTTKRP input)
-                    const int sm = tile * TS + src;
-#pragma unroll
-                    for (int k = 0; k < D; ++k) P.Ycoord[(int64_t)sm * P.ystride + k] = ii[k];
-                    P.Yval[(int64_t)sm * P.vstride] = ((is_nz || uniform) ? P.w_nz : P.w_z) * df * scale;
-                }
+            if constexpr (EVAL) {  // the sample's own lane takes it from here
+                if (glane == 0) slot[D] = __float_as_int(m);
             } else {
+                const float xs = __int_as_float(slot[D]);
+                const bool is_nz = !uniform && ((unsigned)tile * TS + src) < (unsigned)p;
+                float f, df;
+                sample_loss(xs, m, is_nz, f, df);
+                if (glane == 0) slot[D] = __float_as_int(f);  // the group has read the value
                 const float y = ((is_nz || uniform) ? P.w_nz : P.w_z) * df * scale;
                 float pre[COLS];
 #pragma unroll
@@ -348,9 +351,21 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
                 }
             }
         }
-        __syncwarp();  // the losses are in their slots
-        const float fl = ok ? __int_as_float(s_slot[st][warp][lane][D]) : 0.0f;
+        __syncwarp();  // the losses (EVAL: the models) are in their slots
+        float fl = ok ? __int_as_float(s_slot[st][warp][lane][D]) : 0.0f;
         const unsigned s0 = (unsigned)tile * TS;
+        if constexpr (EVAL) {
+            const bool is_nz = !uniform && s0 + lane < (unsigned)p;
+            float df = 0.0f;
+            if (ok) sample_loss(xl, fl, is_nz, fl, df);
+            if (P.Yval && lane < (int)TS && s0 + lane < (unsigned)S) {
+                // the gradient tensor entry; no sample: a zero at a valid cell
+                const int64_t sm = s0 + lane;
+#pragma unroll
+                for (int k = 0; k < D; ++k) P.Ycoord[sm * P.ystride + k] = s_slot[st][warp][lane][k];
+                P.Yval[sm * P.vstride] = ok ? ((is_nz || uniform) ? P.w_nz : P.w_z) * df * scale : 0.0f;
+            }
+        }
         if (uniform || s0 + TS <= (unsigned)p) {
             acc_nz += (double)warp_sum(fl);
         } else if (s0 >= (unsigned)p) {

@@ -960,6 +960,31 @@ def test_loss_bits_do_not_depend_on_the_pass(env, dims, R, loss, dtype):
     assert all(len(v) == 1 for v in L.values()), L
 
 
+@pytest.mark.parametrize("R", [3, 20, 64])
+@pytest.mark.parametrize("loss", ["gaussian", "poisson", "bernoulli", "gamma"])
+def test_semi_stratified_passes_that_evaluate_samples_by_lane(env, loss, R):
+    """Passes without reductions evaluate a sample in its own lane, a gradient
+    pass in its group: with the f(x,m) - f(0,m) terms of the semi-stratified
+    samples too the losses agree bit for bit, and the gradient formed from the
+    written tensor entries with the oracle's."""
+    gcp, torch = env
+    dims = [61, 47, 900]
+    coords, vals, factors = problem(dims, 4000, R, loss, 821)
+    L = {}
+    for mttkrp in ("atomic", "nonfused", "deterministic"):
+        ctx = gcp.gcp_create(dims, coords, vals, R, loss, seed=822, mttkrp=mttkrp, sampling="semi")
+        ctx.set_factors(factors)
+        for p, q in [(3, 2), (700, 911), (20001, 15000)]:
+            Lg, Gg = gpu_grad(gcp, torch, ctx, 1, p, q)
+            L.setdefault((p, q), set()).update({ctx.loss_value(1, p, q), Lg})
+            idx, x, w, semi = oracle.semi_stratified_samples(822, 1, p, q, dims, coords, vals)
+            _, Go = oracle.sampled_loss_grad(dims, factors, loss, idx, x, w, semi=semi)
+            for n, (a, b) in enumerate(zip(split(Gg, dims, R), Go)):
+                assert rel_err(a, b) <= TOL_FP32, (mttkrp, p, n, rel_err(a, b))
+        ctx.close()
+    assert all(len(v) == 1 for v in L.values()), L
+
+
 @pytest.mark.parametrize("p,q", [(40, 33), (3000, 2800), (300000, 300000)])
 @pytest.mark.parametrize("dtype", ["fp32", "bf16"])
 def test_back_to_back_calls_wait_for_one_another(env, p, q, dtype):

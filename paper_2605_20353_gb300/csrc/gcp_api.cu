@@ -783,7 +783,10 @@ gcp_status refresh_bf16(gcp_ctx *c) {
 gcp_status setup_hot_rows(gcp_ctx *c, const std::vector<int64_t> &counts) {
     std::vector<int> slot((size_t)c->total_rows, -1), row;
     for (int k = 0; k < c->d; ++k) c->share_cell = std::max(c->share_cell, 1.0 / (double)c->dims[k]);
-    int64_t most = 0;  // nonzeros of the fullest row
+    // nonzeros of the fullest row among those with replicas: the fullest of all
+    // wherever there are any, since a mode of at most 512 rows has a row with
+    // 1/512 of the nonzeros and a row without replicas holds less
+    int64_t most = 0;
     for (int k = 0; k < c->d; ++k) {
         c->small_base[k] = -1;
         if (c->dims[k] > 512) continue;
@@ -799,13 +802,10 @@ gcp_status setup_hot_rows(gcp_ctx *c, const std::vector<int64_t> &counts) {
         if (c->dims[k] <= 512) continue;
         std::vector<std::pair<int64_t, int>> hot;
         const int64_t *at = counts.data() + c->rowoff[k];
-        int64_t fullest = 0;
-        for (int64_t i = 0; i < c->dims[k]; ++i) {
-            fullest = std::max(fullest, at[i]);
+        for (int64_t i = 0; i < c->dims[k]; ++i)
             if (at[i] >= floor_hot) hot.push_back({at[i], (int)(c->rowoff[k] + i)});
-        }
-        most = std::max(most, fullest);
         std::stable_sort(hot.begin(), hot.end(), [](const auto &x, const auto &y) { return x.first > y.first; });
+        if (!hot.empty()) most = std::max(most, hot.front().first);
         if (hot.size() > 256) hot.resize(256);
         for (const auto &h : hot) {
             slot[(size_t)h.second] = (int)row.size();

@@ -93,9 +93,11 @@ __device__ __forceinline__ void load_record(const int32_t *__restrict__ rec, uin
 //      beyond the rank hold zeros and are not reduced; they are loaded, as
 //      a test around the loads costs more than the sectors (orders 2 to 8,
 //      ranks 20 to 65, 2^20 samples: 0 to 15% slower with it).
-// The loss: the group's first lane leaves f in the sample's slot; after the
-// tile each lane takes its own sample's f.  Without reductions (EVAL) no lane
-// of the group needs f', so the group leaves m there instead and each lane
+// The loss: the group's first lane leaves f in shared memory, in words that
+// nothing else uses during phase B (the stage's hash buckets, all read by
+// then: the other lanes of the group may still be reading the sample's slot);
+// after the tile each lane takes its own sample's f.  Without reductions
+// (EVAL) no lane of the group needs f', so the group leaves m there and each lane
 // evaluates its own sample: one evaluation per tile instead of one per group
 // round, and the gradient tensor's entries written by neighbouring lanes
 // (2^19 samples of the 4-way Zipf counts in BF16, a loss call: 48.1 -> 45.3
@@ -264,15 +266,14 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
         cp_async_wait<1>();  // this lane's copies into stage st have landed
         const bool ok = finish(tile, st, key);
         const unsigned okmask = __ballot_sync(0xFFFFFFFFu, ok);
-        [[maybe_unused]] float xl = 0.0f;  // EVAL: this lane's own value, as m takes its place
-        if (EVAL && ok) xl = __int_as_float(s_slot[st][warp][lane][D]);
-        __syncwarp();  // every lane's staged sample is visible to the warp
+        __syncwarp();  // every lane's staged sample is visible to the warp, and every bucket has been read
+        float *const handoff = reinterpret_cast<float *>(&s_bkt[st][warp][0][0]);  // [32]: f (EVAL: m) per sample
 
         // phase B: one sample per group
         for (int it = 0; it * ngrp < (int)TS; ++it) {
             const int src = it * ngrp + grp;
             if (!((okmask >> src) & 1u)) continue;  // uniform within the group
-            int32_t *slot = s_slot[st][warp][src];
+            const int32_t *slot = s_slot[st][warp][src];
             int32_t ii[D];
 #pragma unroll
             for (int k = 0; k < D; ++k) ii[k] = slot[k];
@@ -303,13 +304,13 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
             for (int o = L >> 1; o > 0; o >>= 1) m += __shfl_xor_sync(gmask, m, o);
 
             if constexpr (EVAL) {  // the sample's own lane takes it from here
-                if (glane == 0) slot[D] = __float_as_int(m);
+                if (glane == 0) handoff[src] = m;
             } else {
                 const float xs = __int_as_float(slot[D]);
                 const bool is_nz = !uniform && ((unsigned)tile * TS + src) < (unsigned)p;
                 float f, df;
                 sample_loss(xs, m, is_nz, f, df);
-                if (glane == 0) slot[D] = __float_as_int(f);  // the group has read the value
+                if (glane == 0) handoff[src] = f;
                 const float y = ((is_nz || uniform) ? P.w_nz : P.w_z) * df * scale;
                 float pre[COLS];
 #pragma unroll
@@ -351,13 +352,13 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
                 }
             }
         }
-        __syncwarp();  // the losses (EVAL: the models) are in their slots
-        float fl = ok ? __int_as_float(s_slot[st][warp][lane][D]) : 0.0f;
+        __syncwarp();  // the losses (EVAL: the models) are handed over
+        float fl = ok ? handoff[lane] : 0.0f;
         const unsigned s0 = (unsigned)tile * TS;
         if constexpr (EVAL) {
             const bool is_nz = !uniform && s0 + lane < (unsigned)p;
             float df = 0.0f;
-            if (ok) sample_loss(xl, fl, is_nz, fl, df);
+            if (ok) sample_loss(__int_as_float(s_slot[st][warp][lane][D]), fl, is_nz, fl, df);
             if (P.Yval && lane < (int)TS && s0 + lane < (unsigned)S) {
                 // the gradient tensor entry; no sample: a zero at a valid cell
                 const int64_t sm = s0 + lane;

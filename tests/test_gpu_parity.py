@@ -271,6 +271,32 @@ def test_grad_scale_and_async_loss(env):
 
 
 # ---------------------------------------------------------------- Adam
+@pytest.mark.parametrize("dtype", ["fp32", "bf16"])
+@pytest.mark.parametrize("d,R", [(2, 8), (3, 8), (4, 16), (2, 32), (5, 32), (3, 64), (8, 64), (2, 128), (4, 128)])
+def test_every_lane_of_a_group_sees_the_sample_value(env, d, R, dtype):
+    """Groups of 2 to 32 lanes (four columns each) evaluate one sample; its
+    first lane hands the loss over in shared memory while the others may still
+    read the value.  With values of about 1000 a lane that took the loss
+    (about 5e5) for the value would be 500 times off in its columns alone:
+    every group of four columns is compared by itself with the oracle."""
+    gcp, torch = env
+    dims = [61, 47, 30, 11, 5, 4, 3, 6][:d]
+    coords, vals, factors = problem(dims, 2000, R, "gaussian", 861)
+    vals = (vals + 1000.0).astype(np.float32)
+    ctx = gcp.gcp_create(dims, coords, vals, R, "gaussian", seed=862, dtype=dtype, lane_cols=4)
+    ctx.set_factors(factors)
+    fac = [bf16_round(a) for a in factors] if dtype == "bf16" else factors
+    for p, q in [(37, 5), (50000, 20001)]:
+        L, G = gpu_grad(gcp, torch, ctx, 3, p, q)
+        idx, x, w, _ = oracle.stratified_samples(862, 3, p, q, dims, coords, vals)
+        Lo, Go = oracle.sampled_loss_grad(dims, fac, "gaussian", idx, x, w)
+        assert abs(L - Lo) <= TOL_FP32 * abs(Lo)
+        for a, b in zip(split(G, dims, R), Go):
+            for c in range(0, R, 4):
+                assert rel_err(a[:, c:c + 4], b[:, c:c + 4]) <= TOL_FP32, (p, c)
+    ctx.close()
+
+
 @pytest.mark.parametrize("where", ["vector", "offset", "host", "pinned"])
 @pytest.mark.parametrize("mttkrp,p,q", [("atomic", 60000, 50000), ("atomic", 7000, 6001), ("atomic", 900, 700),
                                         ("atomic", 150, 130), ("deterministic", 900, 700)])

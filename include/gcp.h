@@ -395,7 +395,8 @@ gcp_status gcp_batch_server_step(gcp_batch *batch, const gcp_adam_params *prm, i
  * array's device address (cudaGetSymbolAddress) with that device current;
  * make that first call before any stream capture.  Every call on a device
  * shares the array: calls whose kernels overlap on the GPU race and must be
- * ordered by the caller (one stream, or events).  Asynchronous: the call
+ * ordered by the caller (one stream, or events); the loss and the gradient of
+ * calls that do overlap are undefined.  Asynchronous: the call
  * returns before any result exists, so a NaN or infinite loss is not a
  * status code here; the caller reads loss_out[0] after the stream. */
 #define GCP_NOALLOC_MAX_SAMPLES 16777216LL

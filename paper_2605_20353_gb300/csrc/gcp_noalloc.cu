@@ -19,6 +19,7 @@
 #include "../../include/gcp.h"
 #include "gcp_device.cuh"
 #include "gcp_internal.h"
+#include "gcp_noalloc_hot.h"
 
 using namespace gcpdev;
 
@@ -28,24 +29,23 @@ constexpr int kNaThreads = 256;
 constexpr int kNaWarps = kNaThreads / 32;
 constexpr int kNaMaxBlocks = 2048;
 constexpr int kNaMaxDevices = 64;
-constexpr int kNaHot = 32;               // hot rows of a mode at most
-constexpr int kNaRepFloats = 23 * 1024;  // replica rows, shared out evenly over the modes
 
-// The hot rows of one mode: nrep replicas of n rows each, n | nrep << 8 in one
-// word (read once by whoever uses it, so that the two always belong together).
+// The hot rows of one mode: how many, with how many replicas each
+// (gcpna::hot_word), and which.
 struct NaHot {
-    int n_nrep;
-    int row[kNaHot];
+    int word;
+    int row[gcpna::kHot];
 };
 
 // Everything a call keeps on the device, shared by every call on it: loss
 // partials (block loss, skipped samples), the hot rows, their replicas.  Each
 // call writes what it reads later, so nothing has to start at zero; calls
-// that overlap on the GPU race on it.
+// that overlap on the GPU race on it, and what a kernel finds is held to its
+// own call's shape before it is used (gcp_noalloc_hot.h).
 struct NaScratch {
     double2 partials[kNaMaxBlocks];
     NaHot hot[GCP_MAX_NDIM];
-    alignas(16) float rep[kNaRepFloats];
+    alignas(16) float rep[gcpna::kRepFloats];
 };
 static_assert(sizeof(NaScratch) <= 128 * 1024, "the documented size of the scratch");
 __device__ __align__(256) unsigned char g_na_scratch[128 * 1024];
@@ -61,14 +61,10 @@ struct NaShape {
     int64_t rowoff[GCP_MAX_NDIM];
 };
 
-// Floats of a replica row, and of one mode's share of the replicas.
-__host__ __device__ constexpr int na_row_floats(int R) { return (R + 3) & ~3; }
-__host__ __device__ constexpr int na_mode_floats(int d) { return (kNaRepFloats / d) & ~3; }
-
 // Blocks k < d (if sh.hot): the hot rows of mode k.  kNaProbe samples spread
 // over the list are counted in a hash table; the rows counted at least T times
 // are hot, T the smallest of 8, 16, 32, ... with which there are at most
-// kNaHot of them and four replicas of each fit the mode's share.  (A row that
+// kHot of them and four replicas of each fit the mode's share.  (A row that
 // takes 1/256 of the samples is counted 8 times.)  The mode's replicas are
 // cleared.  The other blocks clear G.
 constexpr int kNaProbe = 2048, kNaTable = 4096;
@@ -117,21 +113,15 @@ __global__ void __launch_bounds__(kNaThreads) k_na_setup(const NaShape sh, int64
         for (int t = 0; t < 8; ++t)
             if (count[i] >= (8u << t)) atomicAdd(&over[t], 1);
     __syncthreads();
-    const int rf = na_row_floats(sh.R), share = na_mode_floats(sh.d);
     int t = 0;
-    while (t < 7 && (over[t] > kNaHot || 4 * over[t] * rf > share)) ++t;
-    const int hot = over[t] <= kNaHot && 4 * over[t] * rf <= share ? over[t] : 0;
-    int nrep = 0;
-    if (hot) {
-        nrep = 4;
-        while (nrep < 32 && 2 * nrep * hot * rf <= share) nrep *= 2;
+    while (t < 7 && over[t] && !gcpna::replicas(over[t], sh.R, sh.d)) ++t;
+    const int word = gcpna::hot_word(over[t], sh.R, sh.d);
+    if (word)
         for (int i = threadIdx.x; i < kNaTable; i += kNaThreads)
             if (count[i] >= (8u << t)) S->hot[k].row[atomicAdd(&slots, 1)] = key[i];
-    }
-    if (threadIdx.x == 0) {
-        S->hot[k].n_nrep = hot | nrep << 8;
-    }
-    for (int i = threadIdx.x; i < hot * nrep * rf; i += kNaThreads) S->rep[k * share + i] = 0.0f;
+    if (threadIdx.x == 0) S->hot[k].word = word;
+    const int floats = gcpna::hot_count(word) * gcpna::hot_replicas(word) * gcpna::row_floats(sh.R);
+    for (int i = threadIdx.x; i < floats; i += kNaThreads) S->rep[k * gcpna::mode_floats(sh.d) + i] = 0.0f;
 }
 
 // V consecutive columns of a row of A, or added to a row of G: one 16-byte
@@ -178,16 +168,16 @@ __global__ void __launch_bounds__(kNaThreads, (D <= 4 ? 3 : 2))
     constexpr int kBuckets = 64;
     __shared__ int s_row[D][kBuckets];             // -1: empty
     __shared__ unsigned char s_slot[D][kBuckets];
-    __shared__ int s_hot[D];
+    __shared__ int s_hot[D];                       // hot_word
     grid_wait();  // G is cleared and the hot rows are known
     grid_trigger();
     if (sh.hot) {
-        if (threadIdx.x < D) s_hot[threadIdx.x] = S->hot[threadIdx.x].n_nrep;
+        if (threadIdx.x < D) s_hot[threadIdx.x] = gcpna::hot_word_for(S->hot[threadIdx.x].word, sh.R, D);
         for (int i = threadIdx.x; i < D * kBuckets; i += kNaThreads) (&s_row[0][0])[i] = -1;
         __syncthreads();
-        for (int i = threadIdx.x; i < D * kNaHot; i += kNaThreads) {
-            const int k = i / kNaHot, j = i % kNaHot;
-            if (j >= (s_hot[k] & 255)) continue;
+        for (int i = threadIdx.x; i < D * gcpna::kHot; i += kNaThreads) {
+            const int k = i / gcpna::kHot, j = i % gcpna::kHot;
+            if (j >= gcpna::hot_count(s_hot[k])) continue;
             const int r = S->hot[k].row[j];
             unsigned h = ((unsigned)r * 2654435769u) >> 26;
             while (atomicCAS(&s_row[k][h], -1, r) != -1) h = (h + 1) & (kBuckets - 1);  // at most half full
@@ -208,13 +198,14 @@ __global__ void __launch_bounds__(kNaThreads, (D <= 4 ? 3 : 2))
     const int TS = sh.tile;
     const int64_t ntiles = (n + TS - 1) / TS;
     const int64_t nwarps = (int64_t)gridDim.x * kNaWarps;
-    const int rf = na_row_floats(sh.R);
+    const int rf = gcpna::row_floats(sh.R);
     int rep[D];  // where this warp's replicas of a mode's hot rows start
 #pragma unroll
     for (int k = 0; k < D; ++k) {
-        rep[k] = k * na_mode_floats(D);
+        rep[k] = k * gcpna::mode_floats(D);
         if (sh.hot && s_hot[k])
-            rep[k] += (((int)blockIdx.x * kNaWarps + warp) & ((s_hot[k] >> 8) - 1)) * (s_hot[k] & 255) * rf;
+            rep[k] += (((int)blockIdx.x * kNaWarps + warp) & (gcpna::hot_replicas(s_hot[k]) - 1)) *
+                      gcpna::hot_count(s_hot[k]) * rf;
     }
     int32_t ni[D];  // the next tile's sample of this lane
     float nx = 0.0f, nw = 0.0f;
@@ -347,11 +338,13 @@ __global__ void __launch_bounds__(kNaThreads) k_na_finish(const NaShape sh, floa
                                                          int nblocks, double *loss_out) {
     grid_wait();
     if (blockIdx.x < gridDim.x - 1) {
-        const int k = blockIdx.x / kNaHot, j = blockIdx.x % kNaHot;
-        const int word = S->hot[k].n_nrep, hot = word & 255, nrep = word >> 8, rf = na_row_floats(sh.R);
+        const int k = blockIdx.x / gcpna::kHot, j = blockIdx.x % gcpna::kHot;
+        const int word = gcpna::hot_word_for(*const_cast<const volatile int *>(&S->hot[k].word), sh.R, sh.d);
+        const int row = *const_cast<const volatile int *>(&S->hot[k].row[j]);  // both read once, then checked
+        const int hot = gcpna::hot_count(word), nrep = gcpna::hot_replicas(word), rf = gcpna::row_floats(sh.R);
         const int c = threadIdx.x;
-        if (j >= hot || c >= sh.R) return;
-        const float *p = S->rep + k * na_mode_floats(sh.d) + j * rf + c;
+        if (j >= hot || c >= sh.R || !gcpna::row_in_mode(row, sh.dims[k])) return;
+        const float *p = S->rep + k * gcpna::mode_floats(sh.d) + j * rf + c;
         float t = 0.0f;
         for (int r = 0; r < nrep; r += 4) {  // 4, 8, 16 or 32
             float v[4];
@@ -359,7 +352,7 @@ __global__ void __launch_bounds__(kNaThreads) k_na_finish(const NaShape sh, floa
             for (int u = 0; u < 4; ++u) v[u] = p[(r + u) * hot * rf];
             t += (v[0] + v[1]) + (v[2] + v[3]);
         }
-        G[(sh.rowoff[k] + S->hot[k].row[j]) * sh.R + c] += t;
+        G[(sh.rowoff[k] + row) * sh.R + c] += t;
         return;
     }
     __shared__ double2 red[kNaThreads];
@@ -505,7 +498,7 @@ extern "C" gcp_status gcp_grad_samples_noalloc(int32_t ndim, const int64_t *dims
         e = gcpk::launch_dependent(k, nblocks, kNaThreads, 0, st, sh, loss, nsamples, idx, x, w, A, G, scratch);
         if (e != cudaSuccess) return na_fail(GCP_ERR_CUDA, cudaGetErrorString(e));
     }
-    e = gcpk::launch_dependent(k_na_finish, (sh.hot ? ndim * kNaHot : 0) + 1, kNaThreads, 0, st, sh, G, scratch, nblocks,
+    e = gcpk::launch_dependent(k_na_finish, (sh.hot ? ndim * gcpna::kHot : 0) + 1, kNaThreads, 0, st, sh, G, scratch, nblocks,
                                loss_out);
     if (e != cudaSuccess) return na_fail(GCP_ERR_CUDA, cudaGetErrorString(e));
     if ((e = cudaGetLastError()) != cudaSuccess) return na_fail(GCP_ERR_CUDA, cudaGetErrorString(e));

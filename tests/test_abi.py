@@ -148,3 +148,46 @@ def test_binding_refuses_undersized_or_mistyped_buffers():
     for buf, dtype in bad:
         with pytest.raises(ValueError):
             gcp._check_buf(buf, 10 if dtype == "float32" else 1, dtype, "buf")
+
+
+def test_hot_row_words_of_other_calls_stay_inside_the_scratch(tmp_path):
+    """What a call without allocation finds in the shared scratch may come from
+    a call of another rank and order that overlapped with it.  For every word
+    such a call can leave, and any other 16 bits, the word as this call uses it
+    addresses only its mode's share of the replicas; its own words it uses as
+    they are; rows outside a mode are refused.  The header is compiled for the
+    host."""
+    src = tmp_path / "hot.cpp"
+    src.write_text('#include "gcp_noalloc_hot.h"\nusing namespace gcpna;\n'
+                   'extern "C" int share(int d) { return mode_floats(d); }\n'
+                   'extern "C" int word(int n, int R, int d) { return hot_word(n, R, d); }\n'
+                   'extern "C" int in_mode(int r, long long I) { return row_in_mode(r, I); }\n'
+                   'extern "C" int floats(int w, int R, int d) {\n'
+                   '    w = hot_word_for(w, R, d);\n'
+                   '    const int n = hot_count(w), r = hot_replicas(w);\n'
+                   '    if (n > kHot || (r & (r - 1))) return 1 << 30;\n'
+                   '    return n * r * row_floats(R);\n'
+                   '}\n'
+                   'extern "C" int largest(const int *w, int m, int R, int d) {\n'
+                   '    int most = 0;\n'
+                   '    for (int i = 0; i < m; ++i) { const int f = floats(w[i], R, d); if (f > most) most = f; }\n'
+                   '    return most;\n'
+                   '}\n')
+    lib = str(tmp_path / "hot.so")
+    csrc = os.path.join(ROOT, "paper_2605_20353_gb300", "csrc")
+    subprocess.check_call(["g++", "-std=c++17", "-O2", "-shared", "-fPIC", f"-I{csrc}", str(src), "-o", lib])
+    import ctypes
+
+    c = ctypes.CDLL(lib)
+    c.in_mode.argtypes = [ctypes.c_int, ctypes.c_longlong]
+    shapes = [(R, d) for R in range(1, 129) for d in range(2, 9)]
+    words = {c.word(n, R, d) for R, d in shapes for n in range(0, 40)}
+    assert max(w >> 8 for w in words) == 32 and max(w & 255 for w in words) == 32
+    words = np.array(sorted(words | set(range(1 << 16)) | {-1, 2**31 - 1, -2**31, (1 << 20) | 32}), dtype=np.int32)
+    for R, d in shapes:
+        assert c.largest(words.ctypes.data_as(ctypes.c_void_p), len(words), R, d) <= c.share(d), (R, d)
+        for n in range(0, 40):
+            own = c.word(n, R, d)
+            if own:  # used as it is: n rows of at least four replicas
+                assert c.floats(own, R, d) >= 4 * n * R
+    assert [c.in_mode(r, 7) for r in (-2**31, -1, 0, 6, 7, 2**31 - 1)] == [0, 0, 1, 1, 0, 0]

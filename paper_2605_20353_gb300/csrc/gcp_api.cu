@@ -360,6 +360,24 @@ gcpk::FusedSpec gcpk_make_spec(const gcp_ctx *c, uint64_t iter, int64_t p, int64
 
 gcp_status gcpk_check_counts(gcp_ctx *c, int64_t p, int64_t q) { return check_counts(c, p, q); }
 
+bool gcpk_begin_gradient(gcp_ctx *c) {
+    cudaStreamCaptureStatus status = cudaStreamCaptureStatusNone;
+    unsigned long long id = 0;
+    bool known = true;
+    if (cudaStreamGetCaptureInfo(c->st, &status, &id) != cudaSuccess) {
+        cudaGetLastError();  // the legacy stream while another thread captures: not this call's error
+        known = false;
+    } else if (status == cudaStreamCaptureStatusNone) {
+        id = 0;
+    } else {
+        c->g_captured = true;
+    }
+    const bool clear = known && c->g_clear && c->g_capture == id && (id != 0 || !c->g_captured);
+    c->g_clear = false;
+    c->g_capture = id;
+    return clear;
+}
+
 namespace {
 
 // Whether kernels of the context can write n bytes at p directly: device
@@ -428,9 +446,9 @@ gcp_status run_fused(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, bool grad,
     if (s) return s;
     double w_nz, w_z;
     gcpk::FusedSpec f = gcpk_make_spec(c, iter, p, q, grad, dscale, &w_nz, &w_z);
-    if (grad) {  // also when G is clear: a captured call is replayed on a G that is not
+    if (grad) {
+        gcpk_begin_gradient(c);  // cleared whatever it returns: the pass starts beside this kernel
         GCP_CUDA(c, gcpk::launch_clear(c->G, c->total_rows * c->Rp, c->st));
-        c->g_clear = false;
     }
     int blocks = 0;
     cudaEvent_t stop = nullptr;
@@ -528,7 +546,7 @@ gcp_status do_step(gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, const gcp_ad
     if ((s = check_counts(c, p, q))) return s;
     double w_nz, w_z;
     gcpk::FusedSpec f = gcpk_make_spec(c, iter, p, q, true, nullptr, &w_nz, &w_z);
-    if (!c->g_clear) GCP_CUDA(c, cudaMemsetAsync(c->G, 0, (size_t)c->total_rows * c->Rp * 4, c->st));
+    if (!gcpk_begin_gradient(c)) GCP_CUDA(c, cudaMemsetAsync(c->G, 0, (size_t)c->total_rows * c->Rp * 4, c->st));
     int blocks = 0;
     cudaEvent_t stop = nullptr;
     if ((s = prof_begin(c, &stop))) return s;

@@ -701,6 +701,8 @@ gcp_status gcp_batch_local_steps(gcp_batch *b, int32_t tau, const gcp_adam_param
         b->graph_blocks = b->blocks;
         b->graph_ts = b->ts;
     }
+    // G will hold the last local step's gradient (this call cannot be captured)
+    for (gcp_ctx *c : b->clients) gcpk_begin_gradient(c);
     BCUDA(b, cudaEventRecord(b->ev_in, b->user_st));  // after the clients' earlier work
     BCUDA(b, cudaStreamWaitEvent(b->st, b->ev_in, 0));
     gcpb::k_batch_set<<<(2 * tau + gcpb::kThreads - 1) / gcpb::kThreads, gcpb::kThreads, 0, b->st>>>(
@@ -708,7 +710,6 @@ gcp_status gcp_batch_local_steps(gcp_batch *b, int32_t tau, const gcp_adam_param
         prm->lower);
     BCUDA(b, cudaGetLastError());
     BCUDA(b, cudaGraphLaunch(b->graph, b->st));
-    for (gcp_ctx *c : b->clients) c->g_clear = false;  // G holds the last local step's gradient
     BCUDA(b, cudaEventRecord(b->ev_out, b->st));  // the clients' later work waits for the steps
     BCUDA(b, cudaStreamWaitEvent(b->user_st, b->ev_out, 0));
     if (prev >= 0 && prev != b->device) cudaSetDevice(prev);

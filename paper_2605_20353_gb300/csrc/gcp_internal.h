@@ -202,7 +202,13 @@ struct gcp_ctx {
     double *h_loss = nullptr;     // pinned mirror of dloss
 
     // hot-row replicas of the gradient
-    bool g_clear = true;          // G is all zero (gcp_step leaves it so)
+    // Whether G is all zero before the next call's work (gcp_step leaves it
+    // so): only where that work runs right after the work that cleared it,
+    // live after live or in one stream capture.  A captured call does not run
+    // now, and its graph may be replayed between any two live calls.
+    bool g_clear = true;                  // the last call on G, live or captured, clears it
+    unsigned long long g_capture = 0;     // the capture that call went into, 0 if it ran
+    bool g_captured = false;              // some call on G was ever captured
     int *hot_slot = nullptr;      // [total_rows] row -> replica slot or -1
     int *hot_row = nullptr;       // [Htot] slot -> row
     int small_base[GCP_MAX_NDIM] = {0};
@@ -261,3 +267,8 @@ void gcpk_set_noctx_error(const char *msg);
 gcpk::FusedSpec gcpk_make_spec(const gcp_ctx *c, uint64_t iter, int64_t p, int64_t q, bool grad,
                                const float *dscale, double *w_nz_out, double *w_z_out);
 gcp_status gcpk_check_counts(gcp_ctx *c, int64_t p, int64_t q);
+
+// A call is about to write c->G on c->st.  Returns whether G is known to be
+// zero when that work runs; from here on G counts as not zero, in the capture
+// that c->st is in, if any (gcp_ctx::g_clear).
+bool gcpk_begin_gradient(gcp_ctx *c);

@@ -1073,6 +1073,85 @@ def test_back_to_back_calls_wait_for_one_another(env, p, q, dtype):
             assert rel_err(a, b) <= 1e-5, (how, rel_err(a, b))
 
 
+@pytest.mark.parametrize("order", ["step captured after a step, replayed after a gradient",
+                                   "live step after a captured gradient's replay",
+                                   "live step after a captured step that never ran",
+                                   "two steps of one capture"])
+def test_steps_start_from_a_clear_gradient_around_captures(env, order):
+    """A step clears the gradient for the next one, which then need not; a
+    captured call does not run when it is made, and its replay may follow any
+    other call.  In each order the factors are those of the same steps made
+    live with nothing between them: an uncleared gradient of the large factors
+    here moves them by far more than 1e-5."""
+    gcp, torch = env
+    dims, R, p, q = [61, 47, 900], 10, 3000, 2800
+    coords, vals, factors = problem(dims, 6000, R, "poisson", 921)
+    prm = gcp.AdamParams(lr=1e-2, beta1=0.9, beta2=0.99, eps=1e-8, lower=0.05)
+    stream = torch.cuda.Stream()
+    ctxs = []
+    with torch.cuda.stream(stream):
+        for _ in range(2):
+            ctxs.append(gcp.gcp_create(dims, coords, vals, R, "poisson", seed=922))
+            ctxs[-1].set_factors(factors)
+    ref, ctx = ctxs
+    G = torch.zeros(ctx.num_params, device="cuda")
+    dl = torch.zeros(1, dtype=torch.float64, device="cuda")
+    torch.cuda.synchronize()
+
+    def capture(*calls):
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream, capture_error_mode="thread_local"):
+            for call in calls:
+                call()
+        return graph
+
+    def step(c, t):
+        c.step(t, p, q, prm, t + 1, dloss=dl)
+
+    def grad():
+        ctx.grad_async(99, p, q, G_out=G)
+
+    def replay(graph):
+        with torch.cuda.stream(stream):
+            graph.replay()
+
+    for t in range(4):
+        step(ref, t)
+    step(ctx, 0)
+    if order.startswith("step captured"):
+        g = capture(lambda: step(ctx, 1))
+        grad()
+        replay(g)
+        step(ctx, 2)
+        step(ctx, 3)
+    elif "replay" in order:
+        grad()
+        g = capture(grad)
+        step(ctx, 1)
+        replay(g)
+        step(ctx, 2)
+        replay(g)
+        step(ctx, 3)
+    elif "never ran" in order:
+        grad()
+        g = capture(lambda: step(ctx, 1))
+        step(ctx, 1)
+        grad()
+        step(ctx, 2)
+        step(ctx, 3)
+    else:
+        g = capture(lambda: step(ctx, 1), lambda: step(ctx, 2))
+        grad()
+        replay(g)
+        grad()
+        step(ctx, 3)
+    torch.cuda.synchronize()
+    a, b = (np.concatenate([f.ravel() for f in c.get_factors()]) for c in (ctx, ref))
+    assert rel_err(a, b) <= 1e-5, rel_err(a, b)
+    for c in ctxs:
+        c.close()
+
+
 @pytest.mark.parametrize("dims,R,dtype", [([100, 256, 40], 6, "fp32"), ([10000, 700, 200], 64, "fp32"),
                                           ([40000, 128, 129], 5, "bf16"), ([100000, 300, 9000], 16, "fp32"),
                                           ([1024, 1025], 33, "fp32"), ([5, 16384, 16385, 3], 20, "fp32")])

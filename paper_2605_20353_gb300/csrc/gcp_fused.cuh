@@ -102,11 +102,11 @@ __device__ __forceinline__ void load_record(const int32_t *__restrict__ rec, uin
 // round, and the gradient tensor's entries written by neighbouring lanes
 // (2^19 samples of the 4-way Zipf counts in BF16, a loss call: 48.1 -> 45.3
 // us; deterministic gradient of 2^21 samples at rank 64: 531 -> 501 us).
-// Then a butterfly sums the tile in
-// FP32 (nonzero and other samples apart), and the warp adds the sum to its
-// FP64 totals.  (FP64 adds are slow here, 16 cycles of the SM's pipe for a
-// warp: a lane's own FP64 totals, reduced over the warp at the end, cost 2 us
-// more per pass of 10,000 samples.)  A sample's m is summed per quad, then
+// Each lane adds its sample's f to its own FP64 totals (nonzero and other
+// samples apart), one FP64 addition per tile and warp.  They are slow here,
+// 16 cycles of the SM's pipe for a warp, so the lanes' totals meet at the end
+// in few instructions (block_totals): with five shuffle steps for each of the
+// two totals in every warp a pass of 10,000 samples took 2 us more.  A sample's m is summed per quad, then
 // over quads Rp / 2 columns apart, then Rp / 4, ..., whatever COLS is, and a
 // sample's lane and warp depend on the tile alone, so a loss pass and a
 // gradient pass over the same samples give the same loss bit for bit
@@ -117,11 +117,36 @@ __device__ __forceinline__ void load_record(const int32_t *__restrict__ rec, uin
 // row is added to G itself.
 constexpr int kWarps = kThreads / 32;
 
-// Sum over the warp's lanes, the same bits in every lane.
-__device__ __forceinline__ float warp_sum(float v) {
+// The block's sums of its threads' a and b and of the warps' counts n, in a
+// fixed order, to out[0..2] (n is the same in every lane of a warp).  Lanes 0
+// to 15 of a warp take its a, lanes 16 to 31 its b, one addition for both; then
+// one warp adds the warps' rows in pairs and the halves of the result: 19
+// additions of a warp a block, in chains of 8.  scratch: kWarps rows of 33
+// doubles, free for use by the whole block.
+__device__ __forceinline__ void block_totals(double a, double b, int n, double (*scratch)[33], double *out) {
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+    const bool low = lane < 16;
+    const double other = __shfl_xor_sync(0xFFFFFFFFu, low ? b : a, 16);
+    scratch[warp][lane] = (low ? a : b) + other;
+    if (lane == 0) scratch[warp][32] = __longlong_as_double((long long)n);
+    __syncthreads();
+    if (warp != 0) return;
+    double t[kWarps];
 #pragma unroll
-    for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xFFFFFFFFu, v, o);
-    return v;
+    for (int w = 0; w < kWarps; ++w) t[w] = scratch[w][lane];
+#pragma unroll
+    for (int h = kWarps / 2; h > 0; h >>= 1)
+#pragma unroll
+        for (int w = 0; w < h; ++w) t[w] += t[w + h];
+#pragma unroll
+    for (int o = 8; o > 0; o >>= 1) t[0] += __shfl_xor_sync(0xFFFFFFFFu, t[0], o);
+    if ((lane & 15) == 0) out[lane >> 4] = t[0];
+    if (lane == 1) {
+        long long c = 0;
+#pragma unroll
+        for (int w = 0; w < kWarps; ++w) c += __double_as_longlong(scratch[w][32]);
+        out[2] = (double)c;
+    }
 }
 
 // EVAL: no reductions (P.G null); P.Yval, if set, receives the gradient tensor.
@@ -367,32 +392,18 @@ __global__ void __launch_bounds__(kThreads, fused_min_blocks(D, EVAL ? 4 : COLS)
                 P.Yval[sm * P.vstride] = ok ? ((is_nz || uniform) ? P.w_nz : P.w_z) * df * scale : 0.0f;
             }
         }
-        if (uniform || s0 + TS <= (unsigned)p) {
-            acc_nz += (double)warp_sum(fl);
-        } else if (s0 >= (unsigned)p) {
-            acc_z += (double)warp_sum(fl);
-        } else {  // the one tile that holds both kinds
-            acc_nz += (double)warp_sum(s0 + lane < (unsigned)p ? fl : 0.0f);
-            acc_z += (double)warp_sum(s0 + lane < (unsigned)p ? 0.0f : fl);
-        }
+        if (uniform || s0 + lane < (unsigned)p)  // apart in one tile at most
+            acc_nz += (double)fl;
+        else
+            acc_z += (double)fl;
     }
     cp_async_wait<0>();
 
-    // block reduction of the warps' FP64 loss sums and the attempt counts
+    // the block's FP64 loss sums and attempt count
     attempts = __reduce_add_sync(0xFFFFFFFFu, attempts);
-    double(*red)[kWarps] = reinterpret_cast<double(*)[kWarps]>(&s_bkt[0][0][0][0]);  // staging is free now
-    __syncthreads();
-    if (lane == 0) {
-        red[0][warp] = acc_nz;
-        red[1][warp] = acc_z;
-        red[2][warp] = (double)attempts;
-    }
-    __syncthreads();
-    if (threadIdx.x < 3) {
-        double t = 0.0;
-        for (int w = 0; w < kWarps; ++w) t += red[threadIdx.x][w];
-        P.partials[4 * blockIdx.x + threadIdx.x] = t;
-    }
+    __syncthreads();  // staging is free now
+    block_totals(acc_nz, acc_z, attempts, reinterpret_cast<double(*)[33]>(&s_bkt[0][0][0][0]),
+                 P.partials + 4 * blockIdx.x);
 }
 
 // Resident blocks, and the launch, of the (dtype, columns) instantiation.

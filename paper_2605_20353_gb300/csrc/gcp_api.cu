@@ -285,24 +285,35 @@ gcp_status check_counts(gcp_ctx *c, int64_t p, int64_t q) {
 // registers (dense 5-way gradient 326 against 334 us), they are kept always.
 bool skewed(const gcp_ctx *c) { return c->d <= 4 && c->share_nz > 2.0 * c->share_cell; }
 
-// Replicas of the hot rows for a sample set.  The reductions that meet in one
-// 128-byte line are applied one after another, about 4.7 ns each (with no
-// replicas the benchmark's step takes 0.90 ms and the dense 5-way gradient
-// 1.92 ms, which is their hottest line's expected count x 4.6-5.5 ns), so the
-// hottest line bounds the pass from below by that count x 4.7 ns / nrep.  A
-// line holds 32 / Rp rows of a padded rank below 32.  Every replica costs the
-// fold 8 B per entry of every hot row: on 16 clients of 500 hot rows and
-// 16,384 samples each, 64 replicas cost 23 us of a 58-us local step.  So
-// replicas are taken until the chain is under 6% of the pass's row traffic
-// (2 x 4 B x D Rp per sample at about 9 TB/s) or under 4 us, less than the
-// latency of the shortest pass, rounded up to a count the folds are built
-// for; and until no row sums more than about 256 terms one after another in
-// FP32 (25,777 samples on six modes of 33 to 91 rows, 781 terms a row: 6.7e-7
-// from the FP64 gradient without replicas, 1.2e-7 with 64).  Measured per call with 0 / 4 / 16 / 64 replicas: benchmark step 900 /
-// 487 / 278 / 247 us (rule: 64); dense 5-way gradient, 2^22 samples 1916 /
-// 852 / 421 / 367 us (64); 172 x 25,000 x 300, rank 50, 2^16 samples 48.5 /
-// 52.3 / 52.3 / 54.3 us (0); 211 x 187 x 95 x 24, rank 10, 10^4 samples 18.7 /
-// 18.6 / 18.6 / 18.6 us per fit iteration (4).
+// Replicas of the hot rows for a sample set.  Two things ask for them:
+//  - time: the reductions that meet in one 128-byte line are applied one after
+//    another, about 4.7 ns each (with no replicas a step of 2^21 samples of
+//    the 4-way Zipf tensor takes 0.78 ms and the dense 5-way gradient of 2^22
+//    samples 1.96 ms: their hottest line's expected count x 4.2-4.7 ns), so the
+//    hottest line bounds the pass from below by that count x 4.7 ns / nrep.  A
+//    line holds 32 / Rp rows of a padded rank below 32.  This chain is to be
+//    under 6% of the pass's row traffic (2 x 4 B x D Rp per sample at about 9
+//    TB/s) or under 4 us, less than the latency of the shortest pass;
+//  - precision: the terms of a row are added in FP32 one after another within
+//    a replica, so the hottest row's expected terms are to be at most 32 in
+//    each.  With 64 replicas whatever the count, rows of up to about 2,000
+//    terms had that too, and shorter chains gain nothing against the FP64
+//    gradient, relative 2-norm: 2,000 samples on modes of 30 to 50 rows (66
+//    terms a row) 8.3e-8 with no replicas, 4.9e-8, 4.5e-8 and 4.5e-8 with 4, 16
+//    and 64; 2^16 samples on modes of 172 to 25,000 rows (381 terms) 2.7e-7,
+//    8.2e-8, 4.8e-8 and 4.5e-8.
+// Against them, every replica costs the fold 8 B per entry of every hot row.
+// The count is rounded up to one the folds are built for, and 64 is the most:
+// rows with more than 2,048 terms have longer chains (the two shapes below
+// with 64 about 5,000 and 3,300 terms a replica at most), and so have rows
+// without replicas, in modes of more than 512 rows.
+// Measured with 0 / 4 / 16 / 64 replicas: step of the 4-way Zipf tensor, rank
+// 32, 2^21 samples 784 / 461 / 276 / 222 us (rule: 64); dense 5-way gradient,
+// rank 16, 2^22 samples 1956 / 724 / 402 / 325 us (64); 172 x 25,000 x 300,
+// rank 50, 2^16 samples 21.6 / 20.3 / 20.9 / 27.1 us (16); 211 x 187 x 95 x 24
+// Zipf, rank 10, 10^4 samples 11.9 / 8.8 / 8.8 / 9.0 us per fit iteration (64);
+// 8 local steps of 16 clients, 500 hot rows and 16,384 samples each, 265 / 268
+// / 296 / 457 us (4).
 int replicas_for(const gcp_ctx *c, int64_t p, int64_t q) {
     if (!c->Grep) return 0;
     const double line = c->Rp >= 32 ? 1.0 : 32.0 / c->Rp;  // rows of a 128-byte line
@@ -312,7 +323,7 @@ int replicas_for(const gcp_ctx *c, int64_t p, int64_t q) {
     const double terms = uniform ? (double)p * c->share_cell
                                  : (double)p * c->share_nz + (double)q * c->share_cell;
     const double pass = (double)(p + q) * 8.0 * c->d * c->Rp / 9000.0;  // ns
-    const double want = std::max(hits * 4.7 / std::max(0.06 * pass, 4000.0), terms / 256.0);
+    const double want = std::max(hits * 4.7 / std::max(0.06 * pass, 4000.0), terms / 32.0);
     return want <= 1.0 ? 0 : (want <= 4.0 ? 4 : (want <= 16.0 ? 16 : gcpk::kReplicas));
 }
 

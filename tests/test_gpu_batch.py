@@ -134,7 +134,7 @@ def test_batch_clients_with_different_replica_counts(env):
     against the oracle."""
     gcp, torch = env
     dims, R = [8, 41, 700], 6
-    counts = [(150, 130), (60000, 50000), (900, 700), (7000, 6001)]
+    counts = [(150, 130), (60000, 50000), (900, 700), (7000, 6001), (100, 90)]
     shards = []
     for i, (p, q) in enumerate(counts):
         coords, vals = synth.uniform_sparse(dims, 5000, 640 + i, lam=2.0)

@@ -776,7 +776,7 @@ def test_replica_counts_in_turn_on_one_context(env, mttkrp):
     dims, R = [8, 41, 700], 6  # one replicated small mode, one of 41 rows, one too large
     coords, vals, factors = problem(dims, 5000, R, "poisson", 611)
     ctx = gcp.gcp_create(dims, coords, vals, R, "poisson", seed=612, mttkrp=mttkrp)
-    for t, (p, q) in enumerate([(60000, 50000), (150, 130), (900, 700), (7000, 6001), (900, 700), (60000, 1),
+    for t, (p, q) in enumerate([(60000, 50000), (150, 130), (100, 90), (900, 700), (7000, 6001), (100, 90), (900, 700), (60000, 1),
                                 (0, 9000), (300, 0)]):
         idx, x, w, _ = oracle.stratified_samples(612, t, p, q, dims, coords, vals)
         Lo, Go = oracle.sampled_loss_grad(dims, factors, "poisson", idx, x, w)
@@ -802,6 +802,28 @@ def one_heavy_row(dims, nnz, heavy, seed):
     cells = np.concatenate([cells, rest[rest % dims[2] != 5][:nnz - heavy]])
     coords = np.stack(np.unravel_index(cells, dims), axis=1)
     return coords.astype(synth.uniform_sparse(dims, 8, 1)[0].dtype), rng.integers(1, 6, nnz).astype(np.float32)
+
+
+@pytest.mark.parametrize("n", [200, 230, 800, 1900])
+def test_hot_rows_are_not_summed_in_one_long_chain(env, n):
+    """About n terms of one sign meet in each row of a mode of 30 rows.  Added
+    one after another in FP32, step i of k rounds within 2^-24 of i / k of the
+    sum: 2^-24 sqrt(k) / 3 of it in rms, 2.8e-7 at 200 terms, in the measured
+    case 2e-7.  In chains of at most 32 it is 1.1e-7 of a chain and, as the
+    chains round independently, at most 4e-8 of the sum of seven or more; the
+    fold adds about as much.  1e-7 divides the two."""
+    gcp, torch = env
+    dims, R, p = [30, 45, 60], 16, 30 * n
+    coords, vals, factors = problem(dims, 40000, R, "gaussian", 951)
+    vals = np.full_like(vals, 1000.0)  # far above the model: every derivative has its sign
+    factors = [np.abs(f) + np.float32(0.1) for f in factors]
+    ctx = gcp.gcp_create(dims, coords, vals, R, "gaussian", seed=952)
+    ctx.set_factors(factors)
+    _, G = gpu_grad(gcp, torch, ctx, 1, p, 0)
+    idx, x, w, _ = oracle.stratified_samples(952, 1, p, 0, dims, coords, vals)
+    _, Go = oracle.sampled_loss_grad(dims, factors, "gaussian", idx, x, w)
+    assert rel_err(split(G, dims, R)[0], Go[0]) <= 1e-7, rel_err(split(G, dims, R)[0], Go[0])
+    ctx.close()
 
 
 @pytest.mark.parametrize("R", [3, 6, 32, 40])

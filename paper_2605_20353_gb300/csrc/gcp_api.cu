@@ -274,16 +274,20 @@ gcp_status check_counts(gcp_ctx *c, int64_t p, int64_t q) {
     return GCP_OK;
 }
 
-// Whether single rows take far more of the nonzeros than a uniform tensor's.
-// Then the reductions gather in few lines, and where those lie counts: with
-// the replicas of a row in consecutive 128-byte lines of their own they spread
-// evenly over the L2 slices, while replicas a whole plane of hot rows apart
-// fell on them as the number of hot rows had it (2^21 samples at rank 32 on
-// 4-way Zipf tensors 216 to 249 us; now 216 to 236).  Without skew the planes,
-// compact per warp, are the better layout (100 x 90 x 80 x 70 at rank 32 215
-// against 217 us), and above order 4, where a row's stride other than Rp costs
-// registers (dense 5-way gradient 326 against 334 us), they are kept always.
-bool skewed(const gcp_ctx *c) { return c->d <= 4 && c->share_nz > 2.0 * c->share_cell; }
+// Whether a hot row's replicas lie one after another, instead of in planes of
+// all hot rows.  Where single rows take far more of the nonzeros than a uniform
+// tensor's, the reductions gather in few lines, and it counts how those fall on
+// the L2 slices.  Rows of two lines and more (padded rank 64 and 128) do better
+// one after another: training steps of 2^20 and 2^19 samples on eight Zipf
+// tensors of 3 and 4 modes 0 to 5% faster than in planes, none slower by more
+// than 0.5% (2000 x 1500 x 1000 x 200 at rank 64 207 -> 193 us).  Shorter rows
+// do not: at ranks 4 to 32, each replica in a line of its own, from 9% faster
+// (4000 x 3000 x 2000 x 500 at rank 32 244 -> 222 us) to 12% slower (1000^4 216
+// -> 238 us at rank 32, 103 -> 115 at rank 4), on average slower.  Without skew
+// planes, compact per warp, are the better layout, and above order 4, where a
+// row's stride other than Rp costs registers (dense 5-way gradient 326 against
+// 334 us), they are kept always.
+bool replica_lines(const gcp_ctx *c) { return c->d <= 4 && c->Rp >= 64 && c->share_nz > 2.0 * c->share_cell; }
 
 // Replicas of the hot rows for a sample set.  Two things ask for them:
 //  - time: the reductions that meet in one 128-byte line are applied one after
@@ -362,8 +366,8 @@ gcpk::FusedSpec gcpk_make_spec(const gcp_ctx *c, uint64_t iter, int64_t p, int64
     for (int k = 0; k < c->d; ++k) f.small_base[k] = f.nrep ? c->small_base[k] : -1;
     f.Grep = f.nrep ? c->Grep : nullptr;
     f.Htot = f.nrep ? c->Htot : 0;
-    f.rplane = skewed(c) ? std::max(c->Rp, 32) : c->Htot * c->Rp;
-    f.rstride = skewed(c) ? f.nrep * f.rplane : c->Rp;
+    f.rplane = replica_lines(c) ? c->Rp : c->Htot * c->Rp;
+    f.rstride = replica_lines(c) ? f.nrep * c->Rp : c->Rp;
     if (w_nz_out) *w_nz_out = w_nz;
     if (w_z_out) *w_z_out = w_z;
     return f;
@@ -844,7 +848,7 @@ gcp_status setup_hot_rows(gcp_ctx *c, const std::vector<int64_t> &counts) {
     c->share_nz = counts.empty() ? 0.0 : (double)most / (double)c->nnz;
     c->Htot = (int)row.size();
     if (c->Htot == 0) return GCP_OK;
-    const size_t rep_bytes = (size_t)gcpk::kReplicas * c->Htot * (skewed(c) ? std::max(c->Rp, 32) : c->Rp) * 4;
+    const size_t rep_bytes = (size_t)gcpk::kReplicas * c->Htot * c->Rp * 4;
     cudaError_t e;
     if ((e = cudaMalloc(&c->hot_slot, slot.size() * 4)) || (e = cudaMalloc(&c->hot_row, row.size() * 4)) ||
         (e = cudaMalloc(&c->Grep, rep_bytes)) ||

@@ -63,7 +63,7 @@ struct FusedSpec {
 // call uses as many as its sample count and the hottest row's share call for
 // (replicas_for): none, 4, 16 or all 64.  Replica r of hot row `slot` starts at
 // slot * rstride + r * rplane floats: planes of Htot rows, or each row's
-// replicas in consecutive lines (skewed in gcp_api.cu).
+// replicas one after another (replica_lines in gcp_api.cu).
 constexpr int kReplicas = 64;
 
 // Where a call's sampled loss goes once the block partials are summed: the

@@ -826,11 +826,11 @@ def test_hot_rows_are_not_summed_in_one_long_chain(env, n):
     ctx.close()
 
 
-@pytest.mark.parametrize("R", [3, 6, 32, 40])
+@pytest.mark.parametrize("R", [3, 6, 32, 40, 100])
 @pytest.mark.parametrize("mttkrp", ["atomic", "nonfused"])
 def test_replica_lines_of_skewed_tensors(env, mttkrp, R):
-    """Replicas in lines of their own (a row with a sixth of the nonzeros;
-    ranks below, at and above the 32 floats of a line): sample counts that
+    """A row with a sixth of the nonzeros: its replicas lie one after another at
+    padded ranks of 64 and 128, in planes below.  Sample counts that
     take none, 4, 16 and 64 of them mixed on one context, so every call must
     find cleared what calls with another replica stride used."""
     gcp, torch = env
@@ -838,7 +838,7 @@ def test_replica_lines_of_skewed_tensors(env, mttkrp, R):
     coords, vals = one_heavy_row(dims, 6000, 1000, 621)
     factors = synth.factors_uniform(dims, R, 622, lo=0.1, hi=1.0)
     ctx = gcp.gcp_create(dims, coords, vals, R, "poisson", seed=623, mttkrp=mttkrp)
-    for t, (p, q) in enumerate([(60000, 50000), (150, 130), (3000, 700), (7000, 6001), (3000, 700), (60000, 1)]):
+    for t, (p, q) in enumerate([(60000, 50000), (150, 130), (500, 200), (3000, 700), (1500, 700), (7000, 6001), (3000, 700), (60000, 1)]):
         idx, x, w, _ = oracle.stratified_samples(623, t, p, q, dims, coords, vals)
         Lo, Go = oracle.sampled_loss_grad(dims, factors, "poisson", idx, x, w)
         ctx.set_factors(factors)

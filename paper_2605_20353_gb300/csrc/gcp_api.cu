@@ -187,14 +187,18 @@ gcp_status init_common(gcp_ctx *c, int32_t ndim, const int64_t *dims, int32_t ra
     // wherever there are eight columns, and still fits four blocks (2^19
     // samples of the 4-way Zipf tensor, rank 32 BF16: kernel 42.8 -> 35.8 us).
     // A gradient pass takes eight from rank 33 on (2^20 samples of 2 to 8
-    // modes at ranks 33 to 65: 12 to 27% faster), and at a padded rank of 32
-    // where few of the second half's columns are in use (rank 20, 2 to 5
-    // modes: 4 to 18% faster; rank 24 the same, rank 32 slower by 12%) or
-    // there are two modes (12%).
+    // modes at ranks 33 to 65: 12 to 27% faster).  At a padded rank of 32 it
+    // takes eight for two modes (ranks 17 to 28, 2^16 and 2^20 samples: 4 to 22%
+    // faster, rank 32 12%), and for three and four where one lane's second quad
+    // is in use at most: ranks 17 to 20 are five quads of columns (1 to 13%
+    // faster, all four ranks alike), ranks 21 to 24 six (2^20 samples 6 to 8%
+    // slower, 2^16 between 4% slower and 3% faster), 26 and 28 slower by up to
+    // 19%.  With five modes and six it costs registers (ranks 17 to 20: five
+    // modes 1 to 16% slower, six between 13% slower and 9% faster).
     int Rp = 4;
     while (Rp < rank) Rp <<= 1;
     c->Rp = Rp;
-    c->cols = Rp >= 64 || (Rp == 32 && (ndim == 2 || (rank <= 20 && ndim <= 5))) ? 8 : 4;
+    c->cols = Rp >= 64 || (Rp == 32 && (ndim == 2 || (rank <= 20 && ndim <= 4))) ? 8 : 4;
     c->eval_cols = Rp >= 8 ? 8 : 4;
     if (c->opt.lane_cols == 4 || (c->opt.lane_cols == 8 && Rp >= 8)) c->cols = c->eval_cols = c->opt.lane_cols;
     else if (c->opt.lane_cols != 0) return fail(nullptr, GCP_ERR_ARG, "lane_cols must be 0, 4 or 8");

@@ -366,7 +366,8 @@ struct gcp_batch {
     int tile_n = 0, total_tiles = 0; // samples per tile and tiles of the captured graph
     int4 *specs = nullptr;           // n x kSpecWords
     int *tile_start = nullptr;       // n + 1: first tile of each client
-    std::vector<gcpb::ClientAux> h_aux;
+    std::vector<gcpb::ClientAux> h_aux;  // sized at creation, as h_tile_start: batch_tiles allocates no host memory
+    std::vector<int> h_tile_start;
     int2 *chunks = nullptr;          // epilogue work list: {client, -1} loss, {client, first quad} Adam
     int nchunks = 0;
     gcpb::ClientAux *aux = nullptr;  // n
@@ -475,7 +476,7 @@ gcp_status batch_tiles(gcp_batch *b) {
         if ((n + warps - 1) / warps > rounds || n >= (int64_t)1 << 30) break;
         t -= ngrp;
     }
-    std::vector<int> tstart(b->n + 1, 0);
+    std::vector<int> &tstart = b->h_tile_start;
     for (int i = 0; i < b->n; ++i) {
         const int nt = (int)((b->p[i] + b->q[i] + t - 1) / t);
         tstart[i + 1] = tstart[i] + nt;
@@ -558,6 +559,7 @@ gcp_status gcp_batch_create(int32_t nclients, gcp_ctx *const *clients, const int
     std::vector<int4> specs((size_t)nclients * gcpb::kSpecWords);
     std::vector<gcpb::ClientAux> &aux = b->h_aux;
     aux.resize(nclients);
+    b->h_tile_start.assign((size_t)nclients + 1, 0);
     int64_t params = 0;
     for (int i = 0; i < nclients; ++i) {
         gcp_ctx *c = clients[i];

@@ -153,7 +153,12 @@ void gcp_options_default(gcp_options *opt);
  * coords (host, nnz x ndim int32, row-major) and vals (host, nnz float) are
  * the nonzeros, which must be distinct and in range.  rank in 1..128.  The
  * context copies the nonzeros into packed device records and a device hash
- * set of their linear indices.  Factors start at zero; set them with
+ * set of their linear indices.  It also holds four FP32 arrays of all rows at
+ * the padded rank (a power of two, at least 4), 64 replicas of the gradient
+ * rows that many samples hit (in a mode of at most 512 rows all of them, in a
+ * larger one at most 256, those with 1/512 of the nonzeros or more), and, where
+ * the rank needs padding, staging rows for copies from and to host arrays (as
+ * many as the model has, 8 MB at most).  Factors start at zero; set them with
  * gcp_set_factors.  Errors: GCP_ERR_ARG (bad sizes, coordinate out of range,
  * non-finite value, unknown loss), GCP_ERR_DOMAIN (negative value for the
  * Poisson/Gamma losses, value not 0/1 for Bernoulli), GCP_ERR_DUPLICATE,

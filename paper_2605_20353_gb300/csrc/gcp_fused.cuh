@@ -101,12 +101,17 @@ __device__ __forceinline__ void load_record(const int32_t *__restrict__ rec, uin
 // evaluates its own sample: one evaluation per tile instead of one per group
 // round, and the gradient tensor's entries written by neighbouring lanes
 // (2^19 samples of the 4-way Zipf counts in BF16, a loss call: 48.1 -> 45.3
-// us; deterministic gradient of 2^21 samples at rank 64: 531 -> 501 us).
+// us; deterministic gradient of 2^21 samples at rank 64: 531 -> 501 us, 494
+// with the losses added as follows).
 // Each lane adds its sample's f to its own FP64 totals (nonzero and other
 // samples apart), one FP64 addition per tile and warp.  They are slow here,
 // 16 cycles of the SM's pipe for a warp, so the lanes' totals meet at the end
 // in few instructions (block_totals): with five shuffle steps for each of the
-// two totals in every warp a pass of 10,000 samples took 2 us more.  A sample's m is summed per quad, then
+// two totals in every warp a pass of 10,000 samples took 2 us more than with
+// FP32 sums of each tile, with block_totals 0.3 us more (8.6 -> 8.9 us per
+// iteration of a fit), and passes of 2^18 samples and more take less, as a tile
+// no longer has five shuffle steps (dense 5-way gradient of 2^22 samples 329 ->
+// 324 us).  A sample's m is summed per quad, then
 // over quads Rp / 2 columns apart, then Rp / 4, ..., whatever COLS is, and a
 // sample's lane and warp depend on the tile alone, so a loss pass and a
 // gradient pass over the same samples give the same loss bit for bit

@@ -153,12 +153,11 @@ __device__ __forceinline__ void na_add(float *p, const float *c) {
 // afterwards; a lane looks its sample's rows up in a small table in shared
 // memory.
 // Bound by the row traffic through L2 (d rows gathered, d rows reduced per
-// sample).  2^18 samples of the 2000 x 1500
-// x 1000 x 200 Zipf tensor at rank 32, drawn with gcp_sample and passed
-// here: 99 us a pass, this kernel 42; 156 us with every reduction added to G itself (the ones
-// that meet in one row are applied one after another, about 4.7 ns each);
-// 745 us with one warp per sample walking 256 samples one after another on
-// 128 blocks.
+// sample).  2^18 samples of the 2000 x 1500 x 1000 x 200 Zipf tensor at rank 32,
+// drawn with gcp_sample and passed here: 99 to 105 us a pass, this kernel 42;
+// 156 us with every reduction added to G itself (the ones that meet in one row
+// are applied one after another, about 4.7 ns each); 745 us with one warp per
+// sample walking 256 samples one after another on 128 blocks.
 template <int D, int V, int NQ>
 __global__ void __launch_bounds__(kNaThreads, (D <= 4 ? 3 : 2))
     k_na_grad(const NaShape sh, int loss, int64_t n, const int32_t *__restrict__ idx, const float *__restrict__ x,

@@ -89,8 +89,7 @@ __global__ void __launch_bounds__(kThreads) k_batch_set(uint64_t *step, double *
 // Block-wide, fixed-order sum of client a's per-tile loss partials, weighted
 // (FP64).  Each thread adds its tiles t, t + kThreads, ... in that order; eight
 // loads are issued before their adds so the chain does not wait on each one.
-__device__ __forceinline__ void finish_client_loss(const ClientAux &a, const float2 *__restrict__ tile_loss,
-                                                   double *out) {
+__device__ __forceinline__ void finish_client_loss(const ClientAux &a, const float2 *tile_loss, double *out) {
     __shared__ double sh[2][kThreads];
     double nz = 0.0, z = 0.0;
     const float2 *tl = tile_loss + a.tile0;
@@ -208,7 +207,7 @@ __device__ __forceinline__ void post_hot_chunk(const ClientAux &a, int64_t h0, c
 
 __global__ void __launch_bounds__(kThreads, kPostMinBlocks) k_batch_post(const ClientAux *__restrict__ aux,
                                                          const int2 *__restrict__ chunks,
-                                                         const float2 *__restrict__ tile_loss, double *client_loss,
+                                                         const float2 *tile_loss, double *client_loss,
                                                          const double *__restrict__ adam,
                                                          const double *__restrict__ corr, bool clear) {
     const int2 ch = chunks[blockIdx.x];
@@ -222,10 +221,14 @@ __global__ void __launch_bounds__(kThreads, kPostMinBlocks) k_batch_post(const C
         return;
     }
     const int log2Rp = __ffs(a.Rp) - 1;  // Rp is a power of two and a multiple of 4
-    float4 *__restrict__ G4 = reinterpret_cast<float4 *>(a.G);
-    const float4 *__restrict__ A4 = reinterpret_cast<const float4 *>(a.A);
-    const float4 *__restrict__ B4 = reinterpret_cast<const float4 *>(a.B);
-    const float4 *__restrict__ C4 = reinterpret_cast<const float4 *>(a.C);
+    // no __restrict__: what earlier grids of the chain write (the tile losses
+    // too) must not be read through the read-only path, as this grid may have
+    // started beside them; all loads of a thread are issued before its stores
+    // by the order of the code
+    float4 *G4 = reinterpret_cast<float4 *>(a.G);
+    const float4 *A4 = reinterpret_cast<const float4 *>(a.A);
+    const float4 *B4 = reinterpret_cast<const float4 *>(a.B);
+    const float4 *C4 = reinterpret_cast<const float4 *>(a.C);
     if (ch.y <= -2) {  // hot quads, one per group of nrep / 4 lanes
         const int64_t h0 = (int64_t)(-2 - ch.y);
         if (a.nrep == 64)
